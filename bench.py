@@ -29,9 +29,8 @@ if ROOT not in sys.path:
 
 METRIC = "hybrid-step MLUPS & % of HBM roofline, FP32 vs plain FP64 at stated error"
 BYTES_PER_SITE = {"fp32": 200, "fp64": 400}
-# fused-step schedules offered to the autotuner, in candidate order
-TILE_NAMES = ["32x8", "32x16", "64x8", "32x8-pipelined-8+8", "32x8-pipelined-6+10", "32x6-pipelined-9+7",
-              "32x6-pipelined-10+6"]
+# tile shapes offered to the autotuner, in candidate order: fields kernel + LB kernel
+TILE_NAMES = ["32x4+32x8", "32x4+32x4", "64x2+64x4", "16x8+16x16", "32x8+32x8", "16x8+16x8", "8x8+8x8"]
 
 
 def workload_params(L, n, prec, **kw):
@@ -50,8 +49,8 @@ def measured_peaks():
 
 # the sources that define the step kernels: an ncu figure is current only while these are
 # unchanged since the capture (the profile records their fingerprint)
-STEP_SOURCES = ["lbcad_fused.cuh", "lbcad_kernels.cuh", "lbcad_internal.h", "lbcad_f32.cu"]
-STEP_SOURCES_FP64 = ["lbcad_fused.cuh", "lbcad_kernels.cuh", "lbcad_internal.h", "lbcad_f64.cu"]
+STEP_SOURCES = ["lbcad_march.cuh", "lbcad_kernels.cuh", "lbcad_internal.h", "lbcad_f32.cu"]
+STEP_SOURCES_FP64 = ["lbcad_march.cuh", "lbcad_kernels.cuh", "lbcad_internal.h", "lbcad_f64.cu"]
 
 
 def kernel_source_sha(sources=None):
@@ -330,7 +329,7 @@ def batch_leg(torch, L, steps=100, warmup=3):
     out = {"mlups": sites / (ms * 1e-3) / 1e6, "ms_per_step": ms, "steps": K, "sites": sites,
            "tiles": {"chosen": TILE_NAMES[cfg], "ms_per_cfg": dict(zip(TILE_NAMES, tms))},
            "workload": "64 droplets, edges from {48,64,80,96}, R = edge/4, zeta in [0.001, 0.01], pitch in "
-                       "[12, 40], seed 7, FP32, one launch per step replayed from a CUDA graph, a6 sums fused",
+                       "[12, 40], seed 7, FP32, two launches per step (28 instances each) replayed from a CUDA graph, a6 sums fused",
            "clocks": clk.summary()}
     sim.close()
     return out
@@ -411,7 +410,7 @@ def main():
         dist.barrier()
     # every timed step is the whole hot path: stencils, fields, stress and force, the order-
     # parameter update, the LB collision and streaming, and the FP64 conserved and centroid
-    # sums of the new state (fused into the same kernel; the library default).  The region of
+    # sums of the new state (fused into the LB kernel; the library default).  The region of
     # exactly K steps is timed repeatedly (the same count on every rank) until about a second of
     # device time has passed, so that the clock sampler sees it; the step time is the median.
     ms_probe = time_steps(sim, torch, K)
@@ -438,7 +437,7 @@ def main():
     sim.set_observe(True)
     sim.step(1)
     without_sums = {"mlups": whole_job_mlups(N, world, ms_nosums), "ms_per_step": ms_nosums,
-                    "note": "same step kernel without the fused FP64 sums (lbcad_set_observe(0))"}
+                    "note": "same step kernels without the fused FP64 sums (lbcad_set_observe(0))"}
 
     # plain FP64 GPU path on the same workload
     fp64 = None
@@ -464,14 +463,14 @@ def main():
         s64.close()
 
     # Sec. 3's sync coupling and predictor-corrector on the same workload, on the fused split
-    # (the LB half in the fused kernel, then the order-parameter kernels) and on the staged path
+    # (fields and LB kernels, then the order-parameter kernels) and on the staged path
     staged = None
     if not args.no_staged:
         staged = {}
         for name, integ, coup, path, launches in (
-                ("euler_sync", L.EULER, L.SYNC, "fused LB half + order-parameter kernel", 2),
+                ("euler_sync", L.EULER, L.SYNC, "fields, LB, order-parameter kernel", 3),
                 ("euler_sync_staged", L.EULER, L.SYNC, "staged", 3),
-                ("heun_sync", L.HEUN, L.SYNC, "fused LB half + predictor, fields, corrector", 4),
+                ("heun_sync", L.HEUN, L.SYNC, "fields, LB, predictor, fields, corrector", 5),
                 ("heun_sync_staged", L.HEUN, L.SYNC, "staged", 5)):
             sv = L.Simulation([(n, n, n)], [workload_params(L, n, L.FP32, integrator=integ, coupling=coup)],
                               seed=1 + rank, device=local)
@@ -593,7 +592,7 @@ def main():
     traffic_site = committed_traffic() if current else None
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": (traffic_site * N) if traffic_site else None,
-                "kernel": "k_step_pipe (one launch = one whole hybrid step, a6 sums included)",
+                "kernel": "k_march_fields + k_march_lb (one whole hybrid step, a6 sums included)",
                 "algorithmic_bytes_per_site": 200,
                 "peak_kind": peak_kind,
                 # the design floor also moves u in and out (224 B per site)
@@ -642,7 +641,7 @@ def main():
                 "tiles": {"chosen": TILE_NAMES[tile_cfg], "ms_per_cfg": dict(zip(TILE_NAMES, tile_ms))},
                 "timing": {"regions": len(region_ms), "steps_per_region": K, "median_ms_per_step": ms,
                            "min_ms_per_step": min(region_ms), "max_ms_per_step": max(region_ms)},
-                "gpu_launches": K, "clocks": csum, "batch64": batch, "step_without_sums": without_sums, "fp64_gpu": fp64, "integrators_fp32": staged, "lb_variants_fp32": variants, "bulk_fp32": bulk, "droplet_256_fp32": large, "adjoint_fp32": adjoint,
+                "gpu_launches": 2 * K, "clocks": csum, "batch64": batch, "step_without_sums": without_sums, "fp64_gpu": fp64, "integrators_fp32": staged, "lb_variants_fp32": variants, "bulk_fp32": bulk, "droplet_256_fp32": large, "adjoint_fp32": adjoint,
                 "speedup_fp32_vs_fp64": (value / world / fp64["mlups"]) if fp64 else None,
                 "observables_finite": finite}
         print(json.dumps(line))

@@ -158,10 +158,11 @@ int lbcad_create_batch(int32_t n, const lbcad_grid* grids, const lbcad_params* p
  * call).  With graphs enabled (lbcad_set_graph), the steps replay a captured CUDA graph. */
 int lbcad_step(lbcad_ctx* c, int64_t n);
 
-/* Kernel path of lbcad_step.  LBCAD_PATH_FUSED (default): one persistent kernel per
- * step with shared-memory halo tiles.  LBCAD_PATH_TWO_KERNEL: a stencil kernel writing
+/* Kernel path of lbcad_step.  LBCAD_PATH_FUSED (default): two kernels per step that march up z through
+ * shared-memory tiles (fields, stress and the update of Q; then force, populations, psi and the sums),
+ * with 12 values per site of scratch allocated at create.  LBCAD_PATH_TWO_KERNEL: a stencil kernel writing
  * H, mu and sigma to a per-site scratch (allocated on the first switch, 15 values per
- * site) and an update kernel; same arithmetic, kept as a cross-check.  Changing the path
+ * site) and an update kernel, one thread per site; same arithmetic, kept as a cross-check.  Changing the path
  * drops a captured graph. */
 #define LBCAD_PATH_FUSED 0
 #define LBCAD_PATH_TWO_KERNEL 1
@@ -171,9 +172,9 @@ int lbcad_step(lbcad_ctx* c, int64_t n);
  * LBCAD_STENCIL_R2, selected at create (fused/two-kernel paths, tile shapes, autotune and the
  * adjoint return LBCAD_E_UNSUPPORTED there); other contexts may select it as a cross-check
  * (same per-site arithmetic).  Scratch: 15 values per site, 27 with LBCAD_HEUN.
- * LBCAD_SYNC or LBCAD_HEUN on the fused path (their default): the fused kernel on one fixed
- * tile shape does the LB half (u of this step; H and mu into the scratch), then tiled
- * z-marching order-parameter kernels on the same tiles (sync: the update; Heun: predictor,
+ * LBCAD_SYNC or LBCAD_HEUN on the fused path (their default): the fields kernel and the LB kernel
+ * (u of this step; H and mu into the scratch), then tiled
+ * z-marching order-parameter kernels (sync: the update; Heun: predictor,
  * fields at the predicted state, corrector); tile shapes, autotune, the two-kernel path and the adjoint return
  * LBCAD_E_UNSUPPORTED there.  LBCAD_D3Q15 and LBCAD_LB_STRESS_EQ run on the fused path (tile
  * shapes 0 and 3 only) and the staged path; the two-kernel path and the adjoint return
@@ -187,10 +188,10 @@ int lbcad_set_path(lbcad_ctx* c, int32_t path);
  * speed), in three rounds that interleave the candidates; a candidate's time is its best
  * round.  Writes the chosen index to *chosen and, if ms_per_cfg is given, the measured
  * milliseconds per launch of up to ncfg candidates (-1 for a shape that does not fit).
- * Candidates: 0 = 32x8 tiles (the FP64 default), 1 = 32x16, 2 = 64x8, 3 (the FP32 default) and 4 = 32x8 software-pipelined
- * (sigma of plane k+1 on 8 or 6 warps while the other 8 or 10 warps output plane k-1, in
- * one phase), 5 and 6 = 32x6 software-pipelined (9 or 10 sigma warps, one round per
- * plane); 1-6 are FP32 only.  With LBCAD_D3Q15 or LBCAD_LB_STRESS_EQ only 0 and 3 are
+ * Candidates (tile of the fields kernel + tile of the LB kernel): 0 = 32x4 + 32x8 (the FP64 default:
+ * 32x8 + 32x8), 1 = 32x4 + 32x4, 2 = 64x2 + 64x4, 3 = 16x8 + 16x16, 4 = 32x8 + 32x8, 5 = 16x8 + 16x8,
+ * 6 = 8x8 + 8x8; 1-6 are FP32 only.  The FP32 default is 0 or 3, whichever covers the boxes with fewer
+ * sites beyond their edges.  With LBCAD_D3Q15 or LBCAD_LB_STRESS_EQ only 0 and 3 are
  * candidates (-1 for the others). */
 int lbcad_autotune(lbcad_ctx* c, int32_t reps, int32_t* chosen, float* ms_per_cfg, int32_t ncfg);
 
@@ -254,8 +255,8 @@ int lbcad_set_state(lbcad_ctx* c, int32_t inst, const void* src, size_t bytes, i
  * step's own arithmetic).  Writes dJ/dzeta and dJ/dq0 (accumulated in FP64; q0 enters through H and
  * sigma, the initial Q held fixed), dJ/dQ(t0) for the five stored Q components
  * ([5][z][y][x], host FP64, may be NULL) and J itself.  Device memory: (ceil(nsteps /
- * ckpt_every) + ckpt_every + 2) states of 28 values per site, plus 15 values per site for
- * each of the ckpt_every states of a segment (their sigma, mu and H, computed once in the
+ * ckpt_every) + ckpt_every + 2) states of 28 values per site, plus 17 values per site for
+ * each of the ckpt_every states of a segment (their stress, mu and H, computed once in the
  * replay) and 139 values per site of work; owned by the context until lbcad_destroy and
  * reused by later calls that fit in them.  The paper has no adjoint; this is the differentiation form
  * of the step (gradient of the droplet's drift with respect to activity, chirality and
@@ -310,7 +311,7 @@ int lbcad_sync(lbcad_ctx* c);
  * up to 279,616 sites in FP32 (64^3 fits) and 139,808 in FP64; larger grids are rejected.
  * Work: two launches on the stream, one that writes the launch descriptor (passed by value
  * as a kernel argument, so no host memory is read after the call returns) into a second
- * static array of 512 bytes, then the step kernels.
+ * static array of 1024 bytes, then the step kernels.
  * Sharing: every call on a device uses the same scratch and descriptor, so calls whose
  * work overlaps on the GPU (different streams, or host threads) race and corrupt each
  * other; serialise them.  The array keeps the last call's contents; nothing needs to

@@ -24,7 +24,8 @@ namespace lbcad {
 // Buffers of one reverse step (all [component][site]).
 template <typename T>
 struct AdjDesc {
-  InstDesc<T> I;      // state s_t in I.*_in, its sigma/mu/H in I.sig/mu/H; *_out unused
+  InstDesc<T> I;      // state s_t in I.*_in, its H in I.H; *_out unused
+  const T* S;         // its stress and mu: three quads per site [3][N][4] (see lbcad_march.cuh)
   const T* lg;        // cotangent of s_{t+1}: g* (19), Q (5), psi (1), u (3)
   const T* lq;
   const T* lp;
@@ -40,6 +41,23 @@ struct AdjDesc {
 };
 
 constexpr int kAdjBlock = 128;
+
+// GlobalAcc with the stress pairs read from the scratch quads (see QuadPlane in lbcad_march.cuh).
+template <typename T>
+struct AdjAcc : GlobalAcc<T> {
+  const T* S;
+  __device__ __forceinline__ Vec2<T> spair(int j, int cx, int cy, int cz) const {
+    const int q = j < 2 ? 0 : (j < 4 ? 1 : 2), o = (j == 1 || j == 2) ? 2 : 0;
+    const T* p = S + 4 * (q * this->N + this->nb.off(cx, cy, cz)) + o;
+    if constexpr (sizeof(T) == 4) {
+      const float2 v = __ldg(reinterpret_cast<const float2*>(p));
+      return Vec2<T>{v.x, v.y};
+    } else {
+      const double2 v = __ldg(reinterpret_cast<const double2*>(p));
+      return Vec2<T>{v.x, v.y};
+    }
+  }
+};
 
 // ---------------------------------------------------------------- reverse mode of update_math
 // Vector-Jacobian product of update_math (D3Q19 body-force collision, Euler update) at one
@@ -639,25 +657,32 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_update(AdjDesc<T> A) {
   const int x = (int)(s % nx);
   const long long t = s / nx;
   const int y = (int)(t % ny), z = (int)(t / ny);
-  GlobalAcc<T> acc;
-  acc.q_ = I.q_in; acc.ps = I.psi_in; acc.sg = I.sig; acc.mu_ = I.mu; acc.u_ = I.u_in;
+  AdjAcc<T> acc;
+  acc.q_ = I.q_in; acc.ps = I.psi_in; acc.S = A.S; acc.u_ = I.u_in;
   acc.N = N;
   acc.nb = make_nbr(x, y, z, nx, ny, nz);
   // forward inputs of update_math, packed: F 0-2, lapmu 3, Wg 4-12, q0 13-17, qf 18-47,
   // p0 48, pf 49-54, u0 55-57, uf 58-63, Hs 64-68, g 69-87
   T in[88];
   {
-    T F[3], lapmu, Wg[3][3], q0[5], qf[6][5], p0, pf[6], u0[3], uf[6];
-    gather_update<T>(acc, F, lapmu, Wg, q0, qf, p0, pf, u0, uf);
+    T F[3], lapmu, Wg[3][3], q0[5], p0, u0[3], uf[6];
+    gather_force<T>(acc, F);
+    lapmu = gather_lapmu<T>(acc);
+    gather_velocity<T>(acc, Wg, u0, uf);
+    for (int k = 0; k < 5; ++k) q0[k] = acc.q(k, 0, 0, 0);
+    p0 = acc.psi(0, 0, 0);
     for (int a = 0; a < 3; ++a) in[a] = F[a];
     in[3] = lapmu;
     for (int a = 0; a < 3; ++a)
       for (int b = 0; b < 3; ++b) in[4 + 3 * a + b] = Wg[a][b];
     for (int k = 0; k < 5; ++k) in[13 + k] = q0[k];
-    for (int f = 0; f < 6; ++f)
-      for (int k = 0; k < 5; ++k) in[18 + 5 * f + k] = qf[f][k];
+#pragma unroll
+    for (int f = 0; f < 6; ++f) {
+      const int cx = lat_c(f + 1, 0), cy = lat_c(f + 1, 1), cz = lat_c(f + 1, 2);
+      for (int k = 0; k < 5; ++k) in[18 + 5 * f + k] = acc.q(k, cx, cy, cz);
+      in[49 + f] = acc.psi(cx, cy, cz);
+    }
     in[48] = p0;
-    for (int f = 0; f < 6; ++f) in[49 + f] = pf[f];
     for (int a = 0; a < 3; ++a) in[55 + a] = u0[a];
     for (int f = 0; f < 6; ++f) in[58 + f] = uf[f];
     for (int k = 0; k < 5; ++k) in[64 + k] = I.H[k * N + s];
@@ -922,6 +947,7 @@ template <typename T, bool SHIFT>
 cudaError_t LaunchAdj<T, SHIFT>::reverse_step(const AdjDescHost<T>& h, cudaStream_t s) {
   AdjDesc<T> A;
   A.I = h.I;
+  A.S = h.S;
   A.lg = h.lg; A.lq = h.lq; A.lp = h.lp; A.lu = h.lu;
   A.A = h.A; A.Bf = h.Bf; A.ls = h.ls;
   A.og = h.og; A.oq = h.oq; A.op = h.op; A.ou = h.ou;

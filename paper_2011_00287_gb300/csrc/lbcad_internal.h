@@ -53,6 +53,15 @@ template <typename T>
 struct Coef {
   T tau_inv, guo, rho0;
   T A0, chi0, chis, K, q0, gammaQ, xi, a, b, kphi, M, W, zeta;
+  // products the kernels would otherwise form at every site
+  T A0chi1, A0chis;        // A0 (chi0 + chis), A0 chis: A0 chi = A0chi1 + A0chis psi
+  T cL, fQ2;               // A0 + 4 K q0^2, A0/2 + 2 K q0^2
+  T K2, Kq, W2;            // 2 K, 2 K q0, 2 W
+  T ah, bq, kh, zh;        // a/2, b/4, kphi/2, zeta/2
+  T xi2, xi23, xi29;       // 2 xi, 2 xi/3, 2 xi/9
+  T xip, xim;              // 1 + xi, 1 - xi
+  T omc;                   // 1 - 1/tau
+  T omw[3], gw3[3], gw9[3];  // per weight class (rest, faces, others): w/tau, 3 w guo, 9 w guo
 };
 
 // One instance of a launch: lattice, state buffers of this step parity, scratch.
@@ -99,29 +108,79 @@ struct Launch {
   static cudaError_t observables(const InstDesc<T>& I, double* partial, int nblocks, double* out, cudaStream_t s);
 };
 
-// One xy tile column of the fused step: instance, tile origin, the instance's nz and the
-// first index of this column in the flattened (tile column, z plane) work space.
-struct FusedTile {
-  int inst, x0, y0, nz;
-  long long start;
+// One instance as the marching kernels read it: sizes, coefficients, and a pointer to every component of
+// every field, so that an access's 64-bit address is one multiply-add of a 32-bit site number and a constant.
+template <typename T>
+struct MarchDesc {
+  int nx, ny, nz;
+  unsigned plane;      // nx ny
+  const T* g_in[19];   // as InstDesc, by component
+  T* g_out[19];
+  const T* q_in[5];
+  T* q_out[5];
+  const T* psi_in;
+  T* psi_out;
+  const T* u_in[3];
+  T* u_out[3];
+  T* S[3];             // scratch of the default path: three quads per site [N][4] (see lbcad_march.cuh)
+  T* H[5];             // sync coupling, Heun: H at t
+  T* rq[6];            // Heun: right-hand side at t, predicted state (Q, psi), H and mu there
+  T* qp[6];
+  T* Hp[6];
+  const T* trig;       // (cos, sin) of 2 pi x/nx, 2 pi y/ny, 2 pi z/nz
+  double mass0;        // N rho0 where the populations are stored shifted, else 0
+  Coef<T> c;
 };
 
-// A tile shape of the fused step and its launch resources.
+// The instances of one launch, passed by value: kernels read them from the constant bank.  Read from device
+// memory they stayed in registers (128^3 FP32: 88 us for k_march_fields instead of 107, and 122 for
+// k_march_lb instead of 148).  kPackMany instances fit a launch's argument space; larger batches take
+// several launches.
+constexpr int kPackMany = 28;
+template <typename T, int MI>
+struct InstPack {
+  MarchDesc<T> d[MI];
+};
+static_assert(sizeof(InstPack<double, kPackMany>) < 32000, "kernel arguments");
+
+// A work item of a marching kernel: the planes [zb, ze) of one xy tile column of an instance (index within
+// the launch).
+struct MarchItem {
+  int inst, x0, y0, zb, ze;
+};
+
+// The items of a launch, in slabs of planes: consecutive items are the tile columns of one slab, so that the
+// blocks that run at the same time share the tiles' halos and the rows they straddle in L2.
+// early: launched with programmatic dependent launch, for boxes whose step is short.
+struct MarchWork {
+  const MarchItem* items = nullptr;
+  int nitems = 0, grid = 0;
+  bool early = false;
+};
+
+// A tile shape of the step: tile sizes and resident blocks per SM of its kernels (see lbcad_march.cuh).
 struct FusedCfg {
-  int tx = 0, ty = 0, threads = 0, blocks_per_sm = 0;
-  size_t smem = 0;
+  int fx = 0, fy = 0, lx = 0, ly = 0;          // tiles of k_march_fields, of k_march_lb and the order-parameter kernels
+  int fields_per_sm = 0, lb_per_sm = 0;        // k_march_fields, k_march_lb
+  int pred_per_sm = 0, op_per_sm[2] = {0, 0};  // sync, Heun: fields at the predicted state, order-parameter kernels
 };
 
-// What a fused step kernel does: the whole step (kFusedPlain), the whole step and the a6 sums
-// (kFusedSums), or the LB half of a sync-coupled step (kFusedLbOnly).
+// The work of one step for a group of instances (at most kPackMany).
+struct StepWork {
+  int first = 0, ninst = 0;  // instances of the group
+  MarchWork fields, lb, pred, op[2];
+};
+
+// What k_march_lb does: collision and psi (kFusedPlain), with the a6 sums (kFusedSums), or the collision
+// alone (kFusedLbOnly: sync coupling, Heun).
 constexpr int kFusedPlain = 0, kFusedSums = 1, kFusedLbOnly = 2;
 
-// The FP64 conserved and centroid sums of the fused step (a6).  Each column segment a block
-// works on has a slot of 12 partial sums (block b, segment j of the block: slot b * maxseg + j);
+// The FP64 conserved and centroid sums of the step (a6).  Each run of items of one instance that a block works
+// on has a slot of 12 partial sums (block b, run j of the block: slot b * maxrun + j);
 // slot_inst[slot] is its instance (-1: unused).  At the end of the kernel each block counts its
 // slots on their instances (cnt; the kernel resets it), and the block whose count completes an
 // instance sums the instance's slots in a fixed order into latest[inst][12]: mass, sum psi,
-// momentum (3), sum phi_c cos (3), sum phi_c sin (3), sum phi_c.
+// momentum (3), sum phi_c cos (3), sum phi_c sin (3), sum phi_c.  Instances are numbered within the launch.
 struct FusedObs {
   double* slots;
   const int* slot_inst;
@@ -130,35 +189,36 @@ struct FusedObs {
   const int* slot_hi;  // [ninst] one past its last slot
   unsigned* cnt;       // [ninst]
   double* latest;      // [ninst][12]
-  int maxseg;
+  int maxrun;
 };
 
-// The fused one-kernel step (lbcad_fused.cuh), in several tile shapes, for each variant
-// of the LB part: variant = (D3Q15 ? 1 : 0) + 2 * (Eq. 9-11 form ? 1 : 0).  prepare returns
-// cudaErrorNotSupported for a tile shape the variant does not come in.
+// The default path (lbcad_march.cuh), in several tile shapes, for each variant of the LB part:
+// variant = (D3Q15 ? 1 : 0) + 2 * (Eq. 9-11 form ? 1 : 0).  prepare returns cudaErrorNotSupported for
+// a tile shape the variant does not come in.
 template <typename T, bool SHIFT>
 struct LaunchFused {
   static int num_configs();
-  static cudaError_t prepare(int variant, int cfg_index, FusedCfg* cfg);
-  // obs: the kernel that also forms the a6 sums of the new state (FusedObs)
-  static cudaError_t step(int variant, int cfg_index, const InstDesc<T>* d_desc, const FusedTile* tiles,
-                          int ntiles, long long total, int grid, const FusedObs& ob, bool obs, cudaStream_t s);
-  // Sync coupling or Heun: the first half of the step (force, pull, collision, u of this step;
-  // H and mu of every site into the scratch), on tile shape sync_config(); op_tiled finishes it.
-  static int sync_config();
-  static cudaError_t step_lb(int variant, const InstDesc<T>* d_desc, const FusedTile* tiles, int ntiles,
-                             long long total, int grid, const FusedObs& ob, cudaStream_t s);
-  // The order-parameter half after step_lb as tiled z-marching kernels on the same tiles (32 x 8,
-  // the tile shape of sync_config()): the update (Euler), or predictor, fields at the predicted
-  // state and corrector (Heun); sync advects with u of this step.
-  static cudaError_t op_tiled(bool heun, bool sync, const InstDesc<T>* d_desc, const FusedTile* tiles, int ntiles,
-                              long long total, cudaStream_t s);
+  // many: for launches of several instances
+  static cudaError_t prepare(int variant, int k, bool many, bool split, bool heun, FusedCfg* cfg);
+  // Euler with the velocity of the previous step; obs: also the a6 sums of the new state (FusedObs).
+  // d: the descriptors of the group's instances (host memory, copied into the launch).
+  static cudaError_t step(int variant, int k, const StepWork& w, const MarchDesc<T>* d, const FusedObs& ob, bool obs,
+                          cudaStream_t s);
+  // Sync coupling or Heun: fields, LB half (u of this step), then the order-parameter half: the update
+  // (Euler), or predictor, fields at the predicted state and corrector (Heun).
+  static cudaError_t split_step(int variant, int k, const StepWork& w, bool heun, bool sync, const MarchDesc<T>* d,
+                                cudaStream_t s);
+  // The adjoint's replay: one Euler step of D3Q19 with the body force that also leaves S and H of the state it
+  // steps from; last: S and H only.
+  static cudaError_t prepare_replay(int k);
+  static cudaError_t replay(int k, const StepWork& w, bool last, const MarchDesc<T>* d, cudaStream_t s);
 };
 
 // Buffers of one reverse step of the adjoint (lbcad_adjoint.cuh).
 template <typename T>
 struct AdjDescHost {
-  InstDesc<T> I;                 // state s_t (inputs) and its sigma/mu/H scratch
+  InstDesc<T> I;                 // state s_t (inputs) and its H
+  const T* S;                    // its stress and mu: three quads per site [3][N][4] (see lbcad_march.cuh)
   const T *lg, *lq, *lp, *lu;    // cotangent of s_{t+1}
   T *A, *Bf, *ls;                // work: 88 + 36 + 15 values per site
   T *og, *oq, *op, *ou;          // cotangent of s_t

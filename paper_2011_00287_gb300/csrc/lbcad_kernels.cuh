@@ -106,36 +106,56 @@ struct Vec2 {
 };
 template <typename T>
 __device__ __forceinline__ Vec2<T> v2(T a, T b) { return Vec2<T>{a, b}; }
-template <typename T>
-__device__ __forceinline__ Vec2<T> add2(Vec2<T> a, Vec2<T> b) { return Vec2<T>{a.x + b.x, a.y + b.y}; }
-template <typename T>
-__device__ __forceinline__ Vec2<T> sub2(Vec2<T> a, Vec2<T> b) { return Vec2<T>{a.x - b.x, a.y - b.y}; }
-template <typename T>
-__device__ __forceinline__ Vec2<T> fma2(Vec2<T> a, Vec2<T> b, Vec2<T> c) {
-  return Vec2<T>{a.x * b.x + c.x, a.y * b.y + c.y};
-}
-template <typename T>
-__device__ __forceinline__ Vec2<T> mul2(Vec2<T> a, Vec2<T> b) { return Vec2<T>{a.x * b.x, a.y * b.y}; }
+// Every multiply-add is an explicit fma and every lone product is rounded on its own, so the
+// stencils round identically in every kernel that inlines them, whatever the compiler would
+// contract.  Scalar overloads let one stencil serve single fields and pairs.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float add2(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add2(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float sub2(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ double sub2(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ float fma2(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma2(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ float mul2(float a, float b) { return mul_rn(a, b); }
+__device__ __forceinline__ double mul2(double a, double b) { return mul_rn(a, b); }
 __device__ __forceinline__ float2 f2(Vec2<float> a) { return make_float2(a.x, a.y); }
 __device__ __forceinline__ Vec2<float> v2f(float2 a) { return Vec2<float>{a.x, a.y}; }
-template <>
 __device__ __forceinline__ Vec2<float> add2(Vec2<float> a, Vec2<float> b) { return v2f(__fadd2_rn(f2(a), f2(b))); }
-template <>
 __device__ __forceinline__ Vec2<float> sub2(Vec2<float> a, Vec2<float> b) {
   return v2f(__ffma2_rn(f2(b), make_float2(-1.f, -1.f), f2(a)));  // a - b, one rounding
 }
-template <>
 __device__ __forceinline__ Vec2<float> fma2(Vec2<float> a, Vec2<float> b, Vec2<float> c) {
   return v2f(__ffma2_rn(f2(a), f2(b), f2(c)));
 }
-template <>
 __device__ __forceinline__ Vec2<float> mul2(Vec2<float> a, Vec2<float> b) { return v2f(__fmul2_rn(f2(a), f2(b))); }
+__device__ __forceinline__ Vec2<double> add2(Vec2<double> a, Vec2<double> b) {
+  return Vec2<double>{add2(a.x, b.x), add2(a.y, b.y)};
+}
+__device__ __forceinline__ Vec2<double> sub2(Vec2<double> a, Vec2<double> b) {
+  return Vec2<double>{sub2(a.x, b.x), sub2(a.y, b.y)};
+}
+__device__ __forceinline__ Vec2<double> fma2(Vec2<double> a, Vec2<double> b, Vec2<double> c) {
+  return Vec2<double>{fma(a.x, b.x, c.x), fma(a.y, b.y, c.y)};
+}
+__device__ __forceinline__ Vec2<double> mul2(Vec2<double> a, Vec2<double> b) {
+  return Vec2<double>{mul_rn(a.x, b.x), mul_rn(a.y, b.y)};
+}
+// The constant k in every lane of a value of type V.
+template <class V>
+struct Bcast {
+  __device__ __forceinline__ static V of(double k) { return V(k); }
+};
+template <typename T>
+struct Bcast<Vec2<T>> {
+  __device__ __forceinline__ static Vec2<T> of(double k) { return Vec2<T>{T(k), T(k)}; }
+};
 
 // Gradient (1/12)[2 D_face + signed edge pairs] from opposite-pair differences D[i] =
-// f(c_i) - f(c_{i+1}), two fields at once.
-template <typename T>
-__device__ __forceinline__ void grad2_from_pairs(const Vec2<T> D[19], Vec2<T> g[3]) {
-  const Vec2<T> k2 = v2(T(2), T(2)), k12 = v2(T(1.0 / 12.0), T(1.0 / 12.0));
+// f(c_i) - f(c_{i+1}) of one field or two (V = T or Vec2<T>).
+template <class V>
+__device__ __forceinline__ void grad_from_pairs(const V D[19], V g[3]) {
+  const V k2 = Bcast<V>::of(2.0), k12 = Bcast<V>::of(1.0 / 12.0);
   g[0] = mul2(fma2(D[1], k2, add2(add2(D[7], D[9]), add2(D[11], D[13]))), k12);
   g[1] = mul2(fma2(D[3], k2, add2(sub2(D[7], D[9]), add2(D[15], D[17]))), k12);
   g[2] = mul2(fma2(D[5], k2, add2(sub2(D[11], D[13]), sub2(D[15], D[17]))), k12);
@@ -163,7 +183,7 @@ __device__ __forceinline__ void local_fields(const Coef<T>& c, const T q[5], T p
   T dQ[3][3][3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) full3(dq[a], dQ[a]);
-  const T chi = c.chi0 + c.chis * (T(1) + psi);
+  const T third = T(1.0 / 3.0);
   // Q.Q is symmetric: six products
   T QQ[3][3];
 #pragma unroll
@@ -193,17 +213,17 @@ __device__ __forceinline__ void local_fields(const Coef<T>& c, const T q[5], T p
       CC[j][i] = CC[i][j];
     }
   const T g2 = dp[0] * dp[0] + dp[1] * dp[1] + dp[2] * dp[2];
-  const T Ac = c.A0 * chi;
-  const T Kq = T(2) * c.K * c.q0;
-  const T lin = -c.A0 * (T(1) - chi / T(3)) - Ac * trQ2 - Kq * T(2) * c.q0;
-  const T iso = (Ac * trQ2 - c.W * g2) / T(3);
+  const T Ac = c.A0chis * psi + c.A0chi1;  // A0 chi
+  const T lin = Ac * (third - trQ2) - c.cL;
+  const T iso = third * (Ac * trQ2 - c.W * g2);
+  const T Wdp[3] = {c.W * dp[0], c.W * dp[1], c.W * dp[2]};
   // H = -dF/dQ (traceless symmetric by construction: tr CC = 0 for symmetric Q)
   const int I5[5] = {0, 0, 0, 1, 1};
   const int J5[5] = {0, 1, 2, 1, 2};
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
     const int i = I5[k], j = J5[k];
-    T h = lin * Q[i][j] + Ac * QQ[i][j] + c.K * lapq[k] - Kq * CC[i][j] - c.W * dp[i] * dp[j];
+    T h = lin * Q[i][j] + Ac * QQ[i][j] + c.K * lapq[k] - c.Kq * CC[i][j] - Wdp[i] * dp[j];
     if (i == j) h -= iso;
     H[k] = h;
   }
@@ -217,29 +237,41 @@ __device__ __forceinline__ void local_fields(const Coef<T>& c, const T q[5], T p
 #pragma unroll
   for (int b = 0; b < 3; ++b) divQdp += (dQ[0][0][b] + dQ[1][1][b] + dQ[2][2][b]) * dp[b];
   const T psi2 = psi * psi;
-  mu = psi * (c.b * psi2 - c.a) - c.kphi * lapp + c.A0 * c.chis * (trQ2 * (T(0.25) * trQ2 - T(1) / T(6)) - trQ3 / T(3)) -
-       T(2) * c.W * (divQdp + Qh);
+  const T bulk = trQ2 * (T(0.25) * trQ2 - T(1.0 / 6.0)) - third * trQ3;
+  mu = psi * (c.b * psi2 - c.a) - c.kphi * lapp + c.A0chis * bulk - c.W2 * (divQdp + Qh);
 
-  // Gram matrix of the Q derivatives (symmetric), Q:curl Q, Q.grad psi
-  T G[3][3];
+  // Elastic stress E_ab = K dQ_a : dQ_b + Kq v_b(dQ_a), v_b(M) = eps_bgm (M Q)_gm the axial vector
+  // of M Q.  Both are linear in dQ_a, so E_ab = dQ_a : t_b with one symmetric t_b = K dQ_b +
+  // Kq n_b per b; on the five stored components of the traceless dQ_a it takes five products
+  // (off-diagonal entries of t doubled, t_zz subtracted from the diagonal).
+  const T kxy = c.Kq * Q[0][1], kxz = c.Kq * Q[0][2], kyz = c.Kq * Q[1][2];
+  const T kzy = c.Kq * (Q[2][2] - Q[1][1]), kxx = c.Kq * (Q[0][0] - Q[2][2]), kyx = c.Kq * (Q[1][1] - Q[0][0]);
+  T t[3][5];
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    const T ax = T(2) * dq[b][0] + dq[b][3], ay = dq[b][0] + T(2) * dq[b][3];
+    t[b][0] = c.K * ax + (b == 0 ? kyz : b == 1 ? -T(2) * kxz : kxy);
+    t[b][3] = c.K * ay + (b == 0 ? T(2) * kyz : b == 1 ? -kxz : -kxy);
+    t[b][1] = c.K2 * dq[b][1] + (b == 0 ? kxz : b == 1 ? -kyz : kyx);
+    t[b][2] = c.K2 * dq[b][2] + (b == 0 ? -kxy : b == 1 ? kxx : kyz);
+    t[b][4] = c.K2 * dq[b][4] + (b == 0 ? kzy : b == 1 ? kxy : -kxz);
+  }
+  T E[3][3];
 #pragma unroll
   for (int a = 0; a < 3; ++a)
 #pragma unroll
-    for (int b = a; b < 3; ++b) {
-      const T s = dQ[a][0][0] * dQ[b][0][0] + dQ[a][1][1] * dQ[b][1][1] + dQ[a][2][2] * dQ[b][2][2] +
-                  T(2) * (dQ[a][0][1] * dQ[b][0][1] + dQ[a][0][2] * dQ[b][0][2] + dQ[a][1][2] * dQ[b][1][2]);
-      G[a][b] = s;
-      G[b][a] = s;
-    }
+    for (int b = 0; b < 3; ++b)
+      E[a][b] = dq[a][0] * t[b][0] + dq[a][1] * t[b][1] + dq[a][2] * t[b][2] + dq[a][3] * t[b][3] + dq[a][4] * t[b][4];
+  // Q:curl Q (= sum_a v_a(dQ_a)), Q.grad psi
   const T QC = Q[0][0] * C[0][0] + Q[1][1] * C[1][1] + Q[2][2] * C[2][2] + Q[0][1] * CC[0][1] +
                Q[0][2] * CC[0][2] + Q[1][2] * CC[1][2];
   T Qdp[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) Qdp[i] = Q[i][0] * dp[0] + Q[i][1] * dp[1] + Q[i][2] * dp[2];
   const T anch = dp[0] * Qdp[0] + dp[1] * Qdp[1] + dp[2] * Qdp[2];
-  const T fden = psi2 * (T(0.25) * c.b * psi2 - T(0.5) * c.a) + T(0.5) * c.kphi * g2 +
-                 c.A0 * (T(0.5) * (T(1) - chi / T(3)) * trQ2 - chi / T(3) * trQ3 + chi / T(4) * trQ2 * trQ2) +
-                 T(0.5) * c.K * (G[0][0] + G[1][1] + G[2][2]) + Kq * QC + Kq * c.q0 * trQ2 + c.W * anch;
+  // K/2 dQ:dQ + Kq Q:curl Q = (tr E + Kq Q:curl Q)/2; the A0 terms are A0/2 trQ2 + A0 chi bulk
+  const T fden = psi2 * (c.bq * psi2 - c.ah) + c.kh * g2 + c.fQ2 * trQ2 + Ac * bulk +
+                 T(0.5) * (E[0][0] + E[1][1] + E[2][2] + c.Kq * QC) + c.W * anch;
   const T P0 = psi * mu - fden;
 
   // reactive and active parts: with (HQ)_ab = (QH)_ba,
@@ -251,267 +283,332 @@ __device__ __forceinline__ void local_fields(const Coef<T>& c, const T q[5], T p
 #pragma unroll
     for (int j = 0; j < 3; ++j) QH[i][j] = Q[i][0] * Hf[0][j] + Q[i][1] * Hf[1][j] + Q[i][2] * Hf[2][j];
   const T trQH = QH[0][0] + QH[1][1] + QH[2][2];
-  const T phic = T(0.5) * (T(1) + psi);
-  const T cQ = T(2) * c.xi * trQH - c.zeta * phic;
-  const T cI = T(2) * c.xi / T(3) * trQH - P0;
-  const T cH = -T(2) * c.xi / T(3);
-  const T cP = T(1) - c.xi, cM = -(T(1) + c.xi);
+  const T cQ = c.xi2 * trQH - (c.zh * psi + c.zh);  // zeta phi_c = zeta (1 + psi)/2
+  const T cI = c.xi23 * trQH - P0;
   T wv[3];
 #pragma unroll
-  for (int b = 0; b < 3; ++b) wv[b] = c.kphi * dp[b] + T(2) * c.W * Qdp[b];
+  for (int b = 0; b < 3; ++b) wv[b] = c.kphi * dp[b] + c.W2 * Qdp[b];
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    // v_b = eps_bgm (dQ_a Q)_gm: the axial vector of the antisymmetric part of dQ_a Q
-    T v[3];
+  for (int a = 0; a < 3; ++a)
 #pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      const int g = (b + 1) % 3, m = (b + 2) % 3;
-      v[b] = dQ[a][g][0] * Q[0][m] + dQ[a][g][1] * Q[1][m] + dQ[a][g][2] * Q[2][m] -
-             (dQ[a][m][0] * Q[0][g] + dQ[a][m][1] * Q[1][g] + dQ[a][m][2] * Q[2][g]);
+    for (int b = a; b < 3; ++b) {
+      const T sb = cQ * Q[a][b] - c.xi23 * Hf[a][b];  // the part symmetric in a, b
+      if (a == b) {
+        sig[4 * a] = sb + cI - c.xi2 * QH[a][a] - E[a][a] - dp[a] * wv[a];
+      } else {
+        sig[3 * a + b] = sb + c.xim * QH[a][b] - c.xip * QH[b][a] - E[a][b] - dp[a] * wv[b];
+        sig[3 * b + a] = sb + c.xim * QH[b][a] - c.xip * QH[a][b] - E[b][a] - dp[b] * wv[a];
+      }
     }
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      T s = cQ * Q[a][b] + cP * QH[a][b] + cM * QH[b][a] + cH * Hf[a][b] - c.K * G[a][b] - Kq * v[b] - dp[a] * wv[b];
-      if (a == b) s += cI;
-      sig[3 * a + b] = s;
-    }
-  }
 }
 
 // ---------------------------------------------------------------- shared per-site pieces
-// Both step paths (two kernels through global memory, one fused kernel through shared
-// memory tiles) evaluate their stencils with the functions below, in the same order and
-// with the same arithmetic, through an accessor A that returns neighbour values:
-//   A::q(k, cx, cy, cz), A::psi(cx, cy, cz)            (gather_fields)
-//   A::sig(k, ...), A::mu(...), A::u(a, ...), q, psi   (gather_update)
-// With cx, cy, cz compile-time constants after unrolling, a shared-memory accessor
-// turns every neighbour read into one load at an immediate offset.
+// Every step path evaluates its stencils with the functions below, in the same order and with
+// the same arithmetic, through an accessor A that returns neighbour values: pairs of fields
+// A::pair(j, ...) (see gather_fields), pairs of stresses A::spair(j, ...) (see sig_pair) and
+// the velocity A::u3(...).
 //
-// D3Q19 velocities come in opposite pairs (i, i+1) for odd i, so the isotropic gradient
-// 3 Sum_i w_i c_i f(x + c_i) is (1/12) Sum_pairs c_i (f_i - f_{i+1}) (x2 for faces):
-//   d_x = [2 D1 + D7 + D9 + D11 + D13]/12,  d_y = [2 D3 + D7 - D9 + D15 + D17]/12,
-//   d_z = [2 D5 + D11 - D13 + D15 - D17]/12,  D_i = f(x + c_i) - f(x + c_{i+1}).
-// Laplacians are sums of differences to the centre value (Sum_i w_i c_i = 0), which
-// keeps them free of cancellation in FP32.
-
-template <typename T>
-__device__ __forceinline__ void grad_from_pairs(const T D[19], T g[3]) {
-  g[0] = (T(2) * D[1] + D[7] + D[9] + D[11] + D[13]) * T(1.0 / 12.0);
-  g[1] = (T(2) * D[3] + D[7] - D[9] + D[15] + D[17]) * T(1.0 / 12.0);
-  g[2] = (T(2) * D[5] + D[11] - D[13] + D[15] - D[17]) * T(1.0 / 12.0);
-}
-
-// Laplacian from differences to the centre: (1/3) Sum_faces d + (1/6) Sum_edges d.
-template <typename T>
-__device__ __forceinline__ T lap_from_diffs(const T d[19]) {
-  const T sf = (d[1] + d[2]) + (d[3] + d[4]) + (d[5] + d[6]);
-  const T se = ((d[7] + d[8]) + (d[9] + d[10])) + ((d[11] + d[12]) + (d[13] + d[14])) +
-               ((d[15] + d[16]) + (d[17] + d[18]));
-  return (T(2) * sf + se) * T(1.0 / 6.0);
-}
+// The 19-point stencils (rest, six faces, twelve edges) are sums over three planes z-1, z, z+1
+// of in-plane sums, and the in-plane sums of a plane serve three output planes.  So the
+// stencils are written as carries: advance() takes the nine points of one new plane, finishes
+// the output of the plane before it and keeps what the next plane needs.  A kernel that
+// marches up z reads nine points per field and plane instead of 19 and adds 38 instead of 63
+// times; a per-site kernel runs the same carry over its three planes, so that all paths round
+// alike.  With D f the in-plane difference f(+1) - f(-1), S the sum of the four in-plane
+// neighbours' differences to the centre, S2 that of the four diagonal ones, and f+- the
+// plane's centre value above and below:
+//   d_x f = [2 D_x + D_x(y+1) + D_x(y-1) + D_x(z+1) + D_x(z-1)] / 12,   d_y likewise,
+//   d_z f = [(6 (f+ - f) + S(z+1)) - (6 (f- - f) + S(z-1))] / 12,
+//   lap f = [2 S + S2 + (6 (f+ - f) + S(z+1)) + (6 (f- - f) + S(z-1))] / 6.
+// Sums are taken of differences to a centre value, which keeps them free of cancellation in
+// FP32.
 
 // a1: gradient and Laplacian of the five Q components and psi, and the Hessian of psi
 // (three-point differences on the diagonal, four corners off it).  The six fields are
-// taken in pairs (Q_xx, Q_xy), (Q_xz, Q_yy), (Q_yz, psi) through A::pair(j, ...), so one
-// two-lane operation advances two fields.
+// taken in pairs (Q_xx, Q_xy), (Q_xz, Q_yy), (Q_yz, psi), so one two-lane operation advances
+// two fields.
+template <typename T>
+struct FieldsCarry {
+  using V = Vec2<T>;
+  V c[3], dx[3], dy[3], s4[3];  // of the last plane: value, differences, sum over the neighbours
+  V A[3], B[3];                 // its own part of 12 d_x, 12 d_y and that of the plane below
+  V L[3], Z[3];                 // ... of 6 lap, and the part of the plane below of 12 d_z
+  T hxx, hyy, hxy;              // psi: in-plane second differences of the last plane
+  T px, py, fm;                 // psi: dx, dy of the plane below, and psi there minus psi
+  __device__ __forceinline__ FieldsCarry() {
+#pragma unroll
+    for (int j = 0; j < 3; ++j) c[j] = dx[j] = dy[j] = s4[j] = A[j] = B[j] = L[j] = Z[j] = V{T(0), T(0)};
+    hxx = hyy = hxy = px = py = fm = T(0);
+  }
+  // pl(j, cx, cy): pair j of the new plane.  Outputs: the plane before it.
+  template <class P>
+  __device__ __forceinline__ void advance(const P& pl, T q0[5], T& p0, T dq[3][5], T lapq[5], T dp[3], T& lapp,
+                                          T hp[6]) {
+    const V k2 = Bcast<V>::of(2.0), k6 = Bcast<V>::of(6.0), m6 = Bcast<V>::of(-6.0);
+    const V k12i = Bcast<V>::of(1.0 / 12.0), k6i = Bcast<V>::of(1.0 / 6.0);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const V f0 = pl(j, 0, 0), fe = pl(j, 1, 0), fw = pl(j, -1, 0), fn = pl(j, 0, 1), fs = pl(j, 0, -1);
+      const V ne = pl(j, 1, 1), sw = pl(j, -1, -1), se = pl(j, 1, -1), nw = pl(j, -1, 1);
+      const V ndx = sub2(fe, fw), ndy = sub2(fn, fs);
+      const V sx = add2(sub2(fe, f0), sub2(fw, f0)), sy = add2(sub2(fn, f0), sub2(fs, f0));
+      const V ns4 = add2(sx, sy);
+      const V s1 = add2(sub2(ne, f0), sub2(sw, f0)), s2 = add2(sub2(se, f0), sub2(nw, f0));
+      const V p = sub2(ne, sw), m = sub2(se, nw);
+      const V gx = fma2(k2, ndx, add2(p, m)), gy = fma2(k2, ndy, sub2(p, m));
+      const V lp = fma2(k2, ns4, add2(s1, s2));
+      // the plane before
+      const V fp = sub2(f0, c[j]);
+      const V e = fma2(k6, fp, ns4);
+      const V ox = mul2(add2(A[j], ndx), k12i), oy = mul2(add2(B[j], ndy), k12i);
+      const V oz = mul2(sub2(e, Z[j]), k12i), ol = mul2(add2(L[j], e), k6i);
+      const int k0 = 2 * j;
+      q0[k0] = c[j].x;
+      dq[0][k0] = ox.x;
+      dq[1][k0] = oy.x;
+      dq[2][k0] = oz.x;
+      lapq[k0] = ol.x;
+      if (j < 2) {
+        q0[k0 + 1] = c[j].y;
+        dq[0][k0 + 1] = ox.y;
+        dq[1][k0 + 1] = oy.y;
+        dq[2][k0 + 1] = oz.y;
+        lapq[k0 + 1] = ol.y;
+      } else {
+        p0 = c[j].y;
+        dp[0] = ox.y;
+        dp[1] = oy.y;
+        dp[2] = oz.y;
+        lapp = ol.y;
+        hp[0] = hxx;
+        hp[1] = hyy;
+        hp[2] = add2(fp.y, fm);
+        hp[3] = hxy;
+        hp[4] = mul_rn(T(0.25), sub2(ndx.y, px));
+        hp[5] = mul_rn(T(0.25), sub2(ndy.y, py));
+        hxx = sx.y;
+        hyy = sy.y;
+        hxy = mul_rn(T(0.25), sub2(s1.y, s2.y));
+        px = dx[j].y;
+        py = dy[j].y;
+        fm = -fp.y;
+      }
+      // this plane
+      Z[j] = fma2(m6, fp, s4[j]);
+      A[j] = add2(gx, dx[j]);
+      B[j] = add2(gy, dy[j]);
+      L[j] = add2(lp, Z[j]);
+      c[j] = f0;
+      dx[j] = ndx;
+      dy[j] = ndy;
+      s4[j] = ns4;
+    }
+  }
+};
+
+// The same at one site, from its three planes.
 template <typename T, class A>
 __device__ __forceinline__ void gather_fields(const A& acc, T q0[5], T& p0, T dq[3][5], T lapq[5], T dp[3],
                                               T& lapp, T hp[6]) {
-  using V = Vec2<T>;
-  const V k2 = v2(T(2), T(2)), k6 = v2(T(1.0 / 6.0), T(1.0 / 6.0));
+  FieldsCarry<T> car;
 #pragma unroll
-  for (int j = 0; j < 3; ++j) {
-    V f[19];
-#pragma unroll
-    for (int i = 0; i < 19; ++i) f[i] = acc.pair(j, lat_c(i, 0), lat_c(i, 1), lat_c(i, 2));
-    V d[19], D[19];
-#pragma unroll
-    for (int i = 1; i < 19; ++i) d[i] = sub2(f[i], f[0]);
-#pragma unroll
-    for (int i = 1; i < 19; i += 2) D[i] = sub2(d[i], d[i + 1]);
-    V g[3];
-    grad2_from_pairs<T>(D, g);
-    // Laplacian from differences to the centre: (1/3) faces + (1/6) edges
-    const V sf = add2(add2(add2(d[1], d[2]), add2(d[3], d[4])), add2(d[5], d[6]));
-    const V se = add2(add2(add2(add2(d[7], d[8]), add2(d[9], d[10])), add2(add2(d[11], d[12]), add2(d[13], d[14]))),
-                      add2(add2(d[15], d[16]), add2(d[17], d[18])));
-    const V lp = mul2(fma2(sf, k2, se), k6);
-    const int k0 = 2 * j;
-    q0[k0] = f[0].x;
-    lapq[k0] = lp.x;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) dq[a][k0] = g[a].x;
-    if (j < 2) {
-      q0[k0 + 1] = f[0].y;
-      lapq[k0 + 1] = lp.y;
-#pragma unroll
-      for (int a = 0; a < 3; ++a) dq[a][k0 + 1] = g[a].y;
-    } else {
-      p0 = f[0].y;
-      lapp = lp.y;
-#pragma unroll
-      for (int a = 0; a < 3; ++a) dp[a] = g[a].y;
-      hp[0] = d[1].y + d[2].y;
-      hp[1] = d[3].y + d[4].y;
-      hp[2] = d[5].y + d[6].y;
-      hp[3] = T(0.25) * ((d[7].y + d[8].y) - (d[9].y + d[10].y));
-      hp[4] = T(0.25) * ((d[11].y + d[12].y) - (d[13].y + d[14].y));
-      hp[5] = T(0.25) * ((d[15].y + d[16].y) - (d[17].y + d[18].y));
-    }
-  }
+  for (int cz = -1; cz <= 1; ++cz)
+    car.advance([&](int j, int cx, int cy) { return acc.pair(j, cx, cy, cz); }, q0, p0, dq, lapq, dp, lapp, hp);
 }
 
-// a3 (divergence): F_a = d_b sigma_ab from opposite-pair differences of sigma, through the
-// stress pairs A::spair(j, ...): (F_x, F_y) from pairs 0-2 two lanes at a time, F_z from
-// pair 3 (sigma_zx, sigma_zy) and lane 0 of pair 4 (sigma_zz).
+// a3 (divergence): F_a = d_b sigma_ab, through the stress pairs of a plane: (F_x, F_y) from
+// pairs 0-2 two lanes at a time, F_z from pair 3 (sigma_zx, sigma_zy) and lane 0 of pair 4
+// (sigma_zz).
+template <class V>
+struct DivCarry {
+  V P, A1, s4, c;  // the last plane's sum so far; its in-plane differences; of sigma_az: neighbours, value
+  __device__ __forceinline__ DivCarry() { P = A1 = s4 = c = Bcast<V>::of(0.0); }
+  // x(cx, cy), y(cx, cy), z(cx, cy): sigma_ax, sigma_ay, sigma_az of the new plane; returns F of
+  // the plane before it.
+  template <class X, class Y, class Zf>
+  __device__ __forceinline__ V advance(const X& x, const Y& y, const Zf& z) {
+    const V k2 = Bcast<V>::of(2.0), k6 = Bcast<V>::of(6.0), m6 = Bcast<V>::of(-6.0), k12i = Bcast<V>::of(1.0 / 12.0);
+    const V a1 = add2(sub2(x(1, 0), x(-1, 0)), sub2(y(0, 1), y(0, -1)));
+    const V d = add2(add2(sub2(x(1, 1), x(-1, -1)), sub2(x(1, -1), x(-1, 1))),
+                     sub2(sub2(y(1, 1), y(-1, -1)), sub2(y(1, -1), y(-1, 1))));
+    const V z0 = z(0, 0);
+    const V ns4 = add2(add2(sub2(z(1, 0), z0), sub2(z(-1, 0), z0)), add2(sub2(z(0, 1), z0), sub2(z(0, -1), z0)));
+    const V e = sub2(z0, c);
+    const V F = mul2(add2(P, add2(a1, fma2(k6, e, ns4))), k12i);
+    P = sub2(add2(fma2(k2, a1, d), A1), fma2(m6, e, s4));
+    A1 = a1;
+    s4 = ns4;
+    c = z0;
+    return F;
+  }
+};
+template <typename T>
+struct ForceCarry {
+  DivCarry<Vec2<T>> xy;
+  DivCarry<T> z;
+  template <class P>
+  __device__ __forceinline__ void advance(const P& sp, T F[3]) {
+    const Vec2<T> f = xy.advance([&](int cx, int cy) { return sp(0, cx, cy); },
+                                 [&](int cx, int cy) { return sp(1, cx, cy); },
+                                 [&](int cx, int cy) { return sp(2, cx, cy); });
+    F[0] = f.x;
+    F[1] = f.y;
+    F[2] = z.advance([&](int cx, int cy) { return sp(3, cx, cy).x; }, [&](int cx, int cy) { return sp(3, cx, cy).y; },
+                     [&](int cx, int cy) { return sp(4, cx, cy).x; });
+  }
+};
+
+// Laplacian of one field; f(cx, cy): the new plane.
+template <typename T>
+struct LapCarry {
+  T c = T(0), s4 = T(0), L = T(0), fm = T(0);
+  template <class P>
+  __device__ __forceinline__ T advance(const P& f) {
+    const T f0 = f(0, 0);
+    const T ns4 = add2(add2(sub2(f(1, 0), f0), sub2(f(-1, 0), f0)), add2(sub2(f(0, 1), f0), sub2(f(0, -1), f0)));
+    const T s2 = add2(add2(sub2(f(1, 1), f0), sub2(f(-1, -1), f0)), add2(sub2(f(1, -1), f0), sub2(f(-1, 1), f0)));
+    const T fp = sub2(f0, c);
+    const T lap = mul2(fma2(T(6), add2(fp, fm), add2(L, ns4)), T(1.0 / 6.0));
+    L = add2(fma2(T(2), ns4, s2), s4);
+    c = f0;
+    s4 = ns4;
+    fm = -fp;
+    return lap;
+  }
+};
+
 template <typename T, class A>
 __device__ __forceinline__ void gather_force(const A& acc, T F[3]) {
+  ForceCarry<T> car;
+#pragma unroll
+  for (int cz = -1; cz <= 1; ++cz)
+    car.advance([&](int j, int cx, int cy) { return acc.spair(j, cx, cy, cz); }, F);
+}
+
+// lap mu (lane 1 of stress pair 4).
+template <typename T, class A>
+__device__ __forceinline__ T gather_lapmu(const A& acc) {
+  LapCarry<T> car;
+  T l = T(0);
+#pragma unroll
+  for (int cz = -1; cz <= 1; ++cz) l = car.advance([&](int cx, int cy) { return acc.spair(4, cx, cy, cz).y; });
+  return l;
+}
+
+// The velocity of one site as (u_x, u_y) and u_z.
+template <typename T>
+struct Vel3 {
+  Vec2<T> xy;
+  T z;
+};
+
+// W_ab = d_b u_a and the axial face velocities (face slot 2a: u_a at +e_a, 2a+1: at -e_a).
+template <typename T, class A>
+__device__ __forceinline__ void gather_velocity(const A& acc, T Wg[3][3], T u0[3], T uf[6]) {
   using V = Vec2<T>;
-  V a2 = v2(T(0), T(0)), a1 = v2(T(0), T(0));
+  V f[19], D[19], g[3];
+  T fz[19], Dz[19];
 #pragma unroll
-  for (int b = 0; b < 3; ++b) {
-#pragma unroll
-    for (int i = 1; i < 19; i += 2) {
-      const int cb = lat_c(i, b);
-      if (cb == 0) continue;
-      const V D = sub2(acc.spair(b, lat_c(i, 0), lat_c(i, 1), lat_c(i, 2)),
-                       acc.spair(b, lat_c(i + 1, 0), lat_c(i + 1, 1), lat_c(i + 1, 2)));
-      if (lat_c2(i) == 1) a2 = cb > 0 ? add2(a2, D) : sub2(a2, D);
-      else a1 = cb > 0 ? add2(a1, D) : sub2(a1, D);
-    }
+  for (int i = 0; i < 19; ++i) {
+    const Vel3<T> v = acc.u3(lat_c(i, 0), lat_c(i, 1), lat_c(i, 2));
+    f[i] = v.xy;
+    fz[i] = v.z;
   }
-  const V fxy = mul2(fma2(a2, v2(T(2), T(2)), a1), v2(T(1.0 / 12.0), T(1.0 / 12.0)));
-  F[0] = fxy.x;
-  F[1] = fxy.y;
-  T z2 = T(0), z1 = T(0);
 #pragma unroll
   for (int i = 1; i < 19; i += 2) {
-    const int cx = lat_c(i, 0), cy = lat_c(i, 1), cz = lat_c(i, 2);
-    const bool face = lat_c2(i) == 1;
-    if (cx || cy) {
-      const V D = sub2(acc.spair(3, cx, cy, cz), acc.spair(3, -cx, -cy, -cz));
-      if (cx) {
-        const T d = cx > 0 ? D.x : -D.x;
-        if (face) z2 += d; else z1 += d;
-      }
-      if (cy) {
-        const T d = cy > 0 ? D.y : -D.y;
-        if (face) z2 += d; else z1 += d;
-      }
-    }
-    if (cz) {
-      const T Dz = acc.spair(4, cx, cy, cz).x - acc.spair(4, -cx, -cy, -cz).x;
-      const T d = cz > 0 ? Dz : -Dz;
-      if (face) z2 += d; else z1 += d;
-    }
+    D[i] = sub2(f[i], f[i + 1]);
+    Dz[i] = sub2(fz[i], fz[i + 1]);
   }
-  F[2] = (T(2) * z2 + z1) * T(1.0 / 12.0);
+  grad_from_pairs(D, g);
+  grad_from_pairs(Dz, Wg[2]);
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    Wg[0][b] = g[b].x;
+    Wg[1][b] = g[b].y;
+  }
+  u0[0] = f[0].x;
+  u0[1] = f[0].y;
+  u0[2] = fz[0];
+  uf[0] = f[1].x;
+  uf[1] = f[2].x;
+  uf[2] = f[3].y;
+  uf[3] = f[4].y;
+  uf[4] = fz[5];
+  uf[5] = fz[6];
 }
 
-// The stencils of a4: lap mu, W_ab = d_b u_a, and the face values of Q, psi and u for the
-// upwind terms (face slot 2a: +e_a, 2a+1: -e_a).
+// Q at the upwind neighbours (side by the sign of u0 along each axis) as the field pairs of
+// A::pair, and psi at the six faces.
 template <typename T, class A>
-__device__ __forceinline__ void gather_op(const A& acc, T& lapmu, T Wg[3][3], T q0[5], T qf[6][5], T& p0, T pf[6],
-                                          T u0[3], T uf[6]) {
-  // lap mu (lane 1 of stress pair 4, so that the loads are shared with the force)
-  {
-    T d[19];
-    const T m0 = acc.spair(4, 0, 0, 0).y;
+__device__ __forceinline__ void gather_upwind(const A& acc, const T u0[3], Vec2<T> qu[3][3], T pf[6]) {
 #pragma unroll
-    for (int i = 1; i < 19; ++i) d[i] = acc.spair(4, lat_c(i, 0), lat_c(i, 1), lat_c(i, 2)).y - m0;
-    lapmu = lap_from_diffs(d);
-  }
-  // grad u and the axial face velocities: (u_x, u_y) as pairs, u_z alone
-  {
-    using V = Vec2<T>;
-    V f[19], D[19], g[3];
+  for (int a = 0; a < 3; ++a)
 #pragma unroll
-    for (int i = 0; i < 19; ++i) f[i] = acc.upair(lat_c(i, 0), lat_c(i, 1), lat_c(i, 2));
+    for (int j = 0; j < 3; ++j) qu[a][j] = acc.pair_upwind(j, a, u0[a] > T(0));
 #pragma unroll
-    for (int i = 1; i < 19; i += 2) D[i] = sub2(f[i], f[i + 1]);
-    grad2_from_pairs<T>(D, g);
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      Wg[0][b] = g[b].x;
-      Wg[1][b] = g[b].y;
-    }
-    u0[0] = f[0].x;
-    u0[1] = f[0].y;
-    uf[0] = f[1].x;
-    uf[1] = f[2].x;
-    uf[2] = f[3].y;
-    uf[3] = f[4].y;
-  }
-  {
-    T f[19], D[19];
-#pragma unroll
-    for (int i = 0; i < 19; ++i) f[i] = acc.u(2, lat_c(i, 0), lat_c(i, 1), lat_c(i, 2));
-#pragma unroll
-    for (int i = 1; i < 19; i += 2) D[i] = f[i] - f[i + 1];
-    grad_from_pairs(D, Wg[2]);
-    u0[2] = f[0];
-    uf[4] = f[5];
-    uf[5] = f[6];
-  }
-  // Q and psi at the centre and the six faces, as the field pairs (Q_xx, Q_xy), (Q_xz, Q_yy),
-  // (Q_yz, psi) of A::pair
-#pragma unroll
-  for (int i = 0; i < 7; ++i) {
-    const int cx = lat_c(i, 0), cy = lat_c(i, 1), cz = lat_c(i, 2);
-    T* qd = i ? qf[i - 1] : q0;
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const Vec2<T> v = acc.pair(j, cx, cy, cz);
-      qd[2 * j] = v.x;
-      if (j < 2) qd[2 * j + 1] = v.y;
-      else if (i) pf[i - 1] = v.y;
-      else p0 = v.y;
-    }
-  }
+  for (int i = 1; i < 7; ++i) pf[i - 1] = acc.psi(lat_c(i, 0), lat_c(i, 1), lat_c(i, 2));
 }
 
-// a3 + the stencils of a4, for the one-pass step.
+// The stencils of a4 at one site: lap mu, W_ab = d_b u_a, Q and psi at the centre, Q at the
+// upwind neighbours, psi and the axial velocities at the faces.
 template <typename T, class A>
-__device__ __forceinline__ void gather_update(const A& acc, T F[3], T& lapmu, T Wg[3][3], T q0[5], T qf[6][5],
-                                              T& p0, T pf[6], T u0[3], T uf[6]) {
-  gather_force<T>(acc, F);
-  gather_op<T>(acc, lapmu, Wg, q0, qf, p0, pf, u0, uf);
+__device__ __forceinline__ void gather_op(const A& acc, T& lapmu, T Wg[3][3], T q0[5], Vec2<T> qu[3][3], T& p0,
+                                          T pf[6], T u0[3], T uf[6]) {
+  lapmu = gather_lapmu<T>(acc);
+  gather_velocity<T>(acc, Wg, u0, uf);
+  gather_upwind<T>(acc, u0, qu, pf);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const Vec2<T> v = acc.pair(j, 0, 0, 0);
+    q0[2 * j] = v.x;
+    if (j < 2) q0[2 * j + 1] = v.y;
+    else p0 = v.y;
+  }
 }
 
-// a4 at one site: Beris-Edwards update of Q (Eq. 2) and Cahn-Hilliard update of psi
-// (Eq. 1) with the advecting velocity u0/uf (and its gradient Wg).  RHS = false gives the
-// Euler step Q + R(Q), RHS = true the right-hand side R(Q) alone (for the Heun stages).
-template <typename T, bool RHS>
-__device__ __forceinline__ void op_update(const Coef<T>& c, T lapmu, const T Wg[3][3], const T q0[5],
-                                          const T qf[6][5], T p0, const T pf[6], const T u0[3], const T uf[6],
-                                          const T Hs[5], T qn[5], T& pn) {
-  T adv[5] = {T(0), T(0), T(0), T(0), T(0)};
+// a4, psi: the divergence of the upwind flux of psi.
+template <typename T>
+__device__ __forceinline__ T flux_divergence(T p0, const T pf[6], const T u0[3], const T uf[6]) {
   T divJ = T(0);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const int ip = 2 * a, im = 2 * a + 1;
-    const T up = u0[a] > T(0) ? u0[a] : T(0);
-    const T um = u0[a] < T(0) ? u0[a] : T(0);
-#pragma unroll
-    for (int k = 0; k < 5; ++k) adv[k] += up * (q0[k] - qf[im][k]) + um * (qf[ip][k] - q0[k]);
-    const T ubp = T(0.5) * (u0[a] + uf[ip]);
-    const T Jp = ubp * (ubp > T(0) ? p0 : pf[ip]);
-    const T ubm = T(0.5) * (uf[im] + u0[a]);
-    const T Jm = ubm * (ubm > T(0) ? pf[im] : p0);
-    divJ += Jp - Jm;
+    const T ubp = mul_rn(T(0.5), add2(u0[a], uf[ip]));
+    const T ubm = mul_rn(T(0.5), add2(uf[im], u0[a]));
+    const T Jm = mul_rn(ubm, ubm > T(0) ? pf[im] : p0);
+    divJ = add2(divJ, fma2(ubp, ubp > T(0) ? p0 : pf[ip], -Jm));
   }
+  return divJ;
+}
+
+// a4, Q: the increment of Q in one step (Eq. 2): co-rotation, Gamma_Q H, and upwind advection
+// with the velocity u0.  up (q0 - q_-) + um (q_+ - q0) with up = max(u, 0), um = min(u, 0) is
+// |u| (q0 - q_upwind), so only the upwind neighbour qu[a] (field pairs) is read.
+template <typename T>
+__device__ __forceinline__ void q_increment(const Coef<T>& c, const T Wg[3][3], const T q0[5],
+                                            const Vec2<T> qu[3][3], const T u0[3], const T Hs[5], T inc[5]) {
+  using V = Vec2<T>;
+  V a01 = v2(T(0), T(0)), a23 = v2(T(0), T(0));
+  T a4 = T(0);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const T ua = fabs(u0[a]);
+    a01 = fma2(v2(ua, ua), sub2(v2(q0[0], q0[1]), qu[a][0]), a01);
+    a23 = fma2(v2(ua, ua), sub2(v2(q0[2], q0[3]), qu[a][1]), a23);
+    a4 = fma2(ua, sub2(q0[4], qu[a][2].x), a4);
+  }
+  const T adv[5] = {a01.x, a01.y, a23.x, a23.y, a4};
   T Q[3][3];
   full3(q0, Q);
   // co-rotation S = (xi D + Om)(Q + I/3) + (Q + I/3)(xi D - Om) - 2 xi tr(QW)(Q + I/3), with
   // D, Om the symmetric and antisymmetric parts of W.  With M = xi D + Om, (xi D - Om) = M^T, so
   // S = P + P^T - 2 xi tr(QW)(Q + I/3) for P = M (Q + I/3); it is projected to its traceless part
   // (its trace is 2 xi tr(D)/3).  M_ij = (xi + 1)/2 W_ij + (xi - 1)/2 W_ji.
-  const T mp = T(0.5) * (c.xi + T(1)), mm = T(0.5) * (c.xi - T(1));
   T M[3][3];
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int j = 0; j < 3; ++j) M[i][j] = mp * Wg[i][j] + mm * Wg[j][i];
+    for (int j = 0; j < 3; ++j) M[i][j] = T(0.5) * (c.xip * Wg[i][j] - c.xim * Wg[j][i]);
   T Qt[3][3];
 #pragma unroll
   for (int i = 0; i < 3; ++i)
@@ -523,12 +620,9 @@ __device__ __forceinline__ void op_update(const Coef<T>& c, T lapmu, const T Wg[
 #pragma unroll
     for (int j = 0; j < 3; ++j) trQW += Q[i][j] * Wg[j][i];
   const T trD = Wg[0][0] + Wg[1][1] + Wg[2][2];
-  const T cq = -T(2) * c.xi * trQW;
-  const T cdiag = -(T(2) * c.xi / T(9)) * trD;
+  const T cq = -c.xi2 * trQW;
+  const T cdiag = -c.xi29 * trD;
   auto P = [&](int i, int j) { return M[i][0] * Qt[0][j] + M[i][1] * Qt[1][j] + M[i][2] * Qt[2][j]; };
-  // The increments are summed first and added to Q and psi once: every addition at the
-  // magnitude of the field rounds to its storage resolution, and three of them per step
-  // (Q - adv, + S, + Gamma H) added half again to the error that FP32 storage alone causes.
   const int I5[5] = {0, 0, 0, 1, 1};
   const int J5[5] = {0, 1, 2, 1, 2};
 #pragma unroll
@@ -536,11 +630,62 @@ __device__ __forceinline__ void op_update(const Coef<T>& c, T lapmu, const T Wg[
     const int i = I5[k], j = J5[k];
     T S = (i == j ? T(2) * P(i, i) : P(i, j) + P(j, i)) + cq * Qt[i][j];
     if (i == j) S += cdiag;
-    const T inc = fma(c.gammaQ, Hs[k], S - adv[k]);
-    qn[k] = RHS ? inc : q0[k] + inc;
+    inc[k] = fma(c.gammaQ, Hs[k], S) - adv[k];
   }
-  const T pinc = fma(c.M, lapmu, -divJ);
+}
+
+// a4 at one site: Beris-Edwards update of Q (Eq. 2) and Cahn-Hilliard update of psi
+// (Eq. 1) with the advecting velocity u0/uf (and its gradient Wg).  RHS = false gives the
+// Euler step Q + R(Q), RHS = true the right-hand side R(Q) alone (for the Heun stages).
+// The increments are summed first and added to Q and psi once: every addition at the
+// magnitude of the field rounds to its storage resolution, and three of them per step
+// (Q - adv, + S, + Gamma H) added half again to the error that FP32 storage alone causes.
+template <typename T, bool RHS>
+__device__ __forceinline__ void op_update(const Coef<T>& c, T lapmu, const T Wg[3][3], const T q0[5],
+                                          const Vec2<T> qu[3][3], T p0, const T pf[6], const T u0[3], const T uf[6],
+                                          const T Hs[5], T qn[5], T& pn) {
+  T inc[5];
+  q_increment<T>(c, Wg, q0, qu, u0, Hs, inc);
+#pragma unroll
+  for (int k = 0; k < 5; ++k) qn[k] = RHS ? inc[k] : q0[k] + inc[k];
+  const T pinc = fma(c.M, lapmu, -flux_divergence(p0, pf, u0, uf));
   pn = RHS ? pinc : p0 + pinc;
+}
+
+// c_i . a of velocity i (components 0, +1, -1).
+template <typename T, class V>
+__device__ __forceinline__ T dot_c(int i, const T a[3]) {
+  T s = T(0);
+  bool first = true;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int ck = V::c(i, k);
+    if (ck == 0) continue;
+    s = first ? (ck > 0 ? a[k] : -a[k]) : (ck > 0 ? add2(s, a[k]) : sub2(s, a[k]));
+    first = false;
+  }
+  return s;
+}
+
+// New values of the velocity pair (i, i+1) of the collision below and, if `two`, of (i+2, i+3), whose weight is
+// the same (class k: 1 faces, 2 the others).
+template <typename T, class V>
+__device__ __forceinline__ void lb_pair_update(const Coef<T>& c, bool two, int i, int k, const T u[3], const T F[3],
+                                               T r45, T r3, T base, T uF, T g[V::Q]) {
+  using W = Vec2<T>;
+  const int j = two ? i + 2 : i;
+  const W cu{dot_c<T, V>(i, u), dot_c<T, V>(j, u)}, cF{dot_c<T, V>(i, F), dot_c<T, V>(j, F)};
+  auto b = [](T v) { return W{v, v}; };
+  const T rest = fma(c.omw[k], base, -mul_rn(c.gw3[k], uF));
+  const W X = fma2(b(mul_rn(c.omw[k], r45)), mul2(cu, cu), fma2(mul2(b(c.gw9[k]), cu), cF, b(rest)));
+  const W Y = fma2(b(mul_rn(c.omw[k], r3)), cu, mul2(b(c.gw3[k]), cF));
+  const W p = fma2(b(c.omc), W{g[i], g[j]}, add2(X, Y)), m = fma2(b(c.omc), W{g[i + 1], g[j + 1]}, sub2(X, Y));
+  g[i] = p.x;
+  g[i + 1] = m.x;
+  if (two) {
+    g[j] = p.y;
+    g[j + 1] = m.y;
+  }
 }
 
 // a5 at one site: moments of the pulled populations g and the force F, then BGK + Guo
@@ -581,26 +726,15 @@ __device__ __forceinline__ void lb_collide(const Coef<T>& c, const T F[3], T g[V
   // (9 cu cF - 3 uF) and the odd part Y = 3 om w rho cu + 3 guo w cF; their coefficients depend
   // on the weight class only, so each class forms them once.
   const T base = fma(T(-1.5) * rho, u2, SHIFT ? m0 : rho);
-  const T om = c.tau_inv;
-  const T omc = T(1) - om;
   const T r45 = T(4.5) * rho;
   const T r3 = T(3) * rho;
-  {
-    const T w = T(V::w(0));
-    g[0] = fma(omc, g[0], fma(om * w, base, (T(-3) * c.guo * w) * uF));
-  }
+  g[0] = fma(c.omc, g[0], fma(c.omw[0], base, -mul_rn(c.gw3[0], uF)));
+  // two velocity pairs of one weight class at a time, the first of each pair in one two-lane value and the
+  // opposite ones in another: the faces' pairs 1, 3 and 5, then the others
+  lb_pair_update<T, V>(c, true, 1, 1, u, F, r45, r3, base, uF, g);
+  lb_pair_update<T, V>(c, false, 5, 1, u, F, r45, r3, base, uF, g);
 #pragma unroll
-  for (int i = 1; i < V::Q; i += 2) {
-    const T w = T(V::w(i));
-    const T omw = om * w, gw = c.guo * w;
-    const T cu = T(V::c(i, 0)) * u[0] + T(V::c(i, 1)) * u[1] + T(V::c(i, 2)) * u[2];
-    const T cF = T(V::c(i, 0)) * F[0] + T(V::c(i, 1)) * F[1] + T(V::c(i, 2)) * F[2];
-    const T X = fma(omw * r45, cu * cu, fma(omw, base, fma((T(9) * gw) * cu, cF, (T(-3) * gw) * uF)));
-    const T Y = fma(omw * r3, cu, (T(3) * gw) * cF);
-    const T gp = g[i], gm = g[i + 1];
-    g[i] = fma(omc, gp, X + Y);
-    g[i + 1] = fma(omc, gm, X - Y);
-  }
+  for (int i = 7; i < V::Q; i += 4) lb_pair_update<T, V>(c, true, i, 2, u, F, r45, r3, base, uF, g);
 }
 
 // a5 in the form of Eqs. 9-11 at one site: the equilibrium carries the symmetric stress,
@@ -665,9 +799,9 @@ __device__ __forceinline__ void lb_collide_stress(const Coef<T>& c, const T FA[3
 // previous step, and the collision of the pulled populations.
 template <typename T, bool SHIFT>
 __device__ __forceinline__ void update_math(const Coef<T>& c, const T F[3], T lapmu, const T Wg[3][3],
-                                            const T q0[5], const T qf[6][5], T p0, const T pf[6], const T u0[3],
+                                            const T q0[5], const Vec2<T> qu[3][3], T p0, const T pf[6], const T u0[3],
                                             const T uf[6], const T Hs[5], T g[19], T qn[5], T& pn, T u[3]) {
-  op_update<T, false>(c, lapmu, Wg, q0, qf, p0, pf, u0, uf, Hs, qn, pn);
+  op_update<T, false>(c, lapmu, Wg, q0, qu, p0, pf, u0, uf, Hs, qn, pn);
   lb_collide<T, SHIFT>(c, F, g, u);
 }
 
@@ -691,14 +825,18 @@ struct GlobalAcc {
     const long long o = nb.off(cx, cy, cz);
     return Vec2<T>{ld(q_ + (2 * j) * N + o), j < 2 ? ld(q_ + (2 * j + 1) * N + o) : ld(ps + o)};
   }
-  // stress pair j (see sig_pair) and the velocity pair (u_x, u_y)
+  __device__ __forceinline__ Vec2<T> pair_upwind(int j, int a, bool from_below) const {
+    const int d = from_below ? -1 : 1;
+    return pair(j, a == 0 ? d : 0, a == 1 ? d : 0, a == 2 ? d : 0);
+  }
+  __device__ __forceinline__ Vel3<T> u3(int cx, int cy, int cz) const {
+    const long long o = nb.off(cx, cy, cz);
+    return Vel3<T>{Vec2<T>{ld(u_ + o), ld(u_ + N + o)}, ld(u_ + 2 * N + o)};
+  }
+  // stress pair j (see sig_pair)
   __device__ __forceinline__ Vec2<T> spair(int j, int cx, int cy, int cz) const {
     const long long o = nb.off(cx, cy, cz);
     return Vec2<T>{ld(sg + pair_c0(j) * N + o), j == 4 ? ld(mu_ + o) : ld(sg + pair_c1(j) * N + o)};
-  }
-  __device__ __forceinline__ Vec2<T> upair(int cx, int cy, int cz) const {
-    const long long o = nb.off(cx, cy, cz);
-    return Vec2<T>{ld(u_ + o), ld(u_ + N + o)};
   }
 };
 
@@ -795,7 +933,7 @@ __device__ __forceinline__ void gather_force_r2(const A& acc, T F[3]) {
 
 // The stencils of a4 with the radius-2 set; the upwind faces stay at distance 1.
 template <typename T, class A>
-__device__ __forceinline__ void gather_op_r2(const A& acc, T& lapmu, T Wg[3][3], T q0[5], T qf[6][5], T& p0,
+__device__ __forceinline__ void gather_op_r2(const A& acc, T& lapmu, T Wg[3][3], T q0[5], Vec2<T> qu[3][3], T& p0,
                                              T pf[6], T u0[3], T uf[6]) {
   {
     auto f = [&](int dx, int dy, int dz) { return acc.mu(dx, dy, dz); };
@@ -822,13 +960,7 @@ __device__ __forceinline__ void gather_op_r2(const A& acc, T& lapmu, T Wg[3][3],
     uf[2 * a] = f(a == 0, a == 1, a == 2);
     uf[2 * a + 1] = f(-(a == 0), -(a == 1), -(a == 2));
   }
-#pragma unroll
-  for (int i = 1; i < 7; ++i) {
-    const int cx = lat_c(i, 0), cy = lat_c(i, 1), cz = lat_c(i, 2);
-#pragma unroll
-    for (int k = 0; k < 5; ++k) qf[i - 1][k] = acc.q(k, cx, cy, cz);
-    pf[i - 1] = acc.psi(cx, cy, cz);
-  }
+  gather_upwind<T>(acc, u0, qu, pf);
 #pragma unroll
   for (int k = 0; k < 5; ++k) q0[k] = acc.q(k, 0, 0, 0);
   p0 = acc.psi(0, 0, 0);
@@ -964,21 +1096,22 @@ __global__ void __launch_bounds__(kStepBlock) k_op(const InstDesc<T>* __restrict
   acc.u_ = sync ? I.u_out : I.u_in;
   acc.N = N;
   acc.nb = make_nbr_st<ST>(x, y, z, nx, ny, nz);
-  T lapmu, Wg[3][3], q0[5], qf[6][5], p0, pf[6], u0[3], uf[6];
-  if constexpr (ST == 1) gather_op_r2<T>(acc, lapmu, Wg, q0, qf, p0, pf, u0, uf);
-  else gather_op<T>(acc, lapmu, Wg, q0, qf, p0, pf, u0, uf);
+  T lapmu, Wg[3][3], q0[5], p0, pf[6], u0[3], uf[6];
+  Vec2<T> qu[3][3];
+  if constexpr (ST == 1) gather_op_r2<T>(acc, lapmu, Wg, q0, qu, p0, pf, u0, uf);
+  else gather_op<T>(acc, lapmu, Wg, q0, qu, p0, pf, u0, uf);
   const T* Hsrc = STAGE == 2 ? I.sig : I.H;
   T Hs[5];
 #pragma unroll
   for (int k = 0; k < 5; ++k) Hs[k] = Hsrc[k * N + s];
   T qn[5], pn;
   if (STAGE == 0) {
-    op_update<T, false>(I.c, lapmu, Wg, q0, qf, p0, pf, u0, uf, Hs, qn, pn);
+    op_update<T, false>(I.c, lapmu, Wg, q0, qu, p0, pf, u0, uf, Hs, qn, pn);
 #pragma unroll
     for (int k = 0; k < 5; ++k) I.q_out[k * N + s] = qn[k];
     I.psi_out[s] = pn;
   } else if (STAGE == 1) {
-    op_update<T, true>(I.c, lapmu, Wg, q0, qf, p0, pf, u0, uf, Hs, qn, pn);
+    op_update<T, true>(I.c, lapmu, Wg, q0, qu, p0, pf, u0, uf, Hs, qn, pn);
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
       I.rq[k * N + s] = qn[k];
@@ -987,7 +1120,7 @@ __global__ void __launch_bounds__(kStepBlock) k_op(const InstDesc<T>* __restrict
     I.rq[5 * N + s] = pn;
     I.qp[5 * N + s] = p0 + pn;
   } else {
-    op_update<T, true>(I.c, lapmu, Wg, q0, qf, p0, pf, u0, uf, Hs, qn, pn);
+    op_update<T, true>(I.c, lapmu, Wg, q0, qu, p0, pf, u0, uf, Hs, qn, pn);
 #pragma unroll
     for (int k = 0; k < 5; ++k) I.q_out[k * N + s] = I.q_in[k * N + s] + T(0.5) * (I.rq[k * N + s] + qn[k]);
     I.psi_out[s] = I.psi_in[s] + T(0.5) * (I.rq[5 * N + s] + pn);
@@ -1015,8 +1148,10 @@ __global__ void __launch_bounds__(kStepBlock) k_update(const InstDesc<T>* __rest
   acc.u_ = I.u_in;
   acc.N = N;
   acc.nb = make_nbr(x, y, z, nx, ny, nz);
-  T F[3], lapmu, Wg[3][3], q0[5], qf[6][5], p0, pf[6], u0[3], uf[6];
-  gather_update<T>(acc, F, lapmu, Wg, q0, qf, p0, pf, u0, uf);
+  T F[3], lapmu, Wg[3][3], q0[5], p0, pf[6], u0[3], uf[6];
+  Vec2<T> qu[3][3];
+  gather_force<T>(acc, F);
+  gather_op<T>(acc, lapmu, Wg, q0, qu, p0, pf, u0, uf);
   T Hs[5];
 #pragma unroll
   for (int k = 0; k < 5; ++k) Hs[k] = I.H[k * N + s];
@@ -1024,7 +1159,7 @@ __global__ void __launch_bounds__(kStepBlock) k_update(const InstDesc<T>* __rest
 #pragma unroll
   for (int i = 0; i < 19; ++i) g[i] = ld(I.g_in + i * N + acc.nb.off(-lat_c(i, 0), -lat_c(i, 1), -lat_c(i, 2)));
   T qn[5], pn, u[3];
-  update_math<T, SHIFT>(I.c, F, lapmu, Wg, q0, qf, p0, pf, u0, uf, Hs, g, qn, pn, u);
+  update_math<T, SHIFT>(I.c, F, lapmu, Wg, q0, qu, p0, pf, u0, uf, Hs, g, qn, pn, u);
 #pragma unroll
   for (int k = 0; k < 5; ++k) I.q_out[k * N + s] = qn[k];
   I.psi_out[s] = pn;
@@ -1108,10 +1243,8 @@ __global__ void k_set_fields(InstDesc<T> I, long long oG, long long oU, long lon
 // and its exact rounding error, which c gathers: s + c carries about twice T's precision.  The
 // a6 sums of the FP32 path are formed this way, so they come out as the FP64 sums of the
 // per-site FP32 shares.
-// a * b rounded to T before any later use: the a6 shares are products that must come out as
-// the same T values in every pass, so they may not be contracted into a following addition.
-__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+// (The shares are products rounded by mul_rn: they must come out as the same T values in every
+// pass, so they may not be contracted into a following addition.)
 
 template <typename T>
 __device__ __forceinline__ void two_sum_add(T& s, T& c, T x) {

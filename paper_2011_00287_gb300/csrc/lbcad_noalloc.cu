@@ -13,6 +13,7 @@
 #include <string>
 
 #include "lbcad.h"
+#include "lbcad_coefs.h"
 #include "lbcad_internal.h"
 #include "lbcad_validate.h"
 
@@ -24,7 +25,7 @@ namespace {
 // until the process exits.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[LBCAD_NOALLOC_SCRATCH_BYTES];
 // The one-instance launch descriptor the step kernels read.
-static __device__ __align__(256) unsigned char g_noalloc_desc[512];
+static __device__ __align__(256) unsigned char g_noalloc_desc[1024];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_setup_mu;
@@ -75,12 +76,7 @@ InstDesc<T> one_desc(const lbcad_grid& g, const lbcad_params& p, const void* g_i
   d.sig = (T*)scratch;
   d.mu = (T*)(scratch + 9 * part);
   d.H = (T*)(scratch + 10 * part);
-  d.c.tau_inv = (T)(1.0 / p.tau);
-  d.c.guo = (T)(1.0 - 0.5 / p.tau);
-  d.c.rho0 = (T)p.rho0;
-  d.c.A0 = (T)p.A0; d.c.chi0 = (T)p.chi0; d.c.chis = (T)p.chis; d.c.K = (T)p.K; d.c.q0 = (T)p.q0;
-  d.c.gammaQ = (T)p.gammaQ; d.c.xi = (T)p.xi; d.c.a = (T)p.a; d.c.b = (T)p.b; d.c.kphi = (T)p.kphi;
-  d.c.M = (T)p.M; d.c.W = (T)p.W; d.c.zeta = (T)p.zeta;
+  d.c = coefs<T>(p);
   return d;
 }
 
@@ -94,7 +90,7 @@ __global__ void k_noalloc_set_desc(InstDesc<T> d) {
 template <typename T, bool SHIFT>
 int run(const lbcad_grid& g, const lbcad_params& p, const void* g_in, const void* q_in, const void* psi_in,
         const void* u_in, void* g_out, void* q_out, void* psi_out, void* u_out, void* scratch, void* desc_dev) {
-  static_assert(sizeof(InstDesc<T>) <= 512, "descriptor slot too small");
+  static_assert(sizeof(InstDesc<T>) <= sizeof(g_noalloc_desc), "descriptor slot too small");
   const InstDesc<T> d = one_desc<T>(g, p, g_in, q_in, psi_in, u_in, g_out, q_out, psi_out, u_out,
                                     (unsigned char*)scratch);
   cudaStream_t s = (cudaStream_t)p.stream;

@@ -9,9 +9,12 @@
 #include <algorithm>
 #include <new>
 #include <string>
+#include <type_traits>
+#include <utility>
 #include <vector>
 
 #include "lbcad.h"
+#include "lbcad_coefs.h"
 #include "lbcad_internal.h"
 #include "lbcad_validate.h"
 
@@ -29,6 +32,7 @@ struct Inst {
   void* qb[2] = {nullptr, nullptr};
   void* pb[2] = {nullptr, nullptr};
   void* ub[2] = {nullptr, nullptr};
+  void* S = nullptr;   // default path: stress, mu, flux divergence, psi (12 per site)
   void* sig = nullptr;
   void* mu = nullptr;
   void* H = nullptr;
@@ -80,22 +84,21 @@ struct lbcad_ctx {
   int lb_form = LBCAD_LB_BODY_FORCE;
   int stencil = LBCAD_STENCIL_ISO;
   bool scratch_ready = false;
-  FusedTile* tiles = nullptr;
-  size_t tiles_cap = 0;
-  int ntiles = 0;
-  long long fused_total = 0;
-  int fused_grid = 0;
+  MarchItem* items = nullptr;  // work items of the default path, all lists of all groups
+  size_t items_cap = 0;
+  std::vector<StepWork> work;  // one per group of instances
+  std::vector<FusedObs> obs;
+  std::vector<MarchDesc<float>> desc32[2];  // by step parity
+  std::vector<MarchDesc<double>> desc64[2];
   int cfg_index = 0;
-  FusedCfg cfg;
   // a6 sums of the fused step (see FusedObs): slots per (block, segment), per-instance
   // bookkeeping, and the sums of the latest state; obs_valid while they describe the state
   double* obs_slots = nullptr;
   size_t obs_slots_cap = 0;
-  int* obs_map = nullptr;  // slot_inst [nslots], then nslot, slot_lo, slot_hi [ninst each]
+  int* obs_map = nullptr;  // per group: slot_inst [nslots], then nslot, slot_lo, slot_hi [ninst each]
   size_t obs_map_cap = 0;
   unsigned* obs_cnt = nullptr;
   double* obs_latest = nullptr;
-  int obs_maxseg = 0;
   bool observe = true;     // fused steps form the a6 sums (lbcad_set_observe)
   bool obs_valid = false;
   void* adj_lam = nullptr;  // cotangent of the initial state of the last lbcad_adjoint
@@ -169,18 +172,6 @@ void release(lbcad_ctx* c) {
 }
 
 template <typename T>
-Coef<T> coefs(const lbcad_params& p) {
-  Coef<T> c;
-  c.tau_inv = (T)(1.0 / p.tau);
-  c.guo = (T)(1.0 - 0.5 / p.tau);
-  c.rho0 = (T)p.rho0;
-  c.A0 = (T)p.A0; c.chi0 = (T)p.chi0; c.chis = (T)p.chis; c.K = (T)p.K; c.q0 = (T)p.q0;
-  c.gammaQ = (T)p.gammaQ; c.xi = (T)p.xi; c.a = (T)p.a; c.b = (T)p.b; c.kphi = (T)p.kphi;
-  c.M = (T)p.M; c.W = (T)p.W; c.zeta = (T)p.zeta;
-  return c;
-}
-
-template <typename T>
 InstDesc<T> make_desc(const Inst& I, int parity) {
   InstDesc<T> d;
   std::memset(&d, 0, sizeof(d));
@@ -197,6 +188,36 @@ InstDesc<T> make_desc(const Inst& I, int parity) {
   d.sig = (T*)I.sig; d.mu = (T*)I.mu; d.H = (T*)I.H;
   d.rq = (T*)I.rq; d.qp = (T*)I.qp;
   d.trig = (const T*)I.trig;
+  d.c = coefs<T>(I.p);
+  return d;
+}
+
+template <typename T>
+MarchDesc<T> make_march_desc(const Inst& I, int parity, bool shifted) {
+  MarchDesc<T> d;
+  std::memset(&d, 0, sizeof(d));
+  d.nx = I.g.nx; d.ny = I.g.ny; d.nz = I.g.nz;
+  d.plane = (unsigned)((long long)I.g.nx * I.g.ny);
+  const long long N = I.N;
+  const int a = parity, b = parity ^ 1, q = (I.p.lattice == LBCAD_D3Q15) ? 15 : 19;
+  auto comps = [&](auto* dst, void* base, int n, long long stride) {
+    for (int k = 0; k < n; ++k) dst[k] = base ? (T*)base + k * stride : nullptr;
+  };
+  comps(d.g_in, I.gb[a], q, N);
+  comps(d.g_out, I.gb[b], q, N);
+  comps(d.q_in, I.qb[a], 5, N);
+  comps(d.q_out, I.qb[b], 5, N);
+  d.psi_in = (const T*)I.pb[a];
+  d.psi_out = (T*)I.pb[b];
+  comps(d.u_in, I.ub[a], 3, N);
+  comps(d.u_out, I.ub[b], 3, N);
+  comps(d.S, I.S, 3, 4 * N);
+  comps(d.H, I.H, 5, N);
+  comps(d.rq, I.rq, 6, N);
+  comps(d.qp, I.qp, 6, N);
+  comps(d.Hp, I.sig, 6, N);
+  d.trig = (const T*)I.trig;
+  d.mass0 = shifted ? (double)(T)I.p.rho0 * (double)N : 0.0;
   d.c = coefs<T>(I.p);
   return d;
 }
@@ -274,7 +295,7 @@ int upload_init(lbcad_ctx* c, Inst& I, uint64_t seed, int idx) {
 int upload_descs(lbcad_ctx* c);
 int prepare_fused(lbcad_ctx* c, int cfg_index);
 int ensure_scratch(lbcad_ctx* c);
-cudaError_t launch_fused_lb(lbcad_ctx* c, int par);
+int default_shape(const lbcad_ctx* c);
 
 int create_impl(int n, const lbcad_grid* grids, const lbcad_params* params, uint64_t seed, lbcad_ctx** out) {
   g_create_err.clear();
@@ -369,6 +390,11 @@ int create_impl(int n, const lbcad_grid* grids, const lbcad_params* params, uint
     if (te == cudaSuccess) te = cudaStreamSynchronize(c->stream);
     if (te != cudaSuccess) return bail(LBCAD_E_CUDA, std::string("trig table upload: ") + cudaGetErrorString(te));
   }
+  if (!c->staged_only())
+    for (Inst& I : c->inst) {
+      I.S = dev_alloc(c, 12 * I.N * es);
+      if (!I.S) return bail(LBCAD_E_OOM, "device allocation failed");
+    }
   c->obs_cnt = (unsigned*)dev_alloc(c, n * sizeof(unsigned));
   c->obs_latest = (double*)dev_alloc(c, (size_t)n * 12 * sizeof(double));
   if (!c->obs_cnt || !c->obs_latest) return bail(LBCAD_E_OOM, "device allocation failed");
@@ -386,11 +412,7 @@ int create_impl(int n, const lbcad_grid* grids, const lbcad_params* params, uint
   c->obs_out = (double*)dev_alloc(c, 12 * sizeof(double));
   if (!c->obs_partial || !c->obs_out) return bail(LBCAD_E_OOM, "device allocation failed");
   if (upload_descs(c) != LBCAD_OK) return bail(LBCAD_E_CUDA, "");
-  // default tile shape: the pipelined 32x8 schedule in FP32 (the fastest candidate from 16^3 to
-  // 128^3; the one sync coupling and Heun run on), 32x8 in FP64 (the only one)
-  const int cfg0 = c->prec == LBCAD_FP64 ? LaunchFused<double, false>::sync_config()
-                                         : LaunchFused<float, true>::sync_config();
-  if ((code = prepare_fused(c, cfg0)) != LBCAD_OK) return bail(code, "");
+  if ((code = prepare_fused(c, default_shape(c))) != LBCAD_OK) return bail(code, "");
   if (c->staged_only() || c->sync_split()) {
     if ((code = ensure_scratch(c)) != LBCAD_OK) return bail(code, "");
   }
@@ -407,6 +429,12 @@ int create_impl(int n, const lbcad_grid* grids, const lbcad_params* params, uint
 int upload_descs(lbcad_ctx* c) {
   const int n = (int)c->inst.size();
   for (int par = 0; par < 2; ++par) {
+    c->desc32[par].clear();
+    c->desc64[par].clear();
+    for (const Inst& I : c->inst) {
+      if (c->prec == LBCAD_FP64) c->desc64[par].push_back(make_march_desc<double>(I, par, false));
+      else c->desc32[par].push_back(make_march_desc<float>(I, par, true));
+    }
     if (c->prec == LBCAD_FP64) {
       std::vector<InstDesc<double>> h(n);
       for (int i = 0; i < n; ++i) h[i] = make_desc<double>(c->inst[i], par);
@@ -442,71 +470,147 @@ int ensure_scratch(lbcad_ctx* c) {
   return upload_descs(c);
 }
 
-// Tile columns of the fused step for tile shape `cfg_index` and its persistent grid size.
+// Tile shape of a new context: candidate 0 (rows of 32 sites) or 3 (rows of 16), whichever covers the boxes
+// with fewer sites beyond their edges; 0, with its longer rows, when they tie.
+int default_shape(const lbcad_ctx* c) {
+  if (c->prec == LBCAD_FP64) return 0;
+  long long wide = 0, square = 0;
+  for (const Inst& I : c->inst) {
+    wide += (long long)((I.g.nx + 31) / 32 * 32) * ((I.g.ny + 7) / 8 * 8) * I.g.nz;
+    square += (long long)((I.g.nx + 15) / 16 * 16) * ((I.g.ny + 15) / 16 * 16) * I.g.nz;
+  }
+  return square < wide ? 3 : 0;
+}
+
+// Largest step (sites) whose kernels are launched with programmatic dependent launch.
+constexpr long long kEarlySites = 1 << 20;
+
+// The items of a group of instances for tx x ty tiles and at most `blocks` resident blocks, appended to `out`.
+// Each box is cut into slabs of about `len` planes; blocks take items in turn, so the slowest block works
+// through ceil(items / blocks) of them, each its planes plus what an item costs besides (two more planes
+// to load, most of a plane's time).  The length is the one with the shortest such time, up to 16
+// planes: neighbouring columns then stay close enough in z to find their halos in L2.
+MarchWork add_items(const lbcad_ctx* c, const StepWork& g, int tx, int ty, int blocks, std::vector<MarchItem>& out) {
+  constexpr double kItemPlanes = 0.8;
+  auto columns = [&](const lbcad_grid& b) { return (long long)((b.nx + tx - 1) / tx) * ((b.ny + ty - 1) / ty); };
+  int best = 1;
+  double best_time = 0.0;
+  for (int len = 1; len <= 16; ++len) {
+    long long n = 0;
+    for (int i = 0; i < g.ninst; ++i) {
+      const lbcad_grid& b = c->inst[g.first + i].g;
+      n += columns(b) * ((b.nz + len - 1) / len);
+    }
+    const double t = (double)((n + blocks - 1) / blocks) * (len + kItemPlanes);
+    if (len == 1 || t < best_time) {
+      best = len;
+      best_time = t;
+    }
+  }
+  MarchWork w;
+  const size_t first = out.size();
+  long long sites = 0;
+  for (int i = 0; i < g.ninst; ++i) {
+    const lbcad_grid& b = c->inst[g.first + i].g;
+    sites += c->inst[g.first + i].N;
+    const int slabs = (b.nz + best - 1) / best;
+    for (int k = 0; k < slabs; ++k) {
+      const int zb = (int)((long long)b.nz * k / slabs), ze = (int)((long long)b.nz * (k + 1) / slabs);
+      for (int y0 = 0; y0 < b.ny; y0 += ty)
+        for (int x0 = 0; x0 < b.nx; x0 += tx) out.push_back(MarchItem{i, x0, y0, zb, ze});
+    }
+  }
+  w.items = (const MarchItem*)(first * sizeof(MarchItem));  // offset; the list's address is added when it is uploaded
+  w.nitems = (int)(out.size() - first);
+  w.grid = w.nitems < blocks ? w.nitems : blocks;
+  // dependent launch hides a kernel's start-up (32^3: 17.4 us a step with it, 21.5 without; 64^3: 36.0 and 43.2),
+  // but blocks that start early disturb the even spread of a large step's blocks (128^3: 212 and 206 us,
+  // 256^3: 1508 and 1430)
+  w.early = sites <= kEarlySites;
+  return w;
+}
+
+// Work items of the default path for tile shape `cfg_index`, and the slots of its a6 sums.
 int prepare_fused(lbcad_ctx* c, int cfg_index) {
   FusedCfg cfg;
   const int v = c->fused_variant();
-  cudaError_t e = (c->prec == LBCAD_FP64) ? LaunchFused<double, false>::prepare(v, cfg_index, &cfg)
-                                          : LaunchFused<float, true>::prepare(v, cfg_index, &cfg);
+  const bool split = c->sync_split(), heun = c->integrator == LBCAD_HEUN, many = c->inst.size() > 1;
+  cudaError_t e = (c->prec == LBCAD_FP64) ? LaunchFused<double, false>::prepare(v, cfg_index, many, split, heun, &cfg)
+                                          : LaunchFused<float, true>::prepare(v, cfg_index, many, split, heun, &cfg);
   if (e == cudaErrorNotSupported)
     return fail(c, LBCAD_E_UNSUPPORTED, "this velocity set and LB form do not come in that tile shape");
   if (e != cudaSuccess) return fail(c, LBCAD_E_CUDA, std::string("fused kernel set-up: ") + cudaGetErrorString(e));
-  if (cfg.blocks_per_sm < 1) return fail(c, LBCAD_E_UNSUPPORTED, "fused tile shape does not fit on an SM");
-  std::vector<FusedTile> t;
-  long long start = 0;
-  for (int i = 0; i < (int)c->inst.size(); ++i) {
-    const Inst& I = c->inst[i];
-    for (int y0 = 0; y0 < I.g.ny; y0 += cfg.ty)
-      for (int x0 = 0; x0 < I.g.nx; x0 += cfg.tx) {
-        t.push_back(FusedTile{i, x0, y0, I.g.nz, start});
-        start += I.g.nz;
-      }
-  }
-  if (t.size() > c->tiles_cap) {
-    c->tiles = (FusedTile*)dev_alloc(c, t.size() * sizeof(FusedTile));
-    if (!c->tiles) return fail(c, LBCAD_E_OOM, "tile list allocation failed");
-    c->tiles_cap = t.size();
-  }
-  CK(c, cudaMemcpyAsync(c->tiles, t.data(), t.size() * sizeof(FusedTile), cudaMemcpyHostToDevice, c->stream));
-  CK(c, cudaStreamSynchronize(c->stream));
+  if (cfg.fields_per_sm < 1 || cfg.lb_per_sm < 1)
+    return fail(c, LBCAD_E_UNSUPPORTED, "fused tile shape does not fit on an SM");
   int sms = 0;
   CK(c, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
-  long long grid = (long long)sms * cfg.blocks_per_sm;
-  if (grid > start) grid = start;
-  // the column segments of each block, split exactly as the kernels split them: slot
-  // (block, segment) -> instance, and each instance's slot count and range
-  const int ninst = (int)c->inst.size();
-  std::vector<std::vector<int>> seg_inst(grid);
-  int maxseg = 1;
-  for (long long b = 0; b < grid; ++b) {
-    const long long begin = (start * b) / grid, end = (start * (b + 1)) / grid;
-    for (long long it = begin; it < end;) {
-      int lo = 0, hi = (int)t.size() - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (t[mid].start <= it) lo = mid; else hi = mid - 1;
-      }
-      const long long seg_end = std::min(end, t[lo].start + t[lo].nz);
-      seg_inst[b].push_back(t[lo].inst);
-      it = seg_end;
+  auto blocks = [&](int per_sm) { return sms * (per_sm > 0 ? per_sm : 1); };
+  std::vector<MarchItem> t;
+  std::vector<StepWork> work;
+  for (int first = 0; first < (int)c->inst.size(); first += kPackMany) {
+    StepWork g;
+    g.first = first;
+    g.ninst = std::min((int)c->inst.size() - first, kPackMany);
+    // a group of several instances launches the kernels prepared for several; a lone last one would not
+    if (many && g.ninst == 1) {
+      work.back().ninst -= 1;
+      g.first -= 1;
+      g.ninst = 2;
     }
-    maxseg = std::max(maxseg, (int)seg_inst[b].size());
+    work.push_back(g);
   }
-  const size_t nslots = (size_t)grid * maxseg;
-  std::vector<int> map(nslots + 3 * (size_t)ninst, -1);
-  int* nslot = map.data() + nslots;
-  int* slot_lo = nslot + ninst;
-  int* slot_hi = slot_lo + ninst;
-  for (int i = 0; i < ninst; ++i) nslot[i] = 0;
-  for (long long b = 0; b < grid; ++b)
-    for (size_t j = 0; j < seg_inst[b].size(); ++j) {
-      const int sl = (int)(b * maxseg + j), i = seg_inst[b][j];
-      map[sl] = i;
-      if (nslot[i]++ == 0) slot_lo[i] = sl;
-      slot_hi[i] = sl + 1;
+  for (StepWork& g : work) {
+    g.fields = add_items(c, g, cfg.fx, cfg.fy, blocks(cfg.fields_per_sm), t);
+    g.lb = add_items(c, g, cfg.lx, cfg.ly, blocks(cfg.lb_per_sm), t);
+    if (split) {
+      g.op[0] = add_items(c, g, cfg.lx, cfg.ly, blocks(cfg.op_per_sm[0]), t);
+      if (heun) {
+        g.pred = add_items(c, g, cfg.fx, cfg.fy, blocks(cfg.pred_per_sm), t);
+        g.op[1] = add_items(c, g, cfg.lx, cfg.ly, blocks(cfg.op_per_sm[1]), t);
+      }
     }
-  for (int i = 0; i < ninst; ++i)
-    if (nslot[i] == 0) return fail(c, LBCAD_E_INVALID_ARG, "an instance has no fused work");
+  }
+  // the runs of each block, as k_march_lb forms them: slot (block, run) -> instance, and each instance's slot
+  // count and range
+  std::vector<int> map;
+  std::vector<FusedObs> obs;
+  size_t nslots = 0;
+  for (const StepWork& g : work) {
+    const MarchItem* items = t.data() + (size_t)g.lb.items / sizeof(MarchItem);
+    const int grid = g.lb.grid;
+    std::vector<std::vector<int>> runs(grid);
+    size_t maxrun = 1;
+    for (int b = 0; b < grid; ++b) {
+      for (int i = b; i < g.lb.nitems; i += grid)
+        if (runs[b].empty() || runs[b].back() != items[i].inst) runs[b].push_back(items[i].inst);
+      maxrun = std::max(maxrun, runs[b].size());
+    }
+    const size_t at = map.size(), n = (size_t)grid * maxrun;
+    map.resize(at + n + 3 * (size_t)g.ninst, -1);
+    int* nslot = map.data() + at + n;
+    int* slot_lo = nslot + g.ninst;
+    int* slot_hi = slot_lo + g.ninst;
+    for (int i = 0; i < g.ninst; ++i) nslot[i] = 0;
+    for (int b = 0; b < grid; ++b)
+      for (size_t j = 0; j < runs[b].size(); ++j) {
+        const int sl = (int)(b * maxrun + j), i = runs[b][j];
+        map[at + sl] = i;
+        if (nslot[i]++ == 0) slot_lo[i] = sl;
+        slot_hi[i] = sl + 1;
+      }
+    FusedObs ob{};
+    ob.slots = (double*)(nslots * 12 * sizeof(double));  // offsets; the arrays' addresses are added below
+    ob.slot_inst = (const int*)(at * sizeof(int));
+    ob.nslot = (const int*)((at + n) * sizeof(int));
+    ob.maxrun = (int)maxrun;
+    obs.push_back(ob);
+    nslots += n;
+  }
+  if (t.size() > c->items_cap) {
+    c->items = (MarchItem*)dev_alloc(c, t.size() * sizeof(MarchItem));
+    if (!c->items) return fail(c, LBCAD_E_OOM, "work list allocation failed");
+    c->items_cap = t.size();
+  }
   if (nslots * 12 > c->obs_slots_cap) {
     c->obs_slots = (double*)dev_alloc(c, nslots * 12 * sizeof(double));
     if (!c->obs_slots) return fail(c, LBCAD_E_OOM, "a6 slot allocation failed");
@@ -517,49 +621,47 @@ int prepare_fused(lbcad_ctx* c, int cfg_index) {
     if (!c->obs_map) return fail(c, LBCAD_E_OOM, "a6 slot map allocation failed");
     c->obs_map_cap = map.size();
   }
+  auto place = [](auto*& p, void* base) { p = (std::remove_reference_t<decltype(p)>)((char*)base + (size_t)p); };
+  for (size_t i = 0; i < work.size(); ++i) {
+    StepWork& g = work[i];
+    for (MarchWork* w : {&g.fields, &g.lb, &g.op[0], &g.pred, &g.op[1]}) place(w->items, c->items);
+    FusedObs& ob = obs[i];
+    place(ob.slots, c->obs_slots);
+    place(ob.slot_inst, c->obs_map);
+    place(ob.nslot, c->obs_map);
+    ob.slot_lo = ob.nslot + g.ninst;
+    ob.slot_hi = ob.slot_lo + g.ninst;
+    ob.cnt = c->obs_cnt + g.first;
+    ob.latest = c->obs_latest + 12 * (size_t)g.first;
+  }
+  CK(c, cudaMemcpyAsync(c->items, t.data(), t.size() * sizeof(MarchItem), cudaMemcpyHostToDevice, c->stream));
   CK(c, cudaMemcpyAsync(c->obs_map, map.data(), map.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   // the kernels leave the per-instance counters at zero; reset them here as well, so that a
   // launch that failed part-way cannot shift the next sums
-  CK(c, cudaMemsetAsync(c->obs_cnt, 0, (size_t)ninst * sizeof(unsigned), c->stream));
+  CK(c, cudaMemsetAsync(c->obs_cnt, 0, c->inst.size() * sizeof(unsigned), c->stream));
   CK(c, cudaStreamSynchronize(c->stream));
-  c->obs_maxseg = maxseg;
+  c->work = std::move(work);
+  c->obs = std::move(obs);
   c->obs_valid = false;
-  c->ntiles = (int)t.size();
-  c->fused_total = start;
-  c->fused_grid = (int)grid;
   c->cfg_index = cfg_index;
-  c->cfg = cfg;
   return LBCAD_OK;
 }
 
 cudaError_t launch_fused(lbcad_ctx* c, int par) {
   const int v = c->fused_variant();
-  const int ninst = (int)c->inst.size();
-  const size_t nslots = (size_t)c->fused_grid * c->obs_maxseg;
-  FusedObs ob;
-  ob.slots = c->obs_slots;
-  ob.slot_inst = c->obs_map;
-  ob.nslot = c->obs_map + nslots;
-  ob.slot_lo = ob.nslot + ninst;
-  ob.slot_hi = ob.slot_lo + ninst;
-  ob.cnt = c->obs_cnt;
-  ob.latest = c->obs_latest;
-  ob.maxseg = c->obs_maxseg;
-  if (c->prec == LBCAD_FP64)
-    return LaunchFused<double, false>::step(v, c->cfg_index, (const InstDesc<double>*)c->desc[par], c->tiles,
-                                            c->ntiles, c->fused_total, c->fused_grid, ob, c->observe, c->stream);
-  return LaunchFused<float, true>::step(v, c->cfg_index, (const InstDesc<float>*)c->desc[par], c->tiles, c->ntiles,
-                                        c->fused_total, c->fused_grid, ob, c->observe, c->stream);
-}
-
-cudaError_t launch_fused_lb(lbcad_ctx* c, int par) {
-  const int v = c->fused_variant();
-  FusedObs ob{};  // the LB half forms no sums
-  if (c->prec == LBCAD_FP64)
-    return LaunchFused<double, false>::step_lb(v, (const InstDesc<double>*)c->desc[par], c->tiles, c->ntiles,
-                                               c->fused_total, c->fused_grid, ob, c->stream);
-  return LaunchFused<float, true>::step_lb(v, (const InstDesc<float>*)c->desc[par], c->tiles, c->ntiles,
-                                           c->fused_total, c->fused_grid, ob, c->stream);
+  const bool split = c->sync_split(), heun = c->integrator == LBCAD_HEUN, sync = c->coupling == LBCAD_SYNC;
+  auto run = [&](auto launch, const auto& d) {
+    using L = decltype(launch);
+    cudaError_t e = cudaSuccess;
+    for (size_t i = 0; i < c->work.size() && e == cudaSuccess; ++i) {
+      const StepWork& g = c->work[i];
+      e = split ? L::split_step(v, c->cfg_index, g, heun, sync, d.data() + g.first, c->stream)
+                : L::step(v, c->cfg_index, g, d.data() + g.first, c->obs[i], c->observe, c->stream);
+    }
+    return e;
+  };
+  return c->prec == LBCAD_FP64 ? run(LaunchFused<double, false>{}, c->desc64[par])
+                               : run(LaunchFused<float, true>{}, c->desc32[par]);
 }
 
 void drop_graph(lbcad_ctx* c) {
@@ -572,17 +674,7 @@ int launch_steps(lbcad_ctx* c, int64_t n) {
     const int par = (int)(c->step & 1);
     cudaError_t e;
     const bool heun = c->integrator == LBCAD_HEUN, sync = c->coupling == LBCAD_SYNC;
-    if (c->path == LBCAD_PATH_FUSED && c->sync_split()) {
-      // the LB half in the fused kernel, then the order-parameter half as tiled kernels on the
-      // same tiles (Euler: the update; Heun: predictor, fields at the predicted state, corrector)
-      e = launch_fused_lb(c, par);
-      if (e == cudaSuccess)
-        e = (c->prec == LBCAD_FP64)
-                ? LaunchFused<double, false>::op_tiled(heun, sync, (const InstDesc<double>*)c->desc[par], c->tiles,
-                                                       c->ntiles, c->fused_total, c->stream)
-                : LaunchFused<float, true>::op_tiled(heun, sync, (const InstDesc<float>*)c->desc[par], c->tiles,
-                                                     c->ntiles, c->fused_total, c->stream);
-    } else if (c->path == LBCAD_PATH_FUSED) {
+    if (c->path == LBCAD_PATH_FUSED) {
       e = launch_fused(c, par);
     } else if (c->path == LBCAD_PATH_STAGED) {
       e = (c->prec == LBCAD_FP64)
@@ -949,13 +1041,26 @@ StateBuf<T> state_at(T* base, long long N) {
   return StateBuf<T>{base, base + 19 * N, base + 24 * N, base + 25 * N};
 }
 
+// Descriptor of one replayed step: from state `in` to `out`, S and H of `in` at `f` (12 and 5 values per site).
 template <typename T>
-InstDesc<T> desc_for(const Inst& I, const StateBuf<T>& in, const StateBuf<T>& out, T* sig, T* mu, T* H) {
-  InstDesc<T> d = make_desc<T>(I, 0);
-  d.blk0 = 0;
-  d.g_in = in.g; d.q_in = in.q; d.psi_in = in.p; d.u_in = in.u;
-  d.g_out = out.g; d.q_out = out.q; d.psi_out = out.p; d.u_out = out.u;
-  d.sig = sig; d.mu = mu; d.H = H;
+MarchDesc<T> replay_desc(const MarchDesc<T>& base, long long N, const StateBuf<T>& in, const StateBuf<T>& out, T* f) {
+  MarchDesc<T> d = base;
+  for (int i = 0; i < 19; ++i) {
+    d.g_in[i] = in.g + i * N;
+    d.g_out[i] = out.g + i * N;
+  }
+  for (int k = 0; k < 5; ++k) {
+    d.q_in[k] = in.q + k * N;
+    d.q_out[k] = out.q + k * N;
+    d.H[k] = f + (12 + k) * N;
+  }
+  for (int a = 0; a < 3; ++a) {
+    d.u_in[a] = in.u + a * N;
+    d.u_out[a] = out.u + a * N;
+    d.S[a] = f + 4 * a * N;
+  }
+  d.psi_in = in.p;
+  d.psi_out = out.p;
   return d;
 }
 
@@ -975,7 +1080,7 @@ int adjoint_impl(lbcad_ctx* c, int64_t nsteps, int k, double* dzeta, double* dq0
   const long long N = I.N;
   const int S = (int)((nsteps + k - 1) / k);
   const size_t st = 28 * (size_t)N;  // elements of one stored state
-  const size_t fs = 15 * (size_t)N;  // elements of one state's sigma (9), mu, H (5)
+  const size_t fs = 17 * (size_t)N;  // elements of one state's stress quads (12) and H (5)
   // buffers through the context's allocator, kept for the next call
   c->adj_lam = nullptr;
   T* ck = (T*)adj_buffer(c, 0, (size_t)S * st * sizeof(T));
@@ -985,13 +1090,15 @@ int adjoint_impl(lbcad_ctx* c, int64_t nsteps, int k, double* dzeta, double* dq0
   T* fl = (T*)adj_buffer(c, 4, (size_t)k * fs * sizeof(T));
   const int nb = LaunchAdj<T, SHIFT>::blocks(N);
   double* pg = (double*)adj_buffer(c, 5, (2 * (size_t)nb + 2) * sizeof(double));
-  InstDesc<T>* dd = (InstDesc<T>*)adj_buffer(c, 6, (size_t)k * sizeof(InstDesc<T>));
-  if (!ck || !seg || !lam || !work || !fl || !pg || !dd) return fail(c, LBCAD_E_OOM, "adjoint buffers");
+  if (!ck || !seg || !lam || !work || !fl || !pg) return fail(c, LBCAD_E_OOM, "adjoint buffers");
   T* A = work;
   T* Bf = A + 88 * N;
   T* ls = Bf + 36 * N;
   double* total = pg + 2 * nb;
   CK(c, cudaMemsetAsync(total, 0, 2 * sizeof(double), c->stream));
+  using Step = LaunchFused<T, SHIFT>;
+  CK(c, Step::prepare_replay(c->cfg_index));
+  const MarchDesc<T> base = make_march_desc<T>(I, 0, SHIFT);
 
   lbcad_obs o0, o1;
   int r = lbcad_observables(c, 0, &o0);
@@ -1031,33 +1138,31 @@ int adjoint_impl(lbcad_ctx* c, int64_t nsteps, int k, double* dzeta, double* dq0
   cudaError_t e = LaunchAdj<T, SHIFT>::seed(desc_now<T>(c, 0), dX, ks, kc, lcur.p, c->stream);
   if (e != cudaSuccess) return fail(c, LBCAD_E_CUDA, std::string("adjoint seed: ") + cudaGetErrorString(e));
 
-  std::vector<InstDesc<T>> hd(k);
+  std::vector<InstDesc<T>> hd(k);  // state j of the segment and its H
   for (int sgi = S - 1; sgi >= 0; --sgi) {
     const int len = (int)std::min<int64_t>(k, nsteps - (int64_t)sgi * k);
-    // replay the segment: states 0 .. len-1 of this segment into seg (state 0 = checkpoint)
+    // replay the segment: states 0 .. len-1 of this segment into seg (state 0 = checkpoint), by the kernels of
+    // the step, so that the replayed states are the forward's
     CK(c, cudaMemcpyAsync(seg, ck + (size_t)sgi * st, st * sizeof(T), cudaMemcpyDeviceToDevice, c->stream));
-    // state j's sigma, mu, H go to its own slice of fl: the replay step that leaves state j
+    // state j's stress, mu and H go to its own slice of fl: the replay step that leaves state j
     // computes them, and its reverse step reads them there
     for (int j = 0; j < len; ++j) {
+      const bool last = j + 1 == len;
       const StateBuf<T> in = state_at<T>(seg + (size_t)j * st, N);
-      const StateBuf<T> out = state_at<T>(seg + (size_t)(j + 1 < len ? j + 1 : j) * st, N);
+      const StateBuf<T> out = state_at<T>(seg + (size_t)(last ? j : j + 1) * st, N);
       T* f = fl + (size_t)j * fs;
-      hd[j] = desc_for<T>(I, in, out, f, f + 9 * N, f + 10 * N);
-    }
-    CK(c, cudaMemcpyAsync(dd, hd.data(), len * sizeof(InstDesc<T>), cudaMemcpyHostToDevice, c->stream));
-    const long long blocks = (N + kStepBlock - 1) / kStepBlock;
-    for (int j = 0; j + 1 < len; ++j) {
-      e = Launch<T, SHIFT>::step(dd + j, 1, blocks, kStepBlock, c->stream);
+      hd[j] = make_desc<T>(I, 0);
+      hd[j].g_in = in.g; hd[j].q_in = in.q; hd[j].psi_in = in.p; hd[j].u_in = in.u;
+      hd[j].H = f + 12 * N;
+      const MarchDesc<T> md = replay_desc<T>(base, N, in, out, f);
+      e = Step::replay(c->cfg_index, c->work[0], last, &md, c->stream);
       if (e != cudaSuccess) return fail(c, LBCAD_E_CUDA, std::string("adjoint replay: ") + cudaGetErrorString(e));
     }
     // reverse steps
     for (int j = len - 1; j >= 0; --j) {
-      if (j == len - 1) {  // the segment's last state was not stepped from in the replay
-        e = Launch<T, SHIFT>::fields(dd + j, 1, blocks, kStepBlock, c->stream);
-        if (e != cudaSuccess) return fail(c, LBCAD_E_CUDA, std::string("adjoint fields: ") + cudaGetErrorString(e));
-      }
       AdjDescHost<T> h;
       h.I = hd[j];
+      h.S = fl + (size_t)j * fs;
       h.lg = lcur.g; h.lq = lcur.q; h.lp = lcur.p; h.lu = lcur.u;
       h.A = A; h.Bf = Bf; h.ls = ls;
       h.og = lnxt.g; h.oq = lnxt.q; h.op = lnxt.p; h.ou = lnxt.u;
