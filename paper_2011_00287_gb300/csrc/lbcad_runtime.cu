@@ -488,22 +488,25 @@ constexpr long long kEarlySites = 1 << 20;
 // The items of a group of instances for tx x ty tiles and at most `blocks` resident blocks, appended to `out`.
 // Each box is cut into slabs of about `len` planes; blocks take items in turn, so the slowest block works
 // through ceil(items / blocks) of them, each its planes plus what an item costs besides (two more planes
-// to load, most of a plane's time).  The length is the one with the shortest such time, up to 16
-// planes: neighbouring columns then stay close enough in z to find their halos in L2.
+// to load and to carry, and a start without overlap: about one plane's time).  The length is the one with the
+// shortest such time, up to 32 planes: neighbouring columns then stay close enough in z to find their halos
+// in L2.
 MarchWork add_items(const lbcad_ctx* c, const StepWork& g, int tx, int ty, int blocks, std::vector<MarchItem>& out) {
-  constexpr double kItemPlanes = 0.8;
+  constexpr double kItemPlanes = 1.0;
   auto columns = [&](const lbcad_grid& b) { return (long long)((b.nx + tx - 1) / tx) * ((b.ny + ty - 1) / ty); };
+  int tallest = 0;
+  for (int i = 0; i < g.ninst; ++i) tallest = std::max(tallest, c->inst[g.first + i].g.nz);
+  auto slabs_of = [&](const lbcad_grid& b, int n) {  // slabs of box b when the tallest box has n
+    return std::max(1, (int)(((long long)b.nz * n + tallest - 1) / tallest));
+  };
   int best = 1;
-  double best_time = 0.0;
-  for (int len = 1; len <= 16; ++len) {
-    long long n = 0;
-    for (int i = 0; i < g.ninst; ++i) {
-      const lbcad_grid& b = c->inst[g.first + i].g;
-      n += columns(b) * ((b.nz + len - 1) / len);
-    }
-    const double t = (double)((n + blocks - 1) / blocks) * (len + kItemPlanes);
-    if (len == 1 || t < best_time) {
-      best = len;
+  double best_time = -1.0;
+  for (int n = (tallest + 31) / 32; n <= tallest; ++n) {
+    long long items = 0;
+    for (int i = 0; i < g.ninst; ++i) items += columns(c->inst[g.first + i].g) * slabs_of(c->inst[g.first + i].g, n);
+    const double t = (double)((items + blocks - 1) / blocks) * ((tallest + n - 1) / n + kItemPlanes);
+    if (best_time < 0.0 || t < best_time) {
+      best = n;
       best_time = t;
     }
   }
@@ -513,7 +516,7 @@ MarchWork add_items(const lbcad_ctx* c, const StepWork& g, int tx, int ty, int b
   for (int i = 0; i < g.ninst; ++i) {
     const lbcad_grid& b = c->inst[g.first + i].g;
     sites += c->inst[g.first + i].N;
-    const int slabs = (b.nz + best - 1) / best;
+    const int slabs = slabs_of(b, best);
     for (int k = 0; k < slabs; ++k) {
       const int zb = (int)((long long)b.nz * k / slabs), ze = (int)((long long)b.nz * (k + 1) / slabs);
       for (int y0 = 0; y0 < b.ny; y0 += ty)
