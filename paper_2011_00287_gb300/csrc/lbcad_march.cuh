@@ -128,7 +128,7 @@ struct Tile {
 };
 
 // Shared-memory planes of a tile.  Q and psi: the field pairs (Q_xx, Q_xy), (Q_xz, Q_yy), (Q_yz, psi), pair j
-// of site k at elements 2 (j SP + k).  Velocity: (u_x, u_y, u_z, -) of site k at 4 k.
+// of site k at elements 2 (j SP + k).  Velocity: (u_x, u_y) of site k at 2 k, u_z at 2 SP + k.
 template <int SP>
 __device__ __forceinline__ int qidx(int f, int k) {
   return (f >> 1) * 2 * SP + 2 * k + (f & 1);
@@ -153,13 +153,8 @@ struct TileAcc {
     return lds2(pl + 2 * (j * G::SP + (from_below ? sc - d : sc + d)));
   }
   __device__ __forceinline__ Vel3<T> u3(int cx, int cy, int cz) const {
-    const T* p = upl[cz + 1] + 4 * at(cx, cy);
-    if constexpr (sizeof(T) == 4) {
-      const float4 v = *reinterpret_cast<const float4*>(p);
-      return Vel3<T>{Vec2<T>{v.x, v.y}, v.z};
-    } else {
-      return Vel3<T>{lds2(p), p[2]};
-    }
+    const int k = at(cx, cy);
+    return Vel3<T>{lds2(upl[cz + 1] + 2 * k), upl[cz + 1][2 * G::SP + k]};
   }
   __device__ __forceinline__ Vec2<T> spair(int, int cx, int cy, int cz) const {
     return Vec2<T>{T(0), mpl[cz + 1][at(cx, cy)]};
@@ -189,7 +184,7 @@ constexpr int kMarchOp = 0, kMarchH = 1, kMarchPred = 2, kMarchOpH = 3;
 template <typename T, class G, int MODE>
 struct FieldsSmem {
   static constexpr int NSLOT = 4;  // planes p-2 (faces below), p-1, p, and the arriving one
-  static constexpr int QSL = 6 * G::SP, USL = MODE == kMarchOp || MODE == kMarchOpH ? 4 * G::SP : 0;
+  static constexpr int QSL = 6 * G::SP, USL = MODE == kMarchOp || MODE == kMarchOpH ? 3 * G::SP : 0;
   static constexpr size_t bytes = (size_t)NSLOT * (QSL + USL) * sizeof(T);
 };
 
@@ -229,9 +224,9 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? blocks_for(TX * TY, 
           for (int f = 0; f < 5; ++f) cp_async_elem(dq + qidx<G::SP>(f, k), (MODE == kMarchPred ? I.qp[f] : I.q_in[f]) + o);
           cp_async_elem(dq + qidx<G::SP>(5, k), (MODE == kMarchPred ? I.qp[5] : I.psi_in) + o);
           if constexpr (OP) {
-            T* du = sU + ((p + 4) & 3) * M::USL + 4 * k;
+            T* du = sU + ((p + 4) & 3) * M::USL;
 #pragma unroll
-            for (int a = 0; a < 3; ++a) cp_async_elem(du + a, I.u_in[a] + o);
+            for (int a = 0; a < 3; ++a) cp_async_elem(du + (a < 2 ? 2 * k + a : 2 * G::SP + k), I.u_in[a] + o);
           }
         }
       }
@@ -642,7 +637,7 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? blocks_for(TX * TY, 
 template <typename T, class G>
 struct OpSmem {
   static constexpr int NSLOT = 4;
-  static constexpr int QSLOT = 6 * G::SP, USLOT = 4 * G::SP, MSLOT = G::SP;
+  static constexpr int QSLOT = 6 * G::SP, USLOT = 3 * G::SP, MSLOT = G::SP;
   __host__ __device__ static constexpr int NSITE(int stage) { return stage == 2 ? 17 : 5; }  // H, rq, Q, psi
   static constexpr size_t site_off = ((size_t)NSLOT * (QSLOT + USLOT + MSLOT) * sizeof(T) + 15) / 16 * 16;
   __host__ __device__ static constexpr size_t bytes(int stage) {
@@ -687,9 +682,9 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 8 ? 2 : blocks_for(TX * 
 #pragma unroll
           for (int f = 0; f < 5; ++f) cp_async_elem(dq + qidx<G::SP>(f, k), (STAGE == 2 ? I.qp[f] : I.q_in[f]) + gs);
           cp_async_elem(dq + qidx<G::SP>(5, k), (STAGE == 2 ? I.qp[5] : I.psi_in) + gs);
-          T* du = sU + sl * M::USLOT + 4 * k;
+          T* du = sU + sl * M::USLOT;
 #pragma unroll
-          for (int a = 0; a < 3; ++a) cp_async_elem(du + a, us[a] + gs);
+          for (int a = 0; a < 3; ++a) cp_async_elem(du + (a < 2 ? 2 * k + a : 2 * G::SP + k), us[a] + gs);
           cp_async_elem(sM + sl * M::MSLOT + k, msrc + (size_t)MST * gs);
         }
       }
