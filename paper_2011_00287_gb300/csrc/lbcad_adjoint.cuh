@@ -25,7 +25,7 @@ namespace lbcad {
 template <typename T>
 struct AdjDesc {
   InstDesc<T> I;      // state s_t in I.*_in, its H in I.H; *_out unused
-  const T* S;         // its stress and mu: three quads per site [3][N][4] (see lbcad_march.cuh)
+  const T* S;         // its stress and mu: arrays of pairs [6][N][2] (see PairPlane in lbcad_march.cuh)
   const T* lg;        // cotangent of s_{t+1}: g* (19), Q (5), psi (1), u (3)
   const T* lq;
   const T* lp;
@@ -42,13 +42,12 @@ struct AdjDesc {
 
 constexpr int kAdjBlock = 128;
 
-// GlobalAcc with the stress pairs read from the scratch quads (see QuadPlane in lbcad_march.cuh).
+// GlobalAcc with the stress pairs read from the step's scratch (see PairPlane in lbcad_march.cuh).
 template <typename T>
 struct AdjAcc : GlobalAcc<T> {
   const T* S;
   __device__ __forceinline__ Vec2<T> spair(int j, int cx, int cy, int cz) const {
-    const int q = j < 2 ? 0 : (j < 4 ? 1 : 2), o = (j == 1 || j == 2) ? 2 : 0;
-    const T* p = S + 4 * (q * this->N + this->nb.off(cx, cy, cz)) + o;
+    const T* p = S + 2 * (j * this->N + this->nb.off(cx, cy, cz));
     if constexpr (sizeof(T) == 4) {
       const float2 v = __ldg(reinterpret_cast<const float2*>(p));
       return Vec2<T>{v.x, v.y};

@@ -114,6 +114,7 @@ template <typename T>
 struct MarchDesc {
   int nx, ny, nz;
   unsigned plane;      // nx ny
+  unsigned N;          // sites
   const T* g_in[19];   // as InstDesc, by component
   T* g_out[19];
   const T* q_in[5];
@@ -122,7 +123,7 @@ struct MarchDesc {
   T* psi_out;
   const T* u_in[3];
   T* u_out[3];
-  T* S[3];             // scratch of the default path: three quads per site [N][4] (see lbcad_march.cuh)
+  T* S[6];             // scratch of the default path: arrays of pairs [N][2] (see PairPlane in lbcad_march.cuh)
   T* H[5];             // sync coupling, Heun: H at t
   T* rq[6];            // Heun: right-hand side at t, predicted state (Q, psi), H and mu there
   T* qp[6];
@@ -218,7 +219,7 @@ struct LaunchFused {
 template <typename T>
 struct AdjDescHost {
   InstDesc<T> I;                 // state s_t (inputs) and its H
-  const T* S;                    // its stress and mu: three quads per site [3][N][4] (see lbcad_march.cuh)
+  const T* S;                    // its stress and mu: arrays of pairs [6][N][2] (see PairPlane in lbcad_march.cuh)
   const T *lg, *lq, *lp, *lu;    // cotangent of s_{t+1}
   T *A, *Bf, *ls;                // work: 88 + 36 + 15 values per site
   T *og, *oq, *op, *ou;          // cotangent of s_t

@@ -2,7 +2,7 @@
 //
 //   k_march_fields (a1-a4): per site the stencils of Q and psi, H, mu and the stress sigma, and
 //     with the lagged Euler step also the whole update of Q and the flux divergence of psi; leaves
-//     sigma, mu, the divergence and psi in a scratch of 12 values per site (three aligned quads);
+//     sigma, mu, the divergence and psi in a scratch of 12 values per site (six arrays of pairs);
 //   k_march_lb (a3, a5, a4 of psi, a6): the force F = div sigma and lap mu from that scratch, the pull of
 //     the populations, the collision, psi, and the conserved sums.
 //
@@ -68,13 +68,9 @@ __device__ __forceinline__ void st_out(T* p, T v) {
   __stcg(p, v);
 }
 template <typename T>
-__device__ __forceinline__ void st_quad(T* p, T a, T b, T c, T d) {
-  if constexpr (sizeof(T) == 4) {
-    __stcg(reinterpret_cast<float4*>(p), make_float4(a, b, c, d));
-  } else {
-    __stcg(reinterpret_cast<double2*>(p), make_double2(a, b));
-    __stcg(reinterpret_cast<double2*>(p) + 1, make_double2(c, d));
-  }
+__device__ __forceinline__ void st_pair(T* p, T a, T b) {
+  if constexpr (sizeof(T) == 4) __stcg(reinterpret_cast<float2*>(p), make_float2(a, b));
+  else __stcg(reinterpret_cast<double2*>(p), make_double2(a, b));
 }
 
 __device__ __forceinline__ void cp_async4(void* smem_dst, const void* gsrc) {
@@ -92,24 +88,31 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
 __device__ __forceinline__ void cp_async_commit_wait_all() {
   asm volatile("cp.async.commit_group;\ncp.async.wait_all;\n" ::: "memory");
 }
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+// Waits until at most the N latest groups are still on their way.
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 template <typename T>
 __device__ __forceinline__ void cp_async_elem(T* dst, const T* src) {
   if constexpr (sizeof(T) == 4) cp_async4(dst, src); else cp_async8(dst, src);
 }
-// Quad s of an array of quads.
+// Component i of a field of n sites from a pointer into component 0: one wide multiply-add (a table of component
+// pointers in the launch's arguments costs a constant load each, through the same queue as the shared-memory
+// accesses).
 template <typename T>
-__device__ __forceinline__ T* quad(T* base, unsigned s) {
-  struct alignas(4 * sizeof(T)) Q { T v[4]; };
-  return reinterpret_cast<T*>(reinterpret_cast<Q*>(base) + s);
+__device__ __forceinline__ T* comp(T* p, int i, unsigned n) {
+  return reinterpret_cast<T*>(reinterpret_cast<uintptr_t>(p) + (unsigned long long)n * (unsigned)(i * (int)sizeof(T)));
+}
+
+// Pair s of an array of pairs.
+template <typename T>
+__device__ __forceinline__ T* pair_at(T* base, unsigned s) {
+  struct alignas(2 * sizeof(T)) P { T v[2]; };
+  return reinterpret_cast<T*>(reinterpret_cast<P*>(base) + s);
 }
 template <typename T>
-__device__ __forceinline__ const T* quad(const T* base, unsigned s) {
-  return quad(const_cast<T*>(base), s);
-}
-template <typename T>
-__device__ __forceinline__ void cp_async_quad(T* dst, const T* src) {
-  cp_async16(dst, src);
-  if constexpr (sizeof(T) == 8) cp_async16(dst + 2, src + 2);
+__device__ __forceinline__ void cp_async_pair(T* dst, const T* src) {
+  if constexpr (sizeof(T) == 4) cp_async8(dst, src); else cp_async16(dst, src);
 }
 
 // Programmatic dependent launch (MarchWork::early): every kernel of a step lets the next one start its blocks
@@ -188,8 +191,8 @@ struct FieldsSmem {
   static constexpr size_t bytes = (size_t)NSLOT * (QSL + USL) * sizeof(T);
 };
 
-// kMarchOp: sigma, mu, the flux divergence and psi of every site into the scratch quads and the new Q
-// (Euler with the velocity of the previous step).  kMarchH: sigma and mu into the quads, H into its
+// kMarchOp: sigma, mu, the flux divergence and psi of every site into the scratch pairs and the new Q
+// (Euler with the velocity of the previous step).  kMarchH: sigma and mu into the pairs, H into its
 // scratch (sync coupling, Heun).  kMarchOpH: both (replay of the adjoint).  kMarchPred: H and mu of the Heun predicted state qp into the sigma
 // scratch (H at sig[0..5N), mu at sig[5N..6N)).
 template <typename T, int MI, int TX, int TY, int MODE>
@@ -262,8 +265,9 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? blocks_for(TX * TY, 
             for (int k = 0; k < 5; ++k) st_out(I.Hp[k] + s, H[k]);
             st_out(I.Hp[5] + s, mu);
           } else {
-            st_quad(quad(I.S[0], s), sig[0], sig[3], sig[1], sig[4]);
-            st_quad(quad(I.S[1], s), sig[6], sig[7], sig[2], sig[5]);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) st_pair(pair_at(I.S[j], s), sig[pair_c0(j)], sig[pair_c1(j)]);
+            st_pair(pair_at(I.S[4], s), sig[8], mu);
             T div = T(0);
             if constexpr (OP) {
               TileAcc<T, G> acc;
@@ -286,7 +290,7 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? blocks_for(TX * TY, 
 #pragma unroll
               for (int k = 0; k < 5; ++k) st_out(I.H[k] + s, H[k]);
             }
-            st_quad(quad(I.S[2], s), sig[8], mu, div, p0);
+            st_pair(pair_at(I.S[5], s), div, p0);
           }
         }
       }
@@ -308,19 +312,19 @@ __device__ __forceinline__ void pull_populations(const MarchDesc<T>& I, const un
 #pragma unroll
   for (int i = 0; i < V::Q; ++i) {
     const unsigned o = zo[1 - V::c(i, 2)] + pyo[1 - V::c(i, 1)] + pxo[1 - V::c(i, 0)];
-    cp_async_elem(dst + i * STRIDE, I.g_in[i] + o);
+    cp_async_elem(dst + i * STRIDE, comp(I.g_in[0], i, I.N) + o);
   }
 }
 
-// The stress pairs of one plane of scratch quads in shared memory (quad q of tile site k at 4 (q SP + k)):
-// (sigma_xx, sigma_yx, sigma_xy, sigma_yy), (sigma_zx, sigma_zy, sigma_xz, sigma_yz), (sigma_zz, mu, div, psi).
+// The scratch pairs of one plane in shared memory (pair j of tile site k at 2 (j SP + k)): the stress pairs (sig_pair) with
+// mu in pair 4, and pair 5 = (flux divergence, psi).  As pairs, a warp's read of one takes two wavefronts; read
+// from quads it took four.
 template <typename T, class G>
-struct QuadPlane {
+struct PairPlane {
   const T* pl;
   int sc;
   __device__ __forceinline__ Vec2<T> spair(int j, int cx, int cy) const {
-    const int q = j < 2 ? 0 : (j < 4 ? 1 : 2), o = (j == 1 || j == 2) ? 2 : 0;
-    return lds2(pl + 4 * (q * G::SP + sc + cy * G::SW + cx) + o);
+    return lds2(pl + 2 * (j * G::SP + sc + cy * G::SW + cx));
   }
   // component c (= 3a + b) of the stress
   __device__ __forceinline__ T comp(int c, int cx, int cy) const {
@@ -524,7 +528,7 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? blocks_for(TX * TY, 
         if (k < G::SP) {
           const unsigned o = gz + off[r];
 #pragma unroll
-          for (int q = 0; q < 3; ++q) cp_async_quad(d + 4 * (q * G::SP + k), quad((const T*)I.S[q], o));
+          for (int j = 0; j < 6; ++j) cp_async_pair(d + 2 * (j * G::SP + k), pair_at(I.S[j], o));
         }
       }
     };
@@ -535,8 +539,8 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? blocks_for(TX * TY, 
     const unsigned pxo[3] = {(unsigned)(x ? x - 1 : nx - 1), (unsigned)x, (unsigned)(x + 1 < nx ? x + 1 : 0)};
     const unsigned pyo[3] = {(unsigned)((y ? y - 1 : ny - 1) * nx), (unsigned)(y * nx),
                              (unsigned)((y + 1 < ny ? y + 1 : 0) * nx)};
-    // the pulled populations arrive like the planes, one plane ahead, each thread's in its own places: read
-    // when they were needed, they left the kernel waiting for memory in 40% of its time
+    // the pulled populations of a plane are copied to each thread's own places while the plane before is worked
+    // on, and waited for just before they are used, not with the planes at the barrier
     T* const pulled = sS + M::NSLOT * M::SL + tid;
     auto pull = [&](int z) {
       const unsigned zo[3] = {(unsigned)wrap_plane(z - 1, nz) * plane, (unsigned)z * plane,
@@ -550,8 +554,10 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? blocks_for(TX * TY, 
     issue(zb - 1);
     issue(zb);
     issue(zb + 1);
+    cp_async_commit();
     if (inside) pull(zb);
-    cp_async_commit_wait_all();
+    cp_async_commit();
+    cp_async_wait<1>();
     Vec2<T> trx = v2(T(0), T(0)), trY = v2(T(0), T(0));
     if constexpr (OBS) {
       if (inside) {
@@ -565,23 +571,24 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? blocks_for(TX * TY, 
 #pragma unroll 1
     for (int p = zb - 1; p <= ze; ++p) {
       if (p > zb && p < ze) issue(p + 1);
+      cp_async_commit();
       if (inside) {
         const int z = p - 1;
         Vec2<T> trz = v2(T(0), T(0));
-        if (p > zb) {
-          if (p < ze) pull(p);
-          if constexpr (OBS) trz = ldg2(I.trig + 2 * (nx + ny + z));
-        }
+        if (OBS && p > zb) trz = ldg2(I.trig + 2 * (nx + ny + z));
         T F[3], lapmu = T(0);
-        const QuadPlane<T, G> np{slot(p), sc};
+        const PairPlane<T, G> np{slot(p), sc};
         if constexpr (FORM == 0) force.advance([&](int j, int cx, int cy) { return np.spair(j, cx, cy); }, F);
         else force.advance([&](int j, int cx, int cy) { return np.apair(j, cx, cy); }, F);
         if constexpr (MODE != kFusedLbOnly) lapmu = lapm.advance([&](int cx, int cy) { return np.spair(4, cx, cy).y; });
         if (p > zb) {
-          const QuadPlane<T, G> cp{slot(z), sc};
+          const PairPlane<T, G> cp{slot(z), sc};
           T g[V::Q], u[3], mom[4];
+          cp_async_wait<1>();  // the populations of plane z; the scratch of plane p + 1 may still be arriving
 #pragma unroll
           for (int i = 0; i < V::Q; ++i) g[i] = pulled[(z & 1) * M::PULL + i * G::NT];
+          if (p < ze) pull(p);
+          cp_async_commit();
           if constexpr (FORM == 0) {
             lb_collide<T, SHIFT, V>(cf, F, g, u, OBS ? mom : nullptr);
           } else {
@@ -591,12 +598,14 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? blocks_for(TX * TY, 
             lb_collide_stress<T, SHIFT, V>(cf, F, sg, g, u, OBS ? mom : nullptr);
           }
           const unsigned s = (unsigned)z * plane + soff;
+          T* const go = I.g_out[0] + s;
+          T* const uo = I.u_out[0] + s;
 #pragma unroll
-          for (int i = 0; i < V::Q; ++i) st_out(I.g_out[i] + s, g[i]);
+          for (int i = 0; i < V::Q; ++i) st_out(comp(go, i, I.N), g[i]);
 #pragma unroll
-          for (int a = 0; a < 3; ++a) st_out(I.u_out[a] + s, u[a]);
+          for (int a = 0; a < 3; ++a) st_out(comp(uo, a, I.N), u[a]);
           if constexpr (MODE != kFusedLbOnly) {
-            const Vec2<T> dp = lds2(cp.pl + 4 * (2 * G::SP + sc) + 2);  // flux divergence, psi
+            const Vec2<T> dp = cp.spair(5, 0, 0);  // flux divergence, psi
             const T pn = dp.y + fma(cf.M, lapmu, -dp.x);
             st_out(I.psi_out + s, pn);
             if constexpr (OBS) {
@@ -611,10 +620,12 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? blocks_for(TX * TY, 
       }
       // the next issue overwrites plane p-1: from p = zb on, every warp is done with it first
       if (p >= zb) {
-        cp_async_commit_wait_all();
+        if (p > zb && inside) cp_async_wait<1>();  // the scratch of plane p + 1; the populations of plane p may still be arriving
+        else cp_async_wait<0>();
         __syncthreads();
       }
     }
+    cp_async_wait<0>();
   }
   if constexpr (OBS) {
     ObsReduce<T, G::NT>::run(sums, smem_raw, ob, blockIdx.x * ob.maxrun + run);
@@ -665,9 +676,9 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 8 ? 2 : blocks_for(TX * 
     const int nx = I.nx, ny = I.ny, nz = I.nz;
     const unsigned plane = I.plane;
     const T* const* const us = sync ? I.u_out : I.u_in;
-    // mu: planar at the predicted state (corrector), lane 1 of the last scratch quad otherwise
-    const T* msrc = STAGE == 2 ? I.Hp[5] : I.S[2] + 1;
-    constexpr int MST = STAGE == 2 ? 1 : 4;
+    // mu: planar at the predicted state (corrector), lane 1 of scratch pair 4 otherwise
+    const T* msrc = STAGE == 2 ? I.Hp[5] : I.S[4] + 1;
+    constexpr int MST = STAGE == 2 ? 1 : 2;
     unsigned off[G::LD];
     tile_offsets<G>(tl, nx, ny, off);
     auto issue = [&](int p) {

@@ -198,6 +198,7 @@ MarchDesc<T> make_march_desc(const Inst& I, int parity, bool shifted) {
   std::memset(&d, 0, sizeof(d));
   d.nx = I.g.nx; d.ny = I.g.ny; d.nz = I.g.nz;
   d.plane = (unsigned)((long long)I.g.nx * I.g.ny);
+  d.N = (unsigned)I.N;
   const long long N = I.N;
   const int a = parity, b = parity ^ 1, q = (I.p.lattice == LBCAD_D3Q15) ? 15 : 19;
   auto comps = [&](auto* dst, void* base, int n, long long stride) {
@@ -211,7 +212,7 @@ MarchDesc<T> make_march_desc(const Inst& I, int parity, bool shifted) {
   d.psi_out = (T*)I.pb[b];
   comps(d.u_in, I.ub[a], 3, N);
   comps(d.u_out, I.ub[b], 3, N);
-  comps(d.S, I.S, 3, 4 * N);
+  comps(d.S, I.S, 6, 2 * N);
   comps(d.H, I.H, 5, N);
   comps(d.rq, I.rq, 6, N);
   comps(d.qp, I.qp, 6, N);
@@ -1060,8 +1061,8 @@ MarchDesc<T> replay_desc(const MarchDesc<T>& base, long long N, const StateBuf<T
   for (int a = 0; a < 3; ++a) {
     d.u_in[a] = in.u + a * N;
     d.u_out[a] = out.u + a * N;
-    d.S[a] = f + 4 * a * N;
   }
+  for (int j = 0; j < 6; ++j) d.S[j] = f + 2 * j * N;
   d.psi_in = in.p;
   d.psi_out = out.p;
   return d;
@@ -1083,7 +1084,7 @@ int adjoint_impl(lbcad_ctx* c, int64_t nsteps, int k, double* dzeta, double* dq0
   const long long N = I.N;
   const int S = (int)((nsteps + k - 1) / k);
   const size_t st = 28 * (size_t)N;  // elements of one stored state
-  const size_t fs = 17 * (size_t)N;  // elements of one state's stress quads (12) and H (5)
+  const size_t fs = 17 * (size_t)N;  // elements of one state's stress pairs (12) and H (5)
   // buffers through the context's allocator, kept for the next call
   c->adj_lam = nullptr;
   T* ck = (T*)adj_buffer(c, 0, (size_t)S * st * sizeof(T));
