@@ -1,90 +1,104 @@
 // lbcad_adjoint.cuh -- reverse mode (vector-Jacobian products) of one hybrid step.
 //
 // The step maps the stored state s_t = (g*, Q, psi, u) to s_{t+1}.  Given the cotangent
-// lam_{t+1} of s_{t+1}, four gather-form kernels produce lam_t:
-//   RK1 k_adj_update : per site, VJP of update_math (upwind/co-rotation Q update,
-//                      Cahn-Hilliard psi update, BGK + Guo collision) with respect to its
-//                      88 inputs (F, lap mu, grad u, Q and psi faces, u faces, H, pulled g),
-//                      by a hand-written reverse sweep (update_math_vjp)
-//   RK2 k_adj_spread : transposes of the stencils that fed update_math: div sigma -> sigma,
-//                      lap mu -> mu, grad u -> u, face reads -> Q/psi/u, the pull -> g*
-//   RK3 k_adj_fields : per site, VJP of local_fields (H, mu, sigma of Eqs. 2-5) with respect
-//                      to its 36 inputs (Q, psi and their stencils) and to zeta and q0, by a
-//                      hand-written reverse sweep (local_fields_vjp)
-//   RK4 k_adj_gather : transposes of the Q/psi stencils (gradient, Laplacian, Hessian)
+// lam_{t+1} of s_{t+1}, three gather-form kernels produce lam_t:
+//   RK1 k_adj_update : per site, VJP of the update (upwind/co-rotation Q update, Cahn-Hilliard psi
+//                      update, BGK + Guo collision) by a hand-written reverse sweep;
+//   RK2 k_adj_fields : transposes of the stencils that fed the update (div sigma -> sigma, lap mu -> mu,
+//                      grad u -> u, face reads -> Q/psi/u, the pull -> g*), then per site the VJP of
+//                      local_fields (H, mu, sigma of Eqs. 2-5) with respect to its inputs and to zeta and
+//                      q0, by a hand-written reverse sweep;
+//   RK3 k_adj_gather : transposes of the Q/psi stencils (gradient, Laplacian, Hessian).
 // The per-site reverse sweeps recompute the forward intermediates of the site and take
 // every branch (upwind sides) as the forward takes it.  Stencil transposes use the negated offsets on the
 // periodic lattice, so no site is written by two threads.
+//
+// What bounds them is the traffic between them: a site's full input cotangents are 88 values of the update and 36
+// of local_fields.  Most of these are a factor known at the reading site times a cotangent it can read anyway
+// (populations: (1 - 1/tau) lam_g plus a linear form of four values; upwind faces: the face velocity times lam_Q
+// or lam_psi; lap mu and H: a coefficient times lam; lap Q, lap psi and the Hessian of psi: K lH, and lmu times
+// Q), so only 16 values of the first and 24 of the second are passed, in quads and pairs.  The force F of
+// each replayed step is kept by the replay (3 values per site and state), so that no stress is needed here.
 #pragma once
 
 #include "lbcad_kernels.cuh"
 
 namespace lbcad {
 
-// Buffers of one reverse step (all [component][site]).
+// Buffers of one reverse step.
 template <typename T>
 struct AdjDesc {
-  InstDesc<T> I;      // state s_t in I.*_in, its H in I.H; *_out unused
-  const T* S;         // its stress and mu: arrays of pairs [6][N][2] (see PairPlane in lbcad_march.cuh)
-  const T* lg;        // cotangent of s_{t+1}: g* (19), Q (5), psi (1), u (3)
+  InstDesc<T> I;      // state s_t in I.*_in; the rest unused
+  const T* F;         // force of the step from s_t [3][site]
+  const T* lg;        // cotangent of s_{t+1}: g* (19), Q (5), psi (1), u (3), [component][site]
   const T* lq;
   const T* lp;
   const T* lu;
-  T* A;               // RK1 output: 88 input cotangents of update_math per site
-  T* Bf;              // RK3 output: 36 input cotangents of local_fields per site
-  T* ls;              // RK2 output: cotangents of sigma (9), mu (1), H (5)
-  T* og;              // cotangent of s_t: g* (19), Q (5), psi (1), u (3)
+  T* A;               // RK1 -> RK2, quads [5][site][4]: (lF, lm0), (lj, -), (lW_ab over a, -) for b = x, y, z
+  T* B;               // RK2 -> RK3: quads [4][site][4]: ldQ_a components 0-3 for a = x, y, z, lH 0-3; then
+                      // pairs [4][site][2]: (ldQ_a component 4, ldpsi_a) for a = x, y, z, (lH 4, lmu)
+  T* og;              // cotangent of s_t: g* (19), Q (5), psi (1), u (3); RK1 leaves the site-local parts of Q, psi, u
   T* oq;
   T* op;
   T* ou;
-  double* pgrad;      // per-block partial sums of d/dzeta, d/dq0 (2 per block)
+  double* pgrad;      // per block: sums over the reverse steps of d/dzeta, d/dq0 (2 per block)
 };
 
 constexpr int kAdjBlock = 128;
 
-// GlobalAcc with the stress pairs read from the step's scratch (see PairPlane in lbcad_march.cuh).
 template <typename T>
-struct AdjAcc : GlobalAcc<T> {
-  const T* S;
-  __device__ __forceinline__ Vec2<T> spair(int j, int cx, int cy, int cz) const {
-    const T* p = S + 2 * (j * this->N + this->nb.off(cx, cy, cz));
-    if constexpr (sizeof(T) == 4) {
-      const float2 v = __ldg(reinterpret_cast<const float2*>(p));
-      return Vec2<T>{v.x, v.y};
-    } else {
-      const double2 v = __ldg(reinterpret_cast<const double2*>(p));
-      return Vec2<T>{v.x, v.y};
-    }
-  }
+struct Quad {
+  T x, y, z, w;
 };
+template <typename T>
+__device__ __forceinline__ Quad<T> ld_quad(const T* base, long long s) {
+  if constexpr (sizeof(T) == 4) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(base) + s);
+    return Quad<T>{v.x, v.y, v.z, v.w};
+  } else {
+    const double2 v = __ldg(reinterpret_cast<const double2*>(base) + 2 * s), w = __ldg(reinterpret_cast<const double2*>(base) + 2 * s + 1);
+    return Quad<T>{v.x, v.y, w.x, w.y};
+  }
+}
+template <typename T>
+__device__ __forceinline__ void st_quad_at(T* base, long long s, T a, T b, T c, T d) {
+  if constexpr (sizeof(T) == 4) {
+    reinterpret_cast<float4*>(base)[s] = make_float4(a, b, c, d);
+  } else {
+    reinterpret_cast<double2*>(base)[2 * s] = make_double2(a, b);
+    reinterpret_cast<double2*>(base)[2 * s + 1] = make_double2(c, d);
+  }
+}
+template <typename T>
+__device__ __forceinline__ Vec2<T> ld_pair(const T* base, long long s) {
+  if constexpr (sizeof(T) == 4) {
+    const float2 v = __ldg(reinterpret_cast<const float2*>(base) + s);
+    return Vec2<T>{v.x, v.y};
+  } else {
+    const double2 v = __ldg(reinterpret_cast<const double2*>(base) + s);
+    return Vec2<T>{v.x, v.y};
+  }
+}
+template <typename T>
+__device__ __forceinline__ void st_pair_at(T* base, long long s, T a, T b) {
+  if constexpr (sizeof(T) == 4) reinterpret_cast<float2*>(base)[s] = make_float2(a, b);
+  else reinterpret_cast<double2*>(base)[s] = make_double2(a, b);
+}
 
 // ---------------------------------------------------------------- reverse mode of update_math
 // Vector-Jacobian product of update_math (D3Q19 body-force collision, Euler update) at one
-// site, by a hand-written reverse sweep over the forward arithmetic: in = the 88 inputs
-// (layout of k_adj_update), lo = the cotangents of the 28 outputs (qn 0-4, pn 5, u 6-8,
-// g 9-27), out = the cotangents of the 88 inputs.  The branches (upwind selection, face
-// fluxes) take the side the forward takes, as forward-mode differentiation of the same
+// site, by a hand-written reverse sweep over the forward arithmetic: lo = the cotangents of the 28 outputs
+// (qn 0-4, pn 5, u 6-8, g 9-27).  Results: lF, lW (grad u), the site-local parts of the cotangents of Q, psi and
+// u (lq0, lp0, lu0), and lm0, lj, in which the cotangent of pulled population i is
+// (1 - 1/tau) lo[9 + i] + lm0 + c_i . lj.  The cotangents of lap mu (M lo[5]), H (Gamma lo[k]) and of the face
+// values are formed where they are read (k_adj_fields).  qu: Q at the upwind neighbours.  The branches (upwind
+// selection, face fluxes) take the side the forward takes, as forward-mode differentiation of the same
 // code would.
 template <typename T, bool SHIFT>
-__device__ __forceinline__ void update_math_vjp(const Coef<T>& c, const T in[88], const T lo[28], T out[88]) {
-  const T* F = in;
-  const T lapmu_unused = in[3];
-  (void)lapmu_unused;
-  T W[3][3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) W[a][b] = in[4 + 3 * a + b];
-  const T* q0 = in + 13;
-  const T* qfl = in + 18;  // qf[f][k] = qfl[5 f + k]
-  const T p0 = in[48];
-  const T* pf = in + 49;
-  const T* u0 = in + 55;
-  const T* uf = in + 58;
-  const T* g = in + 69;
-#pragma unroll
-  for (int j = 0; j < 88; ++j) out[j] = T(0);
-
+__device__ __forceinline__ void update_math_vjp(const Coef<T>& c, const T F[3], const T W[3][3], const T q0[5],
+                                                const T qu[3][5], T p0, const T pf[6], const T u0[3], const T uf[6],
+                                                const T g[19], const T lo[28], T lF[3], T lW[3][3], T lq0[5], T& lp0,
+                                                T lu0v[3], T& lm0, T lj[3]) {
   // ---- LB collision (outputs u 6-8, g 9-27)
   T m0 = g[0];
   T jm[3] = {T(0), T(0), T(0)};
@@ -104,12 +118,11 @@ __device__ __forceinline__ void update_math_vjp(const Coef<T>& c, const T in[88]
   const T u2 = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
   const T r45 = T(4.5) * rho, r3 = T(3) * rho, om = c.tau_inv;
   T lu[3] = {lo[6], lo[7], lo[8]};
-  T lF[3] = {T(0), T(0), T(0)};
+  lF[0] = lF[1] = lF[2] = T(0);
   T lbase = T(0), lr45 = T(0), lr3 = T(0), luF = T(0);
   {
     const T w = T(lat_w(0));
     const T l0 = lo[9];
-    out[69] += (T(1) - om) * l0;
     lbase += om * w * l0;
     luF += -T(3) * c.guo * w * l0;
   }
@@ -119,8 +132,6 @@ __device__ __forceinline__ void update_math_vjp(const Coef<T>& c, const T in[88]
     const T cu = T(lat_c(i, 0)) * u[0] + T(lat_c(i, 1)) * u[1] + T(lat_c(i, 2)) * u[2];
     const T cF = T(lat_c(i, 0)) * F[0] + T(lat_c(i, 1)) * F[1] + T(lat_c(i, 2)) * F[2];
     const T lp = lo[9 + i], lm = lo[10 + i];
-    out[69 + i] += (T(1) - om) * lp;
-    out[70 + i] += (T(1) - om) * lm;
     const T lA = om * (lp + lm), lB = om * (lp - lm), lC = lp + lm, lE = lp - lm;
     lbase += w * lA;
     lr45 += w * cu * cu * lA;
@@ -137,7 +148,8 @@ __device__ __forceinline__ void update_math_vjp(const Coef<T>& c, const T in[88]
     }
   }
   // base = m0 - 1.5 rho u2 (shifted) or rho - 1.5 rho u2; r45 = 4.5 rho; r3 = 3 rho
-  T lm0 = T(0), lrho = T(0), lu2 = T(0);
+  T lrho = T(0), lu2 = T(0);
+  lm0 = T(0);
   if (SHIFT) lm0 += lbase; else lrho += lbase;
   lrho += -T(1.5) * u2 * lbase + T(4.5) * lr45 + T(3) * lr3;
   lu2 += -T(1.5) * rho * lbase;
@@ -147,7 +159,7 @@ __device__ __forceinline__ void update_math_vjp(const Coef<T>& c, const T in[88]
     lF[a] += u[a] * luF;
   }
   // u = (j + F/2) / rho
-  T lrinv = T(0), lj[3];
+  T lrinv = T(0);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     lrinv += (jm[a] + T(0.5) * F[a]) * lu[a];
@@ -156,27 +168,12 @@ __device__ __forceinline__ void update_math_vjp(const Coef<T>& c, const T in[88]
   }
   lrho += -rinv * rinv * lrinv;
   lm0 += lrho;
-#pragma unroll
-  for (int i = 0; i < 19; ++i) {
-    T v = lm0;
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-      if (lat_c(i, a)) v += T(lat_c(i, a)) * lj[a];
-    out[69 + i] += v;
-  }
-#pragma unroll
-  for (int a = 0; a < 3; ++a) out[a] += lF[a];
 
   // ---- order-parameter update (outputs qn 0-4, pn 5)
   const T xi = c.xi;
-  T lq0[5];
 #pragma unroll
-  for (int k = 0; k < 5; ++k) {
-    lq0[k] = lo[k];
-    out[64 + k] += c.gammaQ * lo[k];
-  }
-  out[48] += lo[5];              // p0
-  out[3] += c.M * lo[5];         // lap mu
+  for (int k = 0; k < 5; ++k) lq0[k] = lo[k];
+  lp0 = lo[5];
   const T ldivJ = -lo[5];
   // co-rotation S of the five stored components
   T Q[3][3];
@@ -195,7 +192,7 @@ __device__ __forceinline__ void update_math_vjp(const Coef<T>& c, const T in[88]
 #pragma unroll
     for (int j = 0; j < 3; ++j) trQW += Q[i][j] * W[j][i];
   const T cq = -T(2) * xi * trQW;
-  const T c23 = T(2) * xi / T(3);
+  const T c23 = c.xi23;
   T lQ[3][3], lD[3][3], lO[3][3];
 #pragma unroll
   for (int i = 0; i < 3; ++i)
@@ -225,10 +222,9 @@ __device__ __forceinline__ void update_math_vjp(const Coef<T>& c, const T in[88]
     if (i == j) lcdiag += L;
   }
   // cdiag = cq/3 - (2 xi/9) trD; cq = -2 xi tr(QW)
-  lcq += lcdiag / T(3);
-  const T ltrD = -(T(2) * xi / T(9)) * lcdiag;
+  lcq += lcdiag * T(1.0 / 3.0);
+  const T ltrD = -c.xi29 * lcdiag;
   const T ltrQW = -T(2) * xi * lcq;
-  T lW[3][3];
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -249,60 +245,44 @@ __device__ __forceinline__ void update_math_vjp(const Coef<T>& c, const T in[88]
       lW[i][j] += T(0.5) * (lD[i][j] + lO[i][j]);
       lW[j][i] += T(0.5) * (lD[i][j] - lO[i][j]);
     }
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) out[4 + 3 * a + b] += lW[a][b];
   lq0[0] += lQ[0][0] - lQ[2][2];
   lq0[1] += lQ[0][1] + lQ[1][0];
   lq0[2] += lQ[0][2] + lQ[2][0];
   lq0[3] += lQ[1][1] - lQ[2][2];
   lq0[4] += lQ[1][2] + lQ[2][1];
-  // upwind advection of Q and the psi face fluxes
+  // upwind advection of Q, -|u| (q0 - qu), and the psi face fluxes
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const int ip = 2 * a, im = 2 * a + 1;
-    const T up = u0[a] > T(0) ? u0[a] : T(0);
-    const T um = u0[a] < T(0) ? u0[a] : T(0);
-    T lup = T(0), lum = T(0);
+    const T ua = fabs(u0[a]);
+    T d = T(0);
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-      const T ladv = -lo[k];
-      lup += (q0[k] - qfl[5 * im + k]) * ladv;
-      lum += (qfl[5 * ip + k] - q0[k]) * ladv;
-      lq0[k] += (up - um) * ladv;
-      out[18 + 5 * im + k] += -up * ladv;
-      out[18 + 5 * ip + k] += um * ladv;
+      d += (q0[k] - qu[a][k]) * lo[k];
+      lq0[k] -= ua * lo[k];
     }
-    T lu0 = (u0[a] > T(0) ? lup : T(0)) + (u0[a] < T(0) ? lum : T(0));
+    T lu0 = u0[a] > T(0) ? -d : (u0[a] < T(0) ? d : T(0));
     const T ubp = T(0.5) * (u0[a] + uf[ip]);
-    const T lJp = ldivJ;
-    if (ubp > T(0)) out[48] += ubp * lJp; else out[49 + ip] += ubp * lJp;
-    const T lubp = (ubp > T(0) ? p0 : pf[ip]) * lJp;
-    lu0 += T(0.5) * lubp;
-    out[58 + ip] += T(0.5) * lubp;
+    if (ubp > T(0)) lp0 += ubp * ldivJ;
+    lu0 += T(0.5) * ((ubp > T(0) ? p0 : pf[ip]) * ldivJ);
     const T ubm = T(0.5) * (uf[im] + u0[a]);
-    const T lJm = -ldivJ;
-    if (ubm > T(0)) out[49 + im] += ubm * lJm; else out[48] += ubm * lJm;
-    const T lubm = (ubm > T(0) ? pf[im] : p0) * lJm;
-    out[58 + im] += T(0.5) * lubm;
-    lu0 += T(0.5) * lubm;
-    out[55 + a] += lu0;
+    if (!(ubm > T(0))) lp0 -= ubm * ldivJ;
+    lu0 -= T(0.5) * ((ubm > T(0) ? pf[im] : p0) * ldivJ);
+    lu0v[a] = lu0;
   }
-#pragma unroll
-  for (int k = 0; k < 5; ++k) out[13 + k] += lq0[k];
 }
 
 // ---------------------------------------------------------------- reverse mode of local_fields
 // Vector-Jacobian product of local_fields at one site by a hand-written reverse sweep: in =
 // the 36 inputs (q0 0-4, psi 5, dq 6-20 as 6 + 5a + k, lapq 21-25, dp 26-28, lapp 29,
 // hp 30-35), lo = the cotangents of its outputs (H 0-4, mu 5, sigma 6-14), out = the
-// cotangents of the 36 inputs; lzeta and lq0 receive the derivatives with respect to the
-// parameters zeta and q0.  Full 3x3 cotangents of Q and dQ_a are accumulated entry by entry
+// cotangents of inputs 0-20 and, at 21-23, of dp; lH and lmu_out, in which those of lapq, lapp and hp are K lH,
+// -kphi lmu and -2 W lmu (Q_aa on the diagonal, 2 Q_ab off it); lzeta and lq0 receive the derivatives with respect
+// to the parameters zeta and q0.  Full 3x3 cotangents of Q and dQ_a are accumulated entry by entry
 // as the forward reads them and folded onto the five stored components at the end.
 template <typename T>
-__device__ __forceinline__ void local_fields_vjp(const Coef<T>& c, const T in[36], const T lo[15], T out[36],
-                                                 T& lzeta, T& lq0) {
+__device__ __forceinline__ void local_fields_vjp(const Coef<T>& c, const T in[36], const T lo[15], T out[24],
+                                                 T lH[5], T& lmu_out, T& lzeta, T& lq0) {
   // ---- forward intermediates
   const T* q = in;
   const T psi = in[5];
@@ -313,6 +293,7 @@ __device__ __forceinline__ void local_fields_vjp(const Coef<T>& c, const T in[36
   for (int a = 0; a < 3; ++a) full3(in + 6 + 5 * a, dQ[a]);
   const T* dp = in + 26;
   const T* hp = in + 30;
+  const T third = T(1.0 / 3.0);
   const T chi = c.chi0 + c.chis * (T(1) + psi);
   T QQ[3][3];
 #pragma unroll
@@ -340,8 +321,8 @@ __device__ __forceinline__ void local_fields_vjp(const Coef<T>& c, const T in[36
   const T g2 = dp[0] * dp[0] + dp[1] * dp[1] + dp[2] * dp[2];
   const T Ac = c.A0 * chi;
   const T Kq = T(2) * c.K * c.q0;
-  const T lin = -c.A0 * (T(1) - chi / T(3)) - Ac * trQ2 - Kq * T(2) * c.q0;
-  const T iso = (Ac * trQ2 - c.W * g2) / T(3);
+  const T lin = -c.A0 * (T(1) - third * chi) - Ac * trQ2 - Kq * T(2) * c.q0;
+  const T iso = third * (Ac * trQ2 - c.W * g2);
   const int I5[5] = {0, 0, 0, 1, 1};
   const int J5[5] = {0, 1, 2, 1, 2};
   T H[5];
@@ -361,7 +342,7 @@ __device__ __forceinline__ void local_fields_vjp(const Coef<T>& c, const T in[36
   for (int b = 0; b < 3; ++b) divQdp += (dQ[0][0][b] + dQ[1][1][b] + dQ[2][2][b]) * dp[b];
   const T psi2 = psi * psi;
   const T mu = psi * (c.b * psi2 - c.a) - c.kphi * in[29] +
-               c.A0 * c.chis * (trQ2 * (T(0.25) * trQ2 - T(1) / T(6)) - trQ3 / T(3)) - T(2) * c.W * (divQdp + Qh);
+               c.A0 * c.chis * (trQ2 * (T(0.25) * trQ2 - T(1.0 / 6.0)) - third * trQ3) - T(2) * c.W * (divQdp + Qh);
   T Qdp[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) Qdp[i] = Q[i][0] * dp[0] + Q[i][1] * dp[1] + Q[i][2] * dp[2];
@@ -375,7 +356,7 @@ __device__ __forceinline__ void local_fields_vjp(const Coef<T>& c, const T in[36
   const T phic = T(0.5) * (T(1) + psi);
   const T trQH = QH[0][0] + QH[1][1] + QH[2][2];
   const T cQ = T(2) * c.xi * trQH - c.zeta * phic;
-  const T cH = -T(2) * c.xi / T(3);
+  const T cH = -c.xi23;
   const T cP = T(1) - c.xi, cM = -(T(1) + c.xi);
   T wv[3];
 #pragma unroll
@@ -436,7 +417,7 @@ __device__ __forceinline__ void local_fields_vjp(const Coef<T>& c, const T in[36
     lQdp[b] += T(2) * c.W * lwv[b];
   }
   // cQ = 2 xi trQH - zeta phic; cI = (2 xi/3) trQH - P0
-  ltrQH += T(2) * c.xi * lcQ + (T(2) * c.xi / T(3)) * lcI;
+  ltrQH += T(2) * c.xi * lcQ + c.xi23 * lcI;
   lzeta += -phic * lcQ;
   lphic += -c.zeta * lcQ;
   lP0 += -lcI;
@@ -459,9 +440,9 @@ __device__ __forceinline__ void local_fields_vjp(const Coef<T>& c, const T in[36
   // fden
   T lpsi2 = (T(0.5) * c.b * psi2 - T(0.5) * c.a) * lf;
   T lg2 = T(0.5) * c.kphi * lf;
-  T lchi = c.A0 * (-(T(0.5) / T(3)) * trQ2 - trQ3 / T(3) + trQ2 * trQ2 / T(4)) * lf;
-  T ltrQ2 = c.A0 * (T(0.5) * (T(1) - chi / T(3)) + chi / T(2) * trQ2) * lf + Kq * c.q0 * lf;
-  T ltrQ3 = -c.A0 * chi / T(3) * lf;
+  T lchi = c.A0 * (-T(0.5 / 3.0) * trQ2 - third * trQ3 + T(0.25) * trQ2 * trQ2) * lf;
+  T ltrQ2 = c.A0 * (T(0.5) * (T(1) - third * chi) + T(0.5) * chi * trQ2) * lf + Kq * c.q0 * lf;
+  T ltrQ3 = -c.A0 * third * chi * lf;
 #pragma unroll
   for (int a = 0; a < 3; ++a) lG[a][a] += T(0.5) * c.K * lf;
   lKq += QC * lf + c.q0 * trQ2 * lf;
@@ -496,24 +477,17 @@ __device__ __forceinline__ void local_fields_vjp(const Coef<T>& c, const T in[36
   // mu
   lpsi += (c.b * psi2 - c.a) * lmu;
   lpsi2 += psi * c.b * lmu;
-  T llapp = -c.kphi * lmu;
-  ltrQ2 += c.A0 * c.chis * (T(0.5) * trQ2 - T(1) / T(6)) * lmu;
-  ltrQ3 += -c.A0 * c.chis / T(3) * lmu;
+  lmu_out = lmu;
+  ltrQ2 += c.A0 * c.chis * (T(0.5) * trQ2 - T(1.0 / 6.0)) * lmu;
+  ltrQ3 += -c.A0chis * third * lmu;
   const T ldiv = -T(2) * c.W * lmu, lQh = -T(2) * c.W * lmu;
   // Qh
-  T lhp[6];
   lQ[0][0] += hp[0] * lQh;
   lQ[1][1] += hp[1] * lQh;
   lQ[2][2] += hp[2] * lQh;
   lQ[0][1] += T(2) * hp[3] * lQh;
   lQ[0][2] += T(2) * hp[4] * lQh;
   lQ[1][2] += T(2) * hp[5] * lQh;
-  lhp[0] = Q[0][0] * lQh;
-  lhp[1] = Q[1][1] * lQh;
-  lhp[2] = Q[2][2] * lQh;
-  lhp[3] = T(2) * Q[0][1] * lQh;
-  lhp[4] = T(2) * Q[0][2] * lQh;
-  lhp[5] = T(2) * Q[1][2] * lQh;
   // divQdp
 #pragma unroll
   for (int b = 0; b < 3; ++b) {
@@ -539,13 +513,12 @@ __device__ __forceinline__ void local_fields_vjp(const Coef<T>& c, const T in[36
         }
     }
   // H (outputs and the uses of Hf)
-  T lH[5];
   lH[0] = lo[0] + lHf[0][0] - lHf[2][2];
   lH[1] = lo[1] + lHf[0][1] + lHf[1][0];
   lH[2] = lo[2] + lHf[0][2] + lHf[2][0];
   lH[3] = lo[3] + lHf[1][1] - lHf[2][2];
   lH[4] = lo[4] + lHf[1][2] + lHf[2][1];
-  T llin = T(0), lAc = T(0), liso = T(0), llapq[5];
+  T llin = T(0), lAc = T(0), liso = T(0);
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
     const int i = I5[k], j = J5[k];
@@ -554,7 +527,6 @@ __device__ __forceinline__ void local_fields_vjp(const Coef<T>& c, const T in[36
     lQ[i][j] += lin * L;
     lAc += QQ[i][j] * L;
     lQQ[i][j] += Ac * L;
-    llapq[k] = c.K * L;
     lKq += -CC[i][j] * L;
     lCC[i][j] += -Kq * L;
     ldp[i] += -c.W * dp[j] * L;
@@ -562,10 +534,10 @@ __device__ __forceinline__ void local_fields_vjp(const Coef<T>& c, const T in[36
     if (i == j) liso += -L;
   }
   // iso, lin, Kq, Ac, g2
-  lAc += trQ2 / T(3) * liso;
-  ltrQ2 += Ac / T(3) * liso;
-  lg2 += -c.W / T(3) * liso;
-  lchi += (c.A0 / T(3)) * llin;
+  lAc += third * trQ2 * liso;
+  ltrQ2 += third * Ac * liso;
+  lg2 += -c.W * third * liso;
+  lchi += c.A0 * third * llin;
   lAc += -trQ2 * llin;
   ltrQ2 += -Ac * llin;
   lKq += -T(2) * c.q0 * llin;
@@ -637,181 +609,194 @@ __device__ __forceinline__ void local_fields_vjp(const Coef<T>& c, const T in[36
     out[6 + 5 * a + 4] = ldQ[a][1][2] + ldQ[a][2][1];
   }
 #pragma unroll
-  for (int k = 0; k < 5; ++k) out[21 + k] = llapq[k];
-#pragma unroll
-  for (int b = 0; b < 3; ++b) out[26 + b] = ldp[b];
-  out[29] = llapp;
-#pragma unroll
-  for (int k = 0; k < 6; ++k) out[30 + k] = lhp[k];
+  for (int b = 0; b < 3; ++b) out[21 + b] = ldp[b];
 }
 
 // ---------------------------------------------------------------- RK1
+// The site of a thread and its neighbour offsets; false past the last site.
+__device__ __forceinline__ bool adj_site(int nx, int ny, int nz, long long N, long long& s, Nbr& nb) {
+  s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= N) return false;
+  const unsigned r = (unsigned)s, t = r / (unsigned)nx;  // a box has at most 2^31 sites
+  nb = make_nbr((int)(r % (unsigned)nx), (int)(t % (unsigned)ny), (int)(t / (unsigned)ny), nx, ny, nz);
+  return true;
+}
+
 template <typename T, bool SHIFT>
 __global__ void __launch_bounds__(kAdjBlock) k_adj_update(AdjDesc<T> A) {
   const InstDesc<T>& I = A.I;
   const long long N = I.N;
-  const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= N) return;
-  const int nx = I.nx, ny = I.ny, nz = I.nz;
-  const int x = (int)(s % nx);
-  const long long t = s / nx;
-  const int y = (int)(t % ny), z = (int)(t / ny);
-  AdjAcc<T> acc;
-  acc.q_ = I.q_in; acc.ps = I.psi_in; acc.S = A.S; acc.u_ = I.u_in;
+  long long s;
+  GlobalAcc<T> acc;
+  if (!adj_site(I.nx, I.ny, I.nz, N, s, acc.nb)) return;
+  acc.q_ = I.q_in; acc.ps = I.psi_in; acc.u_ = I.u_in;
   acc.N = N;
-  acc.nb = make_nbr(x, y, z, nx, ny, nz);
-  // forward inputs of update_math, packed: F 0-2, lapmu 3, Wg 4-12, q0 13-17, qf 18-47,
-  // p0 48, pf 49-54, u0 55-57, uf 58-63, Hs 64-68, g 69-87
-  T in[88];
-  {
-    T F[3], lapmu, Wg[3][3], q0[5], p0, u0[3], uf[6];
-    gather_force<T>(acc, F);
-    lapmu = gather_lapmu<T>(acc);
-    gather_velocity<T>(acc, Wg, u0, uf);
-    for (int k = 0; k < 5; ++k) q0[k] = acc.q(k, 0, 0, 0);
-    p0 = acc.psi(0, 0, 0);
-    for (int a = 0; a < 3; ++a) in[a] = F[a];
-    in[3] = lapmu;
-    for (int a = 0; a < 3; ++a)
-      for (int b = 0; b < 3; ++b) in[4 + 3 * a + b] = Wg[a][b];
-    for (int k = 0; k < 5; ++k) in[13 + k] = q0[k];
+  T F[3], W[3][3], q0[5], qu[3][5], pf[6], u0[3], uf[6], g[19];
 #pragma unroll
-    for (int f = 0; f < 6; ++f) {
-      const int cx = lat_c(f + 1, 0), cy = lat_c(f + 1, 1), cz = lat_c(f + 1, 2);
-      for (int k = 0; k < 5; ++k) in[18 + 5 * f + k] = acc.q(k, cx, cy, cz);
-      in[49 + f] = acc.psi(cx, cy, cz);
-    }
-    in[48] = p0;
-    for (int a = 0; a < 3; ++a) in[55 + a] = u0[a];
-    for (int f = 0; f < 6; ++f) in[58 + f] = uf[f];
-    for (int k = 0; k < 5; ++k) in[64 + k] = I.H[k * N + s];
-    for (int i = 0; i < 19; ++i) in[69 + i] = I.g_in[i * N + acc.nb.off(-lat_c(i, 0), -lat_c(i, 1), -lat_c(i, 2))];
+  for (int a = 0; a < 3; ++a) F[a] = A.F[a * N + s];
+  gather_velocity<T>(acc, W, u0, uf);
+#pragma unroll
+  for (int k = 0; k < 5; ++k) q0[k] = ld(I.q_in + k * N + s);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int d = u0[a] > T(0) ? -1 : 1;
+    const long long o = acc.nb.off(a == 0 ? d : 0, a == 1 ? d : 0, a == 2 ? d : 0);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) qu[a][k] = ld(I.q_in + k * N + o);
   }
+#pragma unroll
+  for (int f = 0; f < 6; ++f) pf[f] = acc.psi(lat_c(f + 1, 0), lat_c(f + 1, 1), lat_c(f + 1, 2));
+  const T p0 = ld(I.psi_in + s);
+#pragma unroll
+  for (int i = 0; i < 19; ++i) g[i] = ld(I.g_in + i * N + acc.nb.off(-lat_c(i, 0), -lat_c(i, 1), -lat_c(i, 2)));
   // output cotangents: qn 0-4, pn 5, u 6-8, g 9-27
   T lo[28];
+#pragma unroll
   for (int k = 0; k < 5; ++k) lo[k] = A.lq[k * N + s];
   lo[5] = A.lp[s];
+#pragma unroll
   for (int a = 0; a < 3; ++a) lo[6 + a] = A.lu[a * N + s];
+#pragma unroll
   for (int i = 0; i < 19; ++i) lo[9 + i] = A.lg[i * N + s];
-  T ci[88];
-  update_math_vjp<T, SHIFT>(I.c, in, lo, ci);
-  for (int j = 0; j < 88; ++j) A.A[j * N + s] = ci[j];
+  T lF[3], lW[3][3], lq0[5], lp0, lu0[3], lm0, lj[3];
+  update_math_vjp<T, SHIFT>(I.c, F, W, q0, qu, p0, pf, u0, uf, g, lo, lF, lW, lq0, lp0, lu0, lm0, lj);
+  st_quad_at(A.A, s, lF[0], lF[1], lF[2], lm0);
+  st_quad_at(A.A + 4 * N, s, lj[0], lj[1], lj[2], T(0));
+#pragma unroll
+  for (int b = 0; b < 3; ++b) st_quad_at(A.A + (8 + 4 * b) * N, s, lW[0][b], lW[1][b], lW[2][b], T(0));
+#pragma unroll
+  for (int k = 0; k < 5; ++k) A.oq[k * N + s] = lq0[k];
+  A.op[s] = lp0;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) A.ou[a * N + s] = lu0[a];
 }
 
 // ---------------------------------------------------------------- RK2
-// Transposes of the stencils of gather_update and of the pull, gathered at site y.
-template <typename T>
-__global__ void __launch_bounds__(kAdjBlock) k_adj_spread(AdjDesc<T> A) {
-  const InstDesc<T>& I = A.I;
-  const long long N = I.N;
-  const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= N) return;
-  const int nx = I.nx, ny = I.ny, nz = I.nz;
-  const int x = (int)(s % nx);
-  const long long t = s / nx;
-  const int y = (int)(t % ny), z = (int)(t / ny);
-  const Nbr nb = make_nbr(x, y, z, nx, ny, nz);
-  const T* __restrict__ a = A.A;
-  // F_a(x) = sum_b sum_{i odd, c_ib != 0} sgn(c_ib) wt_i (sigma_ab(x + c_i) - sigma_ab(x - c_i))
-  T ls[9];
-  for (int k = 0; k < 9; ++k) ls[k] = T(0);
-  T lu[3] = {T(0), T(0), T(0)};
-#pragma unroll
-  for (int i = 1; i < 19; i += 2) {
-    const int cx = lat_c(i, 0), cy = lat_c(i, 1), cz = lat_c(i, 2);
-    const T wt = lat_c2(i) == 1 ? T(2.0 / 12.0) : T(1.0 / 12.0);
-    const long long m = nb.off(-cx, -cy, -cz);  // y - c_i
-    const long long p = nb.off(cx, cy, cz);     // y + c_i
-    const int cc[3] = {cx, cy, cz};
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      if (cc[b] == 0) continue;
-      const T w = cc[b] > 0 ? wt : -wt;
-#pragma unroll
-      for (int aa = 0; aa < 3; ++aa) {
-        ls[3 * aa + b] += w * (a[aa * N + m] - a[aa * N + p]);                       // F
-        lu[aa] += w * (a[(4 + 3 * aa + b) * N + m] - a[(4 + 3 * aa + b) * N + p]);  // grad u
-      }
-    }
-  }
-  // lap mu(x) = sum_i lw_i mu(x + c_i) - 4 mu(x): symmetric
-  T lmu = -T(4) * a[3 * N + s];
-#pragma unroll
-  for (int i = 1; i < 19; ++i) {
-    const T lw = lat_c2(i) == 1 ? T(1.0 / 3.0) : T(1.0 / 6.0);
-    lmu += lw * a[3 * N + nb.off(-lat_c(i, 0), -lat_c(i, 1), -lat_c(i, 2))];
-  }
-  for (int k = 0; k < 9; ++k) A.ls[k * N + s] = ls[k];
-  A.ls[9 * N + s] = lmu;
-  for (int k = 0; k < 5; ++k) A.ls[(10 + k) * N + s] = a[(64 + k) * N + s];
-  // face reads: qf[f](x) = q(x + c_{f+1}), uf[2a](x) = u_a(x + e_a), uf[2a+1](x) = u_a(x - e_a)
-  T lq[5], lp = a[48 * N + s];
-  for (int k = 0; k < 5; ++k) lq[k] = a[(13 + k) * N + s];
-#pragma unroll
-  for (int f = 0; f < 6; ++f) {
-    const int i = f + 1;
-    const long long m = nb.off(-lat_c(i, 0), -lat_c(i, 1), -lat_c(i, 2));
-#pragma unroll
-    for (int k = 0; k < 5; ++k) lq[k] += a[(18 + 5 * f + k) * N + m];
-    lp += a[(49 + f) * N + m];
-  }
-#pragma unroll
-  for (int aa = 0; aa < 3; ++aa) {
-    lu[aa] += a[(55 + aa) * N + s];
-    const int ip = 1 + 2 * aa, im = 2 + 2 * aa;  // +e_a, -e_a
-    lu[aa] += a[(58 + 2 * aa) * N + nb.off(-lat_c(ip, 0), -lat_c(ip, 1), -lat_c(ip, 2))];
-    lu[aa] += a[(59 + 2 * aa) * N + nb.off(-lat_c(im, 0), -lat_c(im, 1), -lat_c(im, 2))];
-  }
-  for (int k = 0; k < 5; ++k) A.oq[k * N + s] = lq[k];
-  A.op[s] = lp;
-  for (int aa = 0; aa < 3; ++aa) A.ou[aa * N + s] = lu[aa];
-  // pull: g[i](x) = g*_i(x - c_i)  =>  lam g*_i(y) = lam g[i](y + c_i)
-#pragma unroll
-  for (int i = 0; i < 19; ++i) A.og[i * N + s] = a[(69 + i) * N + nb.off(lat_c(i, 0), lat_c(i, 1), lat_c(i, 2))];
-}
-
-// ---------------------------------------------------------------- RK3
-// Inputs of local_fields, packed: q0 0-4, p0 5, dq 6-20 (a*5 + k), lapq 21-25, dp 26-28,
-// lapp 29, hp 30-35; two more tangent directions: zeta (36), q0 parameter (37).
+// Transposes of the stencils of the update and of the pull, gathered at the site, then the VJP of local_fields there
+// (its inputs packed: q0 0-4, p0 5, dq 6-20 (a*5 + k), lapq 21-25, dp 26-28, lapp 29, hp 30-35).
 template <typename T>
 __global__ void __launch_bounds__(kAdjBlock) k_adj_fields(AdjDesc<T> A) {
   const InstDesc<T>& I = A.I;
   const long long N = I.N;
-  const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   double pz = 0.0, pq = 0.0;
-  if (s < N) {
-    const int nx = I.nx, ny = I.ny, nz = I.nz;
-    const int x = (int)(s % nx);
-    const long long t = s / nx;
-    const int y = (int)(t % ny), z = (int)(t / ny);
-    GlobalAcc<T> acc;
+  long long s;
+  GlobalAcc<T> acc;
+  if (adj_site(I.nx, I.ny, I.nz, N, s, acc.nb)) {
     acc.q_ = I.q_in; acc.ps = I.psi_in; acc.N = N;
-    acc.nb = make_nbr(x, y, z, nx, ny, nz);
+    const Nbr& nb = acc.nb;
+    const Coef<T>& c = I.c;
+    // pull: g[i](x) = g*_i(x - c_i)  =>  lam g*_i(y) = lam g[i](y + c_i).  F_a(x) = sum_b sum_{i odd, c_ib != 0}
+    // sgn(c_ib) wt_i (sigma_ab(x + c_i) - sigma_ab(x - c_i)), and grad u the same, so both transposes take
+    // the difference of the values at y - c_i and y + c_i.
+    T ls[9], lu[3];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) ls[k] = T(0);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) lu[a] = A.ou[a * N + s];
+    {
+      const Quad<T> f = ld_quad(A.A, s);
+      A.og[s] = c.omc * ld(A.lg + s) + f.w;
+    }
+#pragma unroll
+    for (int i = 1; i < 19; i += 2) {
+      const int cx = lat_c(i, 0), cy = lat_c(i, 1), cz = lat_c(i, 2);
+      const T wt = lat_c2(i) == 1 ? T(2.0 / 12.0) : T(1.0 / 12.0);
+      const long long m = nb.off(-cx, -cy, -cz), p = nb.off(cx, cy, cz);
+      const Quad<T> fm = ld_quad(A.A, m), fp = ld_quad(A.A, p);
+      const Quad<T> jm = ld_quad(A.A + 4 * N, m), jp = ld_quad(A.A + 4 * N, p);
+      A.og[i * N + s] = c.omc * ld(A.lg + i * N + p) + fp.w + (T(cx) * jp.x + T(cy) * jp.y + T(cz) * jp.z);
+      A.og[(i + 1) * N + s] = c.omc * ld(A.lg + (i + 1) * N + m) + fm.w - (T(cx) * jm.x + T(cy) * jm.y + T(cz) * jm.z);
+      const T df[3] = {fm.x - fp.x, fm.y - fp.y, fm.z - fp.z};
+      const int cc[3] = {cx, cy, cz};
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        if (cc[b] == 0) continue;
+        const T w = cc[b] > 0 ? wt : -wt;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) ls[3 * a + b] += w * df[a];
+        const Quad<T> wm = ld_quad(A.A + (8 + 4 * b) * N, m), wp = ld_quad(A.A + (8 + 4 * b) * N, p);
+        lu[0] += w * (wm.x - wp.x);
+        lu[1] += w * (wm.y - wp.y);
+        lu[2] += w * (wm.z - wp.z);
+      }
+    }
+    // lap mu(x) = sum_i lw_i mu(x + c_i) - 4 mu(x): symmetric; its cotangent is M lam_psi
+    const T lpc = ld(A.lp + s);
+    T lmu = -T(4) * lpc;
+#pragma unroll
+    for (int i = 1; i < 19; ++i)
+      lmu += (lat_c2(i) == 1 ? T(1.0 / 3.0) : T(1.0 / 6.0)) * ld(A.lp + nb.off(-lat_c(i, 0), -lat_c(i, 1), -lat_c(i, 2)));
+    lmu *= c.M;
+    // face reads of the sites at y - e_a (their upper face) and y + e_a (their lower face)
+    T lq[5], lp = A.op[s], lqc[5];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      lq[k] = A.oq[k * N + s];
+      lqc[k] = ld(A.lq + k * N + s);
+    }
+    const T p0 = ld(I.psi_in + s);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const int ex = a == 0, ey = a == 1, ez = a == 2;
+      const long long m = nb.off(-ex, -ey, -ez), p = nb.off(ex, ey, ez);
+      const T uc = ld(I.u_in + a * N + s), um = ld(I.u_in + a * N + m), up = ld(I.u_in + a * N + p);
+      // Q: the site below takes this one as its upwind neighbour if its velocity is negative, the one above if positive
+      const T wm = um < T(0) ? -um : T(0), wp = up > T(0) ? up : T(0);
+#pragma unroll
+      for (int k = 0; k < 5; ++k) lq[k] += wm * ld(A.lq + k * N + m) + wp * ld(A.lq + k * N + p);
+      // psi fluxes: upper face of the site below, cotangent -lam_psi; lower face of the site above, +lam_psi
+      const T lm = -ld(A.lp + m), lpp = ld(A.lp + p);
+      const T ubp = T(0.5) * (um + uc), ubm = T(0.5) * (uc + up);
+      if (!(ubp > T(0))) lp += ubp * lm;
+      if (ubm > T(0)) lp += ubm * lpp;
+      lu[a] += T(0.5) * ((ubp > T(0) ? ld(I.psi_in + m) : p0) * lm + (ubm > T(0) ? p0 : ld(I.psi_in + p)) * lpp);
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) A.ou[a * N + s] = lu[a];
+    // local_fields
     T in[36];
     {
-      T q0[5], p0, dq[3][5], lapq[5], dp[3], lapp, hp[6];
-      gather_fields<T>(acc, q0, p0, dq, lapq, dp, lapp, hp);
+      T q0[5], pc, dq[3][5], lapq[5], dp[3], lapp, hp[6];
+      gather_fields<T>(acc, q0, pc, dq, lapq, dp, lapp, hp);
+#pragma unroll
       for (int k = 0; k < 5; ++k) in[k] = q0[k];
-      in[5] = p0;
+      in[5] = pc;
+#pragma unroll
       for (int a = 0; a < 3; ++a)
+#pragma unroll
         for (int k = 0; k < 5; ++k) in[6 + 5 * a + k] = dq[a][k];
+#pragma unroll
       for (int k = 0; k < 5; ++k) in[21 + k] = lapq[k];
+#pragma unroll
       for (int a = 0; a < 3; ++a) in[26 + a] = dp[a];
       in[29] = lapp;
+#pragma unroll
       for (int k = 0; k < 6; ++k) in[30 + k] = hp[k];
     }
     // output cotangents: H 0-4, mu 5, sigma 6-14
     T lo[15];
-    for (int k = 0; k < 5; ++k) lo[k] = A.ls[(10 + k) * N + s];
-    lo[5] = A.ls[9 * N + s];
-    for (int k = 0; k < 9; ++k) lo[6 + k] = A.ls[k * N + s];
-    T ci[36], lz, lq;
-    local_fields_vjp<T>(I.c, in, lo, ci, lz, lq);
-    for (int j = 0; j < 36; ++j) A.Bf[j * N + s] = ci[j];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) lo[k] = c.gammaQ * lqc[k];
+    lo[5] = lmu;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) lo[6 + k] = ls[k];
+    T ci[24], lH[5], lmo, lz, lq0;
+    local_fields_vjp<T>(c, in, lo, ci, lH, lmo, lz, lq0);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) A.oq[k * N + s] = lq[k] + ci[k];
+    A.op[s] = lp + ci[5];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      st_quad_at(A.B + 4 * a * N, s, ci[6 + 5 * a], ci[7 + 5 * a], ci[8 + 5 * a], ci[9 + 5 * a]);
+      st_pair_at(A.B + (16 + 2 * a) * N, s, ci[10 + 5 * a], ci[21 + a]);
+    }
+    st_quad_at(A.B + 12 * N, s, lH[0], lH[1], lH[2], lH[3]);
+    st_pair_at(A.B + 22 * N, s, lH[4], lmo);
     pz = (double)lz;
-    pq = (double)lq;
+    pq = (double)lq0;
   }
-  // per-block FP64 sums of the parameter gradients (fixed order: deterministic)
+  // per-block FP64 sums of the parameter gradients (fixed order: deterministic), added to the block's own over the
+  // reverse steps; one pass over the blocks at the end sums them
   __shared__ double sh[2][kAdjBlock / 32];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -821,34 +806,42 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_fields(AdjDesc<T> A) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   if (lane == 0) { sh[0][wid] = pz; sh[1][wid] = pq; }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double a0 = 0.0, a1 = 0.0;
-    for (int w = 0; w < kAdjBlock / 32; ++w) { a0 += sh[0][w]; a1 += sh[1][w]; }
-    A.pgrad[2 * blockIdx.x] = a0;
-    A.pgrad[2 * blockIdx.x + 1] = a1;
+  if (threadIdx.x < 2) {
+    double a0 = 0.0;
+    for (int w = 0; w < kAdjBlock / 32; ++w) a0 += sh[threadIdx.x][w];
+    A.pgrad[2 * blockIdx.x + threadIdx.x] += a0;
   }
 }
 
-// ---------------------------------------------------------------- RK4
+// ---------------------------------------------------------------- RK3
 // Transposes of gather_fields, added to the partial cotangents of Q and psi:
 //   d_a f(x) = sum_i 3 w_i c_ia f(x + c_i),  lap f(x) = sum_i lw_i f(x + c_i) - 4 f(x),
 //   hess_aa f(x) = f(x + e_a) + f(x - e_a) - 2 f(x),
-//   hess_ab f(x) = 1/4 sum_{edges in the ab plane} c_a c_b f(x + c).
+//   hess_ab f(x) = 1/4 sum_{edges in the ab plane} c_a c_b f(x + c),
+// with the cotangents K lH of lap Q, -kphi lmu of lap psi and -2 W lmu (Q_aa; 2 Q_ab) of the Hessian.
 template <typename T>
 __global__ void __launch_bounds__(kAdjBlock) k_adj_gather(AdjDesc<T> A) {
   const InstDesc<T>& I = A.I;
   const long long N = I.N;
-  const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= N) return;
-  const int nx = I.nx, ny = I.ny, nz = I.nz;
-  const int x = (int)(s % nx);
-  const long long t = s / nx;
-  const int y = (int)(t % ny), z = (int)(t / ny);
-  const Nbr nb = make_nbr(x, y, z, nx, ny, nz);
-  const T* __restrict__ b = A.Bf;
-  T lq[5], lp;
-  for (int k = 0; k < 5; ++k) lq[k] = b[k * N + s] - T(4) * b[(21 + k) * N + s];
-  lp = b[5 * N + s] - T(4) * b[29 * N + s] - T(2) * (b[30 * N + s] + b[31 * N + s] + b[32 * N + s]);
+  long long s;
+  Nbr nb;
+  if (!adj_site(I.nx, I.ny, I.nz, N, s, nb)) return;
+  const Coef<T>& c = I.c;
+  const T* __restrict__ q = I.q_in;
+  T dq[5], lapH[5], dps = T(0), lapm, hess;
+  {
+    const Quad<T> h = ld_quad(A.B + 12 * N, s);
+    const Vec2<T> h4 = ld_pair(A.B + 22 * N, s);
+    lapH[0] = -T(4) * h.x;
+    lapH[1] = -T(4) * h.y;
+    lapH[2] = -T(4) * h.z;
+    lapH[3] = -T(4) * h.w;
+    lapH[4] = -T(4) * h4.x;
+    lapm = -T(4) * h4.y;
+    hess = T(0);  // -2 (Q_xx + Q_yy + Q_zz) lmu = 0: Q is traceless
+  }
+#pragma unroll
+  for (int k = 0; k < 5; ++k) dq[k] = T(0);
 #pragma unroll
   for (int i = 1; i < 19; ++i) {
     const int cx = lat_c(i, 0), cy = lat_c(i, 1), cz = lat_c(i, 2);
@@ -861,24 +854,34 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_gather(AdjDesc<T> A) {
     for (int a = 0; a < 3; ++a) {
       if (cc[a] == 0) continue;
       const T w = cc[a] > 0 ? gw : -gw;
-#pragma unroll
-      for (int k = 0; k < 5; ++k) lq[k] += w * b[(6 + 5 * a + k) * N + m];
-      lp += w * b[(26 + a) * N + m];
+      const Quad<T> d = ld_quad(A.B + 4 * a * N, m);
+      const Vec2<T> e = ld_pair(A.B + (16 + 2 * a) * N, m);
+      dq[0] += w * d.x;
+      dq[1] += w * d.y;
+      dq[2] += w * d.z;
+      dq[3] += w * d.w;
+      dq[4] += w * e.x;
+      dps += w * e.y;
     }
-#pragma unroll
-    for (int k = 0; k < 5; ++k) lq[k] += lw * b[(21 + k) * N + m];
-    lp += lw * b[29 * N + m];
+    const Quad<T> h = ld_quad(A.B + 12 * N, m);
+    const Vec2<T> h4 = ld_pair(A.B + 22 * N, m);
+    lapH[0] += lw * h.x;
+    lapH[1] += lw * h.y;
+    lapH[2] += lw * h.z;
+    lapH[3] += lw * h.w;
+    lapH[4] += lw * h4.x;
+    lapm += lw * h4.y;
     if (face) {
-      const int a = cx ? 0 : (cy ? 1 : 2);
-      lp += b[(30 + a) * N + m];
+      const T Qaa = cx ? ld(q + m) : (cy ? ld(q + 3 * N + m) : -ld(q + m) - ld(q + 3 * N + m));
+      hess += Qaa * h4.y;
     } else {
-      const T sgn = T(0.25) * T(cx * cy + cx * cz + cy * cz);
-      const int k = (cz == 0) ? 3 : (cy == 0 ? 4 : 5);
-      lp += sgn * b[(30 + k) * N + m];
+      const int k = cz == 0 ? 1 : (cy == 0 ? 2 : 4);  // Q_xy, Q_xz, Q_yz
+      hess += (T(0.5) * T(cx * cy + cx * cz + cy * cz)) * (ld(q + k * N + m) * h4.y);
     }
   }
-  for (int k = 0; k < 5; ++k) A.oq[k * N + s] += lq[k];
-  A.op[s] += lp;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) A.oq[k * N + s] += dq[k] + c.K * lapH[k];
+  A.op[s] += dps - c.kphi * lapm - c.W2 * hess;
 }
 
 // ---------------------------------------------------------------- objective seed
@@ -946,14 +949,13 @@ template <typename T, bool SHIFT>
 cudaError_t LaunchAdj<T, SHIFT>::reverse_step(const AdjDescHost<T>& h, cudaStream_t s) {
   AdjDesc<T> A;
   A.I = h.I;
-  A.S = h.S;
+  A.F = h.F;
   A.lg = h.lg; A.lq = h.lq; A.lp = h.lp; A.lu = h.lu;
-  A.A = h.A; A.Bf = h.Bf; A.ls = h.ls;
+  A.A = h.A; A.B = h.B;
   A.og = h.og; A.oq = h.oq; A.op = h.op; A.ou = h.ou;
   A.pgrad = h.pgrad;
   const unsigned nb = (unsigned)((h.I.N + kAdjBlock - 1) / kAdjBlock);
   k_adj_update<T, SHIFT><<<nb, kAdjBlock, 0, s>>>(A);
-  k_adj_spread<T><<<nb, kAdjBlock, 0, s>>>(A);
   k_adj_fields<T><<<nb, kAdjBlock, 0, s>>>(A);
   k_adj_gather<T><<<nb, kAdjBlock, 0, s>>>(A);
   return cudaGetLastError();

@@ -125,6 +125,7 @@ struct MarchDesc {
   T* u_out[3];
   T* S[6];             // scratch of the default path: arrays of pairs [N][2] (see PairPlane in lbcad_march.cuh)
   T* H[5];             // sync coupling, Heun: H at t
+  T* F[3];             // replay of the adjoint: force
   T* rq[6];            // Heun: right-hand side at t, predicted state (Q, psi), H and mu there
   T* qp[6];
   T* Hp[6];
@@ -173,8 +174,8 @@ struct StepWork {
 };
 
 // What k_march_lb does: collision and psi (kFusedPlain), with the a6 sums (kFusedSums), or the collision
-// alone (kFusedLbOnly: sync coupling, Heun).
-constexpr int kFusedPlain = 0, kFusedSums = 1, kFusedLbOnly = 2;
+// alone (kFusedLbOnly: sync coupling, Heun); kFusedForce: kFusedPlain, and the force is written (replay of the adjoint).
+constexpr int kFusedPlain = 0, kFusedSums = 1, kFusedLbOnly = 2, kFusedForce = 3;
 
 // The FP64 conserved and centroid sums of the step (a6).  Each run of items of one instance that a block works
 // on has a slot of 12 partial sums (block b, run j of the block: slot b * maxrun + j);
@@ -209,22 +210,23 @@ struct LaunchFused {
   // (Euler), or predictor, fields at the predicted state and corrector (Heun).
   static cudaError_t split_step(int variant, int k, const StepWork& w, bool heun, bool sync, const MarchDesc<T>* d,
                                 cudaStream_t s);
-  // The adjoint's replay: one Euler step of D3Q19 with the body force that also leaves S and H of the state it
-  // steps from; last: S and H only.
+  // The adjoint's replay: one Euler step of D3Q19 with the body force, without the sums, that also leaves its
+  // force (MarchDesc::F).
   static cudaError_t prepare_replay(int k);
-  static cudaError_t replay(int k, const StepWork& w, bool last, const MarchDesc<T>* d, cudaStream_t s);
+  static cudaError_t replay(int k, const StepWork& w, const MarchDesc<T>* d, cudaStream_t s);
 };
 
 // Buffers of one reverse step of the adjoint (lbcad_adjoint.cuh).
 template <typename T>
 struct AdjDescHost {
-  InstDesc<T> I;                 // state s_t (inputs) and its H
-  const T* S;                    // its stress and mu: arrays of pairs [6][N][2] (see PairPlane in lbcad_march.cuh)
+  InstDesc<T> I;                 // state s_t (inputs)
+  const T* F;                    // force of the step from it [3][N]
   const T *lg, *lq, *lp, *lu;    // cotangent of s_{t+1}
-  T *A, *Bf, *ls;                // work: 88 + 36 + 15 values per site
+  T *A, *B;                      // work: kAdjWorkA and kAdjWorkB values per site
   T *og, *oq, *op, *ou;          // cotangent of s_t
-  double* pgrad;                 // per-block partial d/dzeta, d/dq0
+  double* pgrad;                 // per-block sums over the reverse steps of d/dzeta, d/dq0
 };
+constexpr int kAdjWorkA = 20, kAdjWorkB = 24;
 
 template <typename T, bool SHIFT>
 struct LaunchAdj {

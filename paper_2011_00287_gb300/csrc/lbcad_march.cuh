@@ -182,23 +182,23 @@ __host__ __device__ constexpr int blocks_for(int threads, int regs) {
 }
 
 // ---------------------------------------------------------------- fields
-constexpr int kMarchOp = 0, kMarchH = 1, kMarchPred = 2, kMarchOpH = 3;
+constexpr int kMarchOp = 0, kMarchH = 1, kMarchPred = 2;
 
 template <typename T, class G, int MODE>
 struct FieldsSmem {
   static constexpr int NSLOT = 4;  // planes p-2 (faces below), p-1, p, and the arriving one
-  static constexpr int QSL = 6 * G::SP, USL = MODE == kMarchOp || MODE == kMarchOpH ? 3 * G::SP : 0;
+  static constexpr int QSL = 6 * G::SP, USL = MODE == kMarchOp ? 3 * G::SP : 0;
   static constexpr size_t bytes = (size_t)NSLOT * (QSL + USL) * sizeof(T);
 };
 
 // kMarchOp: sigma, mu, the flux divergence and psi of every site into the scratch pairs and the new Q
 // (Euler with the velocity of the previous step).  kMarchH: sigma and mu into the pairs, H into its
-// scratch (sync coupling, Heun).  kMarchOpH: both (replay of the adjoint).  kMarchPred: H and mu of the Heun predicted state qp into the sigma
+// scratch (sync coupling, Heun).  kMarchPred: H and mu of the Heun predicted state qp into the sigma
 // scratch (H at sig[0..5N), mu at sig[5N..6N)).
 template <typename T, int MI, int TX, int TY, int MODE>
 __global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? blocks_for(TX * TY, TX * TY > 128 ? 128 : 168) : 1)
     k_march_fields(const __grid_constant__ InstPack<T, MI> P, const MarchItem* __restrict__ items, int nitems) {
-  constexpr bool OP = MODE == kMarchOp || MODE == kMarchOpH, WH = MODE == kMarchH || MODE == kMarchOpH;
+  constexpr bool OP = MODE == kMarchOp, WH = MODE == kMarchH;
   using G = Tile<TX, TY>;
   using M = FieldsSmem<T, G, MODE>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -604,6 +604,10 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? blocks_for(TX * TY, 
           for (int i = 0; i < V::Q; ++i) st_out(comp(go, i, I.N), g[i]);
 #pragma unroll
           for (int a = 0; a < 3; ++a) st_out(comp(uo, a, I.N), u[a]);
+          if constexpr (MODE == kFusedForce) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) st_out(I.F[a] + s, F[a]);
+          }
           if constexpr (MODE != kFusedLbOnly) {
             const Vec2<T> dp = cp.spair(5, 0, 0);  // flux divergence, psi
             const T pn = dp.y + fma(cf.M, lapmu, -dp.x);
@@ -891,22 +895,15 @@ struct MarchShape {
     op<MI, 2>(P, w.op[1], sync, s);
     return cudaGetLastError();
   }
-  // One replayed step of the adjoint: the Euler step without the sums, leaving S and H of the state it steps from;
-  // last: S and H only.
+  // One replayed step of the adjoint: the Euler step without the sums, leaving its force too.
   static cudaError_t prepare_replay() {
     int n = 0;
-    cudaError_t e = prepare_kernel(k_march_fields<T, 1, FX, FY, kMarchOpH>, FG::NT, fields_smem<kMarchOpH>(), &n);
-    if (e == cudaSuccess) e = prepare_kernel(k_march_fields<T, 1, FX, FY, kMarchH>, FG::NT, fields_smem<kMarchH>(), &n);
-    return e;
+    return prepare_kernel(k_march_lb<T, SHIFT, 1, LX, LY, V, FORM, kFusedForce>, G::NT, lb_smem<kFusedForce>(), &n);
   }
-  static cudaError_t replay(const StepWork& w, bool last, const MarchDesc<T>* d, cudaStream_t s) {
+  static cudaError_t replay(const StepWork& w, const MarchDesc<T>* d, cudaStream_t s) {
     const InstPack<T, 1> P = pack<1>(w, d);
-    if (last) {
-      fields<1, kMarchH>(P, w.fields, s);
-    } else {
-      fields<1, kMarchOpH>(P, w.fields, s);
-      lb<1, kFusedPlain>(P, w.lb, FusedObs{}, s);
-    }
+    fields<1, kMarchOp>(P, w.fields, s);
+    lb<1, kFusedForce>(P, w.lb, FusedObs{}, s);
     return cudaGetLastError();
   }
   static cudaError_t split(const StepWork& w, bool heun, bool sync, const MarchDesc<T>* d, cudaStream_t s) {
@@ -974,9 +971,9 @@ cudaError_t LaunchFused<T, SHIFT>::prepare_replay(int k) {
 }
 
 template <typename T, bool SHIFT>
-cudaError_t LaunchFused<T, SHIFT>::replay(int k, const StepWork& w, bool last, const MarchDesc<T>* d, cudaStream_t s) {
+cudaError_t LaunchFused<T, SHIFT>::replay(int k, const StepWork& w, const MarchDesc<T>* d, cudaStream_t s) {
   return with_variant<T, SHIFT>(0, k, false, [&](auto sh) {
-    if constexpr (decltype(sh)::kDefaultLb) return decltype(sh)::replay(w, last, d, s);
+    if constexpr (decltype(sh)::kDefaultLb) return decltype(sh)::replay(w, d, s);
     else return cudaErrorNotSupported;
   });
 }

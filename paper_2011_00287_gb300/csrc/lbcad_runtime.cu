@@ -1045,9 +1045,9 @@ StateBuf<T> state_at(T* base, long long N) {
   return StateBuf<T>{base, base + 19 * N, base + 24 * N, base + 25 * N};
 }
 
-// Descriptor of one replayed step: from state `in` to `out`, S and H of `in` at `f` (12 and 5 values per site).
+// Descriptor of one replayed step: from state `in` to `out`, its force to F (3 values per site).
 template <typename T>
-MarchDesc<T> replay_desc(const MarchDesc<T>& base, long long N, const StateBuf<T>& in, const StateBuf<T>& out, T* f) {
+MarchDesc<T> replay_desc(const MarchDesc<T>& base, long long N, const StateBuf<T>& in, const StateBuf<T>& out, T* F) {
   MarchDesc<T> d = base;
   for (int i = 0; i < 19; ++i) {
     d.g_in[i] = in.g + i * N;
@@ -1056,13 +1056,12 @@ MarchDesc<T> replay_desc(const MarchDesc<T>& base, long long N, const StateBuf<T
   for (int k = 0; k < 5; ++k) {
     d.q_in[k] = in.q + k * N;
     d.q_out[k] = out.q + k * N;
-    d.H[k] = f + (12 + k) * N;
   }
   for (int a = 0; a < 3; ++a) {
     d.u_in[a] = in.u + a * N;
     d.u_out[a] = out.u + a * N;
+    d.F[a] = F + a * N;
   }
-  for (int j = 0; j < 6; ++j) d.S[j] = f + 2 * j * N;
   d.psi_in = in.p;
   d.psi_out = out.p;
   return d;
@@ -1084,22 +1083,21 @@ int adjoint_impl(lbcad_ctx* c, int64_t nsteps, int k, double* dzeta, double* dq0
   const long long N = I.N;
   const int S = (int)((nsteps + k - 1) / k);
   const size_t st = 28 * (size_t)N;  // elements of one stored state
-  const size_t fs = 17 * (size_t)N;  // elements of one state's stress pairs (12) and H (5)
+  const size_t fs = 3 * (size_t)N;   // elements of one step's force
   // buffers through the context's allocator, kept for the next call
   c->adj_lam = nullptr;
   T* ck = (T*)adj_buffer(c, 0, (size_t)S * st * sizeof(T));
-  T* seg = (T*)adj_buffer(c, 1, (size_t)k * st * sizeof(T));
+  T* seg = (T*)adj_buffer(c, 1, (size_t)(k + 1) * st * sizeof(T));
   T* lam = (T*)adj_buffer(c, 2, 2 * st * sizeof(T));
-  T* work = (T*)adj_buffer(c, 3, (88 + 36 + 15) * (size_t)N * sizeof(T));
+  T* work = (T*)adj_buffer(c, 3, (kAdjWorkA + kAdjWorkB) * (size_t)N * sizeof(T));
   T* fl = (T*)adj_buffer(c, 4, (size_t)k * fs * sizeof(T));
   const int nb = LaunchAdj<T, SHIFT>::blocks(N);
   double* pg = (double*)adj_buffer(c, 5, (2 * (size_t)nb + 2) * sizeof(double));
   if (!ck || !seg || !lam || !work || !fl || !pg) return fail(c, LBCAD_E_OOM, "adjoint buffers");
   T* A = work;
-  T* Bf = A + 88 * N;
-  T* ls = Bf + 36 * N;
+  T* B = A + kAdjWorkA * N;
   double* total = pg + 2 * nb;
-  CK(c, cudaMemsetAsync(total, 0, 2 * sizeof(double), c->stream));
+  CK(c, cudaMemsetAsync(pg, 0, (2 * (size_t)nb + 2) * sizeof(double), c->stream));
   using Step = LaunchFused<T, SHIFT>;
   CK(c, Step::prepare_replay(c->cfg_index));
   const MarchDesc<T> base = make_march_desc<T>(I, 0, SHIFT);
@@ -1142,41 +1140,35 @@ int adjoint_impl(lbcad_ctx* c, int64_t nsteps, int k, double* dzeta, double* dq0
   cudaError_t e = LaunchAdj<T, SHIFT>::seed(desc_now<T>(c, 0), dX, ks, kc, lcur.p, c->stream);
   if (e != cudaSuccess) return fail(c, LBCAD_E_CUDA, std::string("adjoint seed: ") + cudaGetErrorString(e));
 
-  std::vector<InstDesc<T>> hd(k);  // state j of the segment and its H
   for (int sgi = S - 1; sgi >= 0; --sgi) {
     const int len = (int)std::min<int64_t>(k, nsteps - (int64_t)sgi * k);
-    // replay the segment: states 0 .. len-1 of this segment into seg (state 0 = checkpoint), by the kernels of
-    // the step, so that the replayed states are the forward's
+    // replay the segment: states 0 .. len of this segment into seg (state 0 = checkpoint), by the kernels of
+    // the step, so that the replayed states are the forward's, and the force of each step into fl
     CK(c, cudaMemcpyAsync(seg, ck + (size_t)sgi * st, st * sizeof(T), cudaMemcpyDeviceToDevice, c->stream));
-    // state j's stress, mu and H go to its own slice of fl: the replay step that leaves state j
-    // computes them, and its reverse step reads them there
     for (int j = 0; j < len; ++j) {
-      const bool last = j + 1 == len;
-      const StateBuf<T> in = state_at<T>(seg + (size_t)j * st, N);
-      const StateBuf<T> out = state_at<T>(seg + (size_t)(last ? j : j + 1) * st, N);
-      T* f = fl + (size_t)j * fs;
-      hd[j] = make_desc<T>(I, 0);
-      hd[j].g_in = in.g; hd[j].q_in = in.q; hd[j].psi_in = in.p; hd[j].u_in = in.u;
-      hd[j].H = f + 12 * N;
-      const MarchDesc<T> md = replay_desc<T>(base, N, in, out, f);
-      e = Step::replay(c->cfg_index, c->work[0], last, &md, c->stream);
+      const MarchDesc<T> md = replay_desc<T>(base, N, state_at<T>(seg + (size_t)j * st, N),
+                                             state_at<T>(seg + (size_t)(j + 1) * st, N), fl + (size_t)j * fs);
+      e = Step::replay(c->cfg_index, c->work[0], &md, c->stream);
       if (e != cudaSuccess) return fail(c, LBCAD_E_CUDA, std::string("adjoint replay: ") + cudaGetErrorString(e));
     }
     // reverse steps
     for (int j = len - 1; j >= 0; --j) {
+      const StateBuf<T> in = state_at<T>(seg + (size_t)j * st, N);
       AdjDescHost<T> h;
-      h.I = hd[j];
-      h.S = fl + (size_t)j * fs;
+      h.I = make_desc<T>(I, 0);
+      h.I.g_in = in.g; h.I.q_in = in.q; h.I.psi_in = in.p; h.I.u_in = in.u;
+      h.F = fl + (size_t)j * fs;
       h.lg = lcur.g; h.lq = lcur.q; h.lp = lcur.p; h.lu = lcur.u;
-      h.A = A; h.Bf = Bf; h.ls = ls;
+      h.A = A; h.B = B;
       h.og = lnxt.g; h.oq = lnxt.q; h.op = lnxt.p; h.ou = lnxt.u;
       h.pgrad = pg;
       e = LaunchAdj<T, SHIFT>::reverse_step(h, c->stream);
-      if (e == cudaSuccess) e = adj_accumulate(pg, nb, total, c->stream);
       if (e != cudaSuccess) return fail(c, LBCAD_E_CUDA, std::string("adjoint reverse step: ") + cudaGetErrorString(e));
       std::swap(lcur, lnxt);
     }
   }
+  e = adj_accumulate(pg, nb, total, c->stream);
+  if (e != cudaSuccess) return fail(c, LBCAD_E_CUDA, std::string("adjoint sums: ") + cudaGetErrorString(e));
   // lcur holds the cotangent of the checkpointed initial state
   c->adj_lam = lcur.g;
   double tot[2];
