@@ -1,14 +1,14 @@
 // lbcad_adjoint.cuh -- reverse mode (vector-Jacobian products) of one hybrid step.
 //
 // The step maps the stored state s_t = (g*, Q, psi, u) to s_{t+1}.  Given the cotangent
-// lam_{t+1} of s_{t+1}, three gather-form kernels produce lam_t:
+// lam_{t+1} of s_{t+1}, four gather-form kernels produce lam_t:
 //   RK1 k_adj_update : per site, VJP of the update (upwind/co-rotation Q update, Cahn-Hilliard psi
 //                      update, BGK + Guo collision) by a hand-written reverse sweep;
-//   RK2 k_adj_fields : transposes of the stencils that fed the update (div sigma -> sigma, lap mu -> mu,
-//                      grad u -> u, face reads -> Q/psi/u, the pull -> g*), then per site the VJP of
-//                      local_fields (H, mu, sigma of Eqs. 2-5) with respect to its inputs and to zeta and
-//                      q0, by a hand-written reverse sweep;
-//   RK3 k_adj_gather : transposes of the Q/psi stencils (gradient, Laplacian, Hessian).
+//   RK2 k_adj_spread : transposes of the stencils that fed the update (div sigma -> sigma, lap mu -> mu,
+//                      grad u -> u, face reads -> Q/psi/u, the pull -> g*);
+//   RK3 k_adj_fields : per site the VJP of local_fields (H, mu, sigma of Eqs. 2-5) with respect to its
+//                      inputs and to zeta and q0, by a hand-written reverse sweep;
+//   RK4 k_adj_gather : transposes of the Q/psi stencils (gradient, Laplacian, Hessian).
 // The per-site reverse sweeps recompute the forward intermediates of the site and take
 // every branch (upwind sides) as the forward takes it.  Stencil transposes use the negated offsets on the
 // periodic lattice, so no site is written by two threads.
@@ -17,11 +17,12 @@
 // of local_fields.  Most of these are a factor known at the reading site times a cotangent it can read anyway
 // (populations: (1 - 1/tau) lam_g plus a linear form of four values; upwind faces: the face velocity times lam_Q
 // or lam_psi; lap mu and H: a coefficient times lam; lap Q, lap psi and the Hessian of psi: K lH, and lmu times
-// Q), so only 16 values of the first and 24 of the second are passed, in quads and pairs.  The force F of
+// Q), so only 16 values of the first and 24 of the second are passed, in quads and pairs (and the 10 cotangents of
+// sigma and mu, at the site only).  The force F of
 // each replayed step is kept by the replay (3 values per site and state), so that no stress is needed here.
 #pragma once
 
-#include "lbcad_kernels.cuh"
+#include "lbcad_march.cuh"
 
 namespace lbcad {
 
@@ -35,7 +36,8 @@ struct AdjDesc {
   const T* lp;
   const T* lu;
   T* A;               // RK1 -> RK2, quads [5][site][4]: (lF, lm0), (lj, -), (lW_ab over a, -) for b = x, y, z
-  T* B;               // RK2 -> RK3: quads [4][site][4]: ldQ_a components 0-3 for a = x, y, z, lH 0-3; then
+  T* L;               // RK2 -> RK3: quads [2][site][4]: cotangents of sigma 0-3, 4-7; pairs [site][2]: (sigma 8, mu)
+  T* B;               // RK3 -> RK4: quads [4][site][4]: ldQ_a components 0-3 for a = x, y, z, lH 0-3; then
                       // pairs [4][site][2]: (ldQ_a component 4, ldpsi_a) for a = x, y, z, (lH 4, lmu)
   T* og;              // cotangent of s_t: g* (19), Q (5), psi (1), u (3); RK1 leaves the site-local parts of Q, psi, u
   T* oq;
@@ -44,7 +46,8 @@ struct AdjDesc {
   double* pgrad;      // per block: sums over the reverse steps of d/dzeta, d/dq0 (2 per block)
 };
 
-constexpr int kAdjBlock = 128;
+using AdjTile = Tile<32, 4>;
+constexpr int kAdjBlock = AdjTile::NT;
 
 template <typename T>
 struct Quad {
@@ -613,7 +616,9 @@ __device__ __forceinline__ void local_fields_vjp(const Coef<T>& c, const T in[36
 }
 
 // ---------------------------------------------------------------- RK1
-// The site of a thread and its neighbour offsets; false past the last site.
+// The site of a thread and its neighbour offsets; false past the last site.  (Blocks that march on tiles, as k_adj_fields
+// does, find more of their neighbours in L1 but run fewer warps: 37 us for k_adj_spread either way, 25 against 20 for
+// k_adj_gather, 64^3.)
 __device__ __forceinline__ bool adj_site(int nx, int ny, int nz, long long N, long long& s, Nbr& nb) {
   s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= N) return false;
@@ -672,18 +677,15 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_update(AdjDesc<T> A) {
 }
 
 // ---------------------------------------------------------------- RK2
-// Transposes of the stencils of the update and of the pull, gathered at the site, then the VJP of local_fields there
-// (its inputs packed: q0 0-4, p0 5, dq 6-20 (a*5 + k), lapq 21-25, dp 26-28, lapp 29, hp 30-35).
+// Transposes of the stencils of the update and of the pull, gathered at the site.
 template <typename T>
-__global__ void __launch_bounds__(kAdjBlock) k_adj_fields(AdjDesc<T> A) {
+__global__ void __launch_bounds__(kAdjBlock) k_adj_spread(AdjDesc<T> A) {
   const InstDesc<T>& I = A.I;
   const long long N = I.N;
-  double pz = 0.0, pq = 0.0;
   long long s;
-  GlobalAcc<T> acc;
-  if (adj_site(I.nx, I.ny, I.nz, N, s, acc.nb)) {
-    acc.q_ = I.q_in; acc.ps = I.psi_in; acc.N = N;
-    const Nbr& nb = acc.nb;
+  Nbr nb;
+  if (!adj_site(I.nx, I.ny, I.nz, N, s, nb)) return;
+  {
     const Coef<T>& c = I.c;
     // pull: g[i](x) = g*_i(x - c_i)  =>  lam g*_i(y) = lam g[i](y + c_i).  F_a(x) = sum_b sum_{i odd, c_ib != 0}
     // sgn(c_ib) wt_i (sigma_ab(x + c_i) - sigma_ab(x - c_i)), and grad u the same, so both transposes take
@@ -728,12 +730,9 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_fields(AdjDesc<T> A) {
       lmu += (lat_c2(i) == 1 ? T(1.0 / 3.0) : T(1.0 / 6.0)) * ld(A.lp + nb.off(-lat_c(i, 0), -lat_c(i, 1), -lat_c(i, 2)));
     lmu *= c.M;
     // face reads of the sites at y - e_a (their upper face) and y + e_a (their lower face)
-    T lq[5], lp = A.op[s], lqc[5];
+    T lq[5], lp = A.op[s];
 #pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      lq[k] = A.oq[k * N + s];
-      lqc[k] = ld(A.lq + k * N + s);
-    }
+    for (int k = 0; k < 5; ++k) lq[k] = A.oq[k * N + s];
     const T p0 = ld(I.psi_in + s);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -753,51 +752,120 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_fields(AdjDesc<T> A) {
     }
 #pragma unroll
     for (int a = 0; a < 3; ++a) A.ou[a * N + s] = lu[a];
-    // local_fields
-    T in[36];
-    {
-      T q0[5], pc, dq[3][5], lapq[5], dp[3], lapp, hp[6];
-      gather_fields<T>(acc, q0, pc, dq, lapq, dp, lapp, hp);
 #pragma unroll
-      for (int k = 0; k < 5; ++k) in[k] = q0[k];
-      in[5] = pc;
+    for (int k = 0; k < 5; ++k) A.oq[k * N + s] = lq[k];
+    A.op[s] = lp;
+    st_quad_at(A.L, s, ls[0], ls[1], ls[2], ls[3]);
+    st_quad_at(A.L + 4 * N, s, ls[4], ls[5], ls[6], ls[7]);
+    st_pair_at(A.L + 8 * N, s, ls[8], lmu);
+  }
+}
+
+// ---------------------------------------------------------------- RK3
+// The VJP of local_fields (inputs packed: q0 0-4, p0 5, dq 6-20 (a*5 + k), lapq 21-25, dp 26-28, lapp 29, hp 30-35).
+// Marches up z on tiles like the step's kernels, with planes of Q and psi in shared memory; without the carry of
+// the stencils, whose 54 registers the reverse sweep needs.
+constexpr int kAdjRing = 4;
+
+template <typename T>
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 3 : 2)
+    k_adj_fields(AdjDesc<T> A, const MarchItem* __restrict__ items, int nitems) {
+  using G = AdjTile;
+  constexpr int QSL = 6 * G::SP;
+  __shared__ __align__(16) T sQ[kAdjRing * QSL];
+  const InstDesc<T>& I = A.I;
+  const int nx = I.nx, ny = I.ny, nz = I.nz;
+  const long long N = I.N;
+  const unsigned plane = (unsigned)(nx * ny);
+  const Coef<T>& c = I.c;
+  const int tid = threadIdx.x, tx = tid % G::TX, ty = tid / G::TX;
+  double pz = 0.0, pq = 0.0;
+  for (int item = blockIdx.x; item < nitems; item += gridDim.x) {
+    const MarchItem tl = items[item];
+    const int zb = tl.zb, ze = tl.ze;
+    unsigned off[G::LD];
+    tile_offsets<G>(tl, nx, ny, off);
+    auto issue = [&](int p) {
+      const unsigned gz = (unsigned)wrap_plane(p, nz) * plane;
+      T* dq = sQ + ((p + 4) & 3) * QSL;
 #pragma unroll
-      for (int a = 0; a < 3; ++a)
+      for (int r = 0; r < G::LD; ++r) {
+        const int k = tid + r * G::NT;
+        if (k < G::SP) {
+          const unsigned o = gz + off[r];
 #pragma unroll
-        for (int k = 0; k < 5; ++k) in[6 + 5 * a + k] = dq[a][k];
+          for (int f = 0; f < 5; ++f) cp_async_elem(dq + qidx<G::SP>(f, k), I.q_in + f * N + o);
+          cp_async_elem(dq + qidx<G::SP>(5, k), I.psi_in + o);
+        }
+      }
+    };
+    __syncthreads();  // the previous item is done with the tiles
+    issue(zb - 1);
+    issue(zb);
+    issue(zb + 1);
+    cp_async_commit_wait_all();
+    __syncthreads();
+    const bool inside = tl.x0 + tx < nx && tl.y0 + ty < ny;
+    const unsigned soff = (unsigned)((tl.y0 + ty) * nx + (tl.x0 + tx));
+    TileAcc<T, G> acc;
+    acc.sc = (ty + 1) * G::SW + (tx + 1);
+#pragma unroll 1
+    for (int z = zb; z < ze; ++z) {
+      if (z + 1 < ze) issue(z + 2);
+      if (inside) {
+        const long long s = (unsigned)z * plane + soff;
 #pragma unroll
-      for (int k = 0; k < 5; ++k) in[21 + k] = lapq[k];
+        for (int j = 0; j < 3; ++j) acc.qpl[j] = sQ + ((z + 3 + j) & 3) * QSL;
+        // output cotangents: H 0-4, mu 5, sigma 6-14
+        T lo[15];
+        const Quad<T> l0 = ld_quad(A.L, s), l1 = ld_quad(A.L + 4 * N, s);
+        const Vec2<T> l2 = ld_pair(A.L + 8 * N, s);
+        lo[6] = l0.x, lo[7] = l0.y, lo[8] = l0.z, lo[9] = l0.w;
+        lo[10] = l1.x, lo[11] = l1.y, lo[12] = l1.z, lo[13] = l1.w;
+        lo[14] = l2.x, lo[5] = l2.y;
 #pragma unroll
-      for (int a = 0; a < 3; ++a) in[26 + a] = dp[a];
-      in[29] = lapp;
+        for (int k = 0; k < 5; ++k) lo[k] = c.gammaQ * ld(A.lq + k * N + s);
+        T in[36];
+        {
+          T q0[5], pc, dq[3][5], lapq[5], dp[3], lapp, hp[6];
+          gather_fields<T>(acc, q0, pc, dq, lapq, dp, lapp, hp);
 #pragma unroll
-      for (int k = 0; k < 6; ++k) in[30 + k] = hp[k];
+          for (int k = 0; k < 5; ++k) in[k] = q0[k];
+          in[5] = pc;
+#pragma unroll
+          for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int k = 0; k < 5; ++k) in[6 + 5 * a + k] = dq[a][k];
+#pragma unroll
+          for (int k = 0; k < 5; ++k) in[21 + k] = lapq[k];
+#pragma unroll
+          for (int a = 0; a < 3; ++a) in[26 + a] = dp[a];
+          in[29] = lapp;
+#pragma unroll
+          for (int k = 0; k < 6; ++k) in[30 + k] = hp[k];
+        }
+        T ci[24], lH[5], lmo, lz, lq0;
+        local_fields_vjp<T>(c, in, lo, ci, lH, lmo, lz, lq0);
+#pragma unroll
+        for (int k = 0; k < 5; ++k) A.oq[k * N + s] += ci[k];
+        A.op[s] += ci[5];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          st_quad_at(A.B + 4 * a * N, s, ci[6 + 5 * a], ci[7 + 5 * a], ci[8 + 5 * a], ci[9 + 5 * a]);
+          st_pair_at(A.B + (16 + 2 * a) * N, s, ci[10 + 5 * a], ci[21 + a]);
+        }
+        st_quad_at(A.B + 12 * N, s, lH[0], lH[1], lH[2], lH[3]);
+        st_pair_at(A.B + 22 * N, s, lH[4], lmo);
+        pz += (double)lz;
+        pq += (double)lq0;
+      }
+      cp_async_commit_wait_all();
+      __syncthreads();
     }
-    // output cotangents: H 0-4, mu 5, sigma 6-14
-    T lo[15];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) lo[k] = c.gammaQ * lqc[k];
-    lo[5] = lmu;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) lo[6 + k] = ls[k];
-    T ci[24], lH[5], lmo, lz, lq0;
-    local_fields_vjp<T>(c, in, lo, ci, lH, lmo, lz, lq0);
-#pragma unroll
-    for (int k = 0; k < 5; ++k) A.oq[k * N + s] = lq[k] + ci[k];
-    A.op[s] = lp + ci[5];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      st_quad_at(A.B + 4 * a * N, s, ci[6 + 5 * a], ci[7 + 5 * a], ci[8 + 5 * a], ci[9 + 5 * a]);
-      st_pair_at(A.B + (16 + 2 * a) * N, s, ci[10 + 5 * a], ci[21 + a]);
-    }
-    st_quad_at(A.B + 12 * N, s, lH[0], lH[1], lH[2], lH[3]);
-    st_pair_at(A.B + 22 * N, s, lH[4], lmo);
-    pz = (double)lz;
-    pq = (double)lq0;
   }
   // per-block FP64 sums of the parameter gradients (fixed order: deterministic), added to the block's own over the
   // reverse steps; one pass over the blocks at the end sums them
-  __shared__ double sh[2][kAdjBlock / 32];
+  __shared__ double sh[2][G::NT / 32];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     pz += __shfl_down_sync(0xffffffffu, pz, o);
@@ -808,12 +876,12 @@ __global__ void __launch_bounds__(kAdjBlock) k_adj_fields(AdjDesc<T> A) {
   __syncthreads();
   if (threadIdx.x < 2) {
     double a0 = 0.0;
-    for (int w = 0; w < kAdjBlock / 32; ++w) a0 += sh[threadIdx.x][w];
+    for (int w = 0; w < G::NT / 32; ++w) a0 += sh[threadIdx.x][w];
     A.pgrad[2 * blockIdx.x + threadIdx.x] += a0;
   }
 }
 
-// ---------------------------------------------------------------- RK3
+// ---------------------------------------------------------------- RK4
 // Transposes of gather_fields, added to the partial cotangents of Q and psi:
 //   d_a f(x) = sum_i 3 w_i c_ia f(x + c_i),  lap f(x) = sum_i lw_i f(x + c_i) - 4 f(x),
 //   hess_aa f(x) = f(x + e_a) + f(x - e_a) - 2 f(x),
@@ -951,19 +1019,22 @@ cudaError_t LaunchAdj<T, SHIFT>::reverse_step(const AdjDescHost<T>& h, cudaStrea
   A.I = h.I;
   A.F = h.F;
   A.lg = h.lg; A.lq = h.lq; A.lp = h.lp; A.lu = h.lu;
-  A.A = h.A; A.B = h.B;
+  A.A = h.A; A.L = h.L; A.B = h.B;
   A.og = h.og; A.oq = h.oq; A.op = h.op; A.ou = h.ou;
   A.pgrad = h.pgrad;
   const unsigned nb = (unsigned)((h.I.N + kAdjBlock - 1) / kAdjBlock);
   k_adj_update<T, SHIFT><<<nb, kAdjBlock, 0, s>>>(A);
-  k_adj_fields<T><<<nb, kAdjBlock, 0, s>>>(A);
+  k_adj_spread<T><<<nb, kAdjBlock, 0, s>>>(A);
+  k_adj_fields<T><<<h.work.grid, kAdjBlock, 0, s>>>(A, h.work.items, h.work.nitems);
   k_adj_gather<T><<<nb, kAdjBlock, 0, s>>>(A);
   return cudaGetLastError();
 }
 
 template <typename T, bool SHIFT>
-int LaunchAdj<T, SHIFT>::blocks(long long N) {
-  return (int)((N + kAdjBlock - 1) / kAdjBlock);
+cudaError_t LaunchAdj<T, SHIFT>::fields_shape(int* tx, int* ty, int* per_sm) {
+  *tx = AdjTile::TX;
+  *ty = AdjTile::TY;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_adj_fields<T>, kAdjBlock, 0);
 }
 
 template <typename T, bool SHIFT>

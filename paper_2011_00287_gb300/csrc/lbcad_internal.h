@@ -222,18 +222,20 @@ struct AdjDescHost {
   InstDesc<T> I;                 // state s_t (inputs)
   const T* F;                    // force of the step from it [3][N]
   const T *lg, *lq, *lp, *lu;    // cotangent of s_{t+1}
-  T *A, *B;                      // work: kAdjWorkA and kAdjWorkB values per site
+  T *A, *L, *B;                  // work: kAdjWorkA, kAdjWorkL and kAdjWorkB values per site
+  MarchWork work;                // items of k_adj_fields
   T *og, *oq, *op, *ou;          // cotangent of s_t
   double* pgrad;                 // per-block sums over the reverse steps of d/dzeta, d/dq0
 };
-constexpr int kAdjWorkA = 20, kAdjWorkB = 24;
+constexpr int kAdjWorkA = 20, kAdjWorkL = 12, kAdjWorkB = 24;  // (L holds 10, rounded up to whole quads)
 
 template <typename T, bool SHIFT>
 struct LaunchAdj {
   static cudaError_t reverse_step(const AdjDescHost<T>& h, cudaStream_t s);
   static cudaError_t seed(const InstDesc<T>& I, const double dX[3], const double ks[3], const double kc[3], T* lp,
                           cudaStream_t s);
-  static int blocks(long long N);
+  // tile and resident blocks per SM of k_adj_fields
+  static cudaError_t fields_shape(int* tx, int* ty, int* per_sm);
   static cudaError_t export_fields(const InstDesc<T>& I, const T* lam, uint32_t mask, double* dst, cudaStream_t s);
 };
 

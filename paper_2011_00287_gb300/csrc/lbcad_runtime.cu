@@ -102,6 +102,8 @@ struct lbcad_ctx {
   bool observe = true;     // fused steps form the a6 sums (lbcad_set_observe)
   bool obs_valid = false;
   void* adj_lam = nullptr;  // cotangent of the initial state of the last lbcad_adjoint
+  void* adj_host = nullptr;  // pinned: the gradient's way to the caller's memory
+  size_t adj_host_bytes = 0;
   // buffers of lbcad_adjoint, kept for the next call (reused when large enough)
   void* adj_buf[8] = {};
   size_t adj_bytes[8] = {};
@@ -164,6 +166,7 @@ void release(lbcad_ctx* c) {
   if (c->stream) cudaStreamSynchronize(c->stream);
   if (c->gexec) cudaGraphExecDestroy(c->gexec);
   if (c->graph) cudaGraphDestroy(c->graph);
+  if (c->adj_host) cudaFreeHost(c->adj_host);
   for (void* p : c->allocs) {
     if (c->free) c->free(p, c->user); else cudaFree(p);
   }
@@ -1089,13 +1092,23 @@ int adjoint_impl(lbcad_ctx* c, int64_t nsteps, int k, double* dzeta, double* dq0
   T* ck = (T*)adj_buffer(c, 0, (size_t)S * st * sizeof(T));
   T* seg = (T*)adj_buffer(c, 1, (size_t)(k + 1) * st * sizeof(T));
   T* lam = (T*)adj_buffer(c, 2, 2 * st * sizeof(T));
-  T* work = (T*)adj_buffer(c, 3, (kAdjWorkA + kAdjWorkB) * (size_t)N * sizeof(T));
+  T* work = (T*)adj_buffer(c, 3, (kAdjWorkA + kAdjWorkL + kAdjWorkB) * (size_t)N * sizeof(T));
   T* fl = (T*)adj_buffer(c, 4, (size_t)k * fs * sizeof(T));
-  const int nb = LaunchAdj<T, SHIFT>::blocks(N);
+  // items of the reverse kernel that marches
+  int tx = 0, ty = 0, per_sm = 0, sms = 0;
+  CK(c, (LaunchAdj<T, SHIFT>::fields_shape(&tx, &ty, &per_sm)));
+  CK(c, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
+  std::vector<MarchItem> items;
+  MarchWork aw = add_items(c, c->work[0], tx, ty, sms * std::max(per_sm, 1), items);
+  const int nb = aw.grid;
   double* pg = (double*)adj_buffer(c, 5, (2 * (size_t)nb + 2) * sizeof(double));
-  if (!ck || !seg || !lam || !work || !fl || !pg) return fail(c, LBCAD_E_OOM, "adjoint buffers");
+  MarchItem* ai = (MarchItem*)adj_buffer(c, 6, items.size() * sizeof(MarchItem));
+  if (!ck || !seg || !lam || !work || !fl || !pg || !ai) return fail(c, LBCAD_E_OOM, "adjoint buffers");
   T* A = work;
-  T* B = A + kAdjWorkA * N;
+  T* L2 = A + kAdjWorkA * N;
+  T* B = L2 + kAdjWorkL * N;
+  aw.items = ai;
+  CK(c, cudaMemcpyAsync(ai, items.data(), items.size() * sizeof(MarchItem), cudaMemcpyHostToDevice, c->stream));
   double* total = pg + 2 * nb;
   CK(c, cudaMemsetAsync(pg, 0, (2 * (size_t)nb + 2) * sizeof(double), c->stream));
   using Step = LaunchFused<T, SHIFT>;
@@ -1159,7 +1172,8 @@ int adjoint_impl(lbcad_ctx* c, int64_t nsteps, int k, double* dzeta, double* dq0
       h.I.g_in = in.g; h.I.q_in = in.q; h.I.psi_in = in.p; h.I.u_in = in.u;
       h.F = fl + (size_t)j * fs;
       h.lg = lcur.g; h.lq = lcur.q; h.lp = lcur.p; h.lu = lcur.u;
-      h.A = A; h.B = B;
+      h.A = A; h.L = L2; h.B = B;
+      h.work = aw;
       h.og = lnxt.g; h.oq = lnxt.q; h.op = lnxt.p; h.ou = lnxt.u;
       h.pgrad = pg;
       e = LaunchAdj<T, SHIFT>::reverse_step(h, c->stream);
@@ -1173,14 +1187,27 @@ int adjoint_impl(lbcad_ctx* c, int64_t nsteps, int k, double* dzeta, double* dq0
   c->adj_lam = lcur.g;
   double tot[2];
   CK(c, cudaMemcpyAsync(tot, total, sizeof(tot), cudaMemcpyDeviceToHost, c->stream));
-  std::vector<T> hq(5 * (size_t)N);
-  CK(c, cudaMemcpyAsync(hq.data(), lcur.q, hq.size() * sizeof(T), cudaMemcpyDeviceToHost, c->stream));
+  // through pinned memory kept with the context: a fresh pageable vector costs its page faults and a staged copy on
+  // every call (64^3: 0.4 ms)
+  const size_t qn = 5 * (size_t)N;
+  if (dQ0 && c->adj_host_bytes < qn * sizeof(T)) {
+    if (c->adj_host) cudaFreeHost(c->adj_host);
+    c->adj_host_bytes = 0;
+    if (cudaHostAlloc(&c->adj_host, qn * sizeof(T), cudaHostAllocDefault) != cudaSuccess) {
+      cudaGetLastError();
+      c->adj_host = nullptr;
+      return fail(c, LBCAD_E_OOM, "pinned host allocation failed");
+    }
+    c->adj_host_bytes = qn * sizeof(T);
+  }
+  const T* hq = (const T*)c->adj_host;
+  if (dQ0) CK(c, cudaMemcpyAsync(c->adj_host, lcur.q, qn * sizeof(T), cudaMemcpyDeviceToHost, c->stream));
   CK(c, cudaStreamSynchronize(c->stream));
   if (dzeta) *dzeta = tot[0];
   if (dq0) *dq0 = tot[1];
   if (J_out) *J_out = J;
   if (dQ0)
-    for (size_t i = 0; i < hq.size(); ++i) dQ0[i] = (double)hq[i];
+    for (size_t i = 0; i < qn; ++i) dQ0[i] = (double)hq[i];
   for (double v : tot)
     if (!std::isfinite(v)) return fail(c, LBCAD_E_NAN, "non-finite adjoint gradient");
   return LBCAD_OK;
