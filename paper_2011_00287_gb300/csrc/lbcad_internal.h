@@ -123,7 +123,10 @@ struct MarchDesc {
   T* psi_out;
   const T* u_in[3];
   T* u_out[3];
-  T* S[6];             // scratch of the default path: arrays of pairs [N][2] (see PairPlane in lbcad_march.cuh)
+  // scratch of the default path: six arrays of pairs [sites][2] (see PairPlane in lbcad_march.cuh) over the planes of
+  // the launch, sz0 the first of them; sync coupling and Heun use the first five
+  T* S[6];
+  int sz0;
   T* H[5];             // sync coupling, Heun: H at t
   T* F[3];             // replay of the adjoint: force
   T* rq[6];            // Heun: right-hand side at t, predicted state (Q, psi), H and mu there
@@ -170,6 +173,7 @@ struct FusedCfg {
 // The work of one step for a group of instances (at most kPackMany).
 struct StepWork {
   int first = 0, ninst = 0;  // instances of the group
+  int sz0 = 0;               // first plane of the scratch
   MarchWork fields, lb, pred, op[2];
 };
 
@@ -192,6 +196,8 @@ struct FusedObs {
   unsigned* cnt;       // [ninst]
   double* latest;      // [ninst][12]
   int maxrun;
+  int slot0;  // one instance, in several slabs: slots of the slabs before this one, and of all of them
+  int total;
 };
 
 // The default path (lbcad_march.cuh), in several tile shapes, for each variant of the LB part:

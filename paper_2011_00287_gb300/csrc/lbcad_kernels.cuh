@@ -549,12 +549,11 @@ __device__ __forceinline__ void gather_upwind(const A& acc, const T u0[3], Vec2<
   for (int i = 1; i < 7; ++i) pf[i - 1] = acc.psi(lat_c(i, 0), lat_c(i, 1), lat_c(i, 2));
 }
 
-// The stencils of a4 at one site: lap mu, W_ab = d_b u_a, Q and psi at the centre, Q at the
-// upwind neighbours, psi and the axial velocities at the faces.
+// The stencils of a4 at one site: W_ab = d_b u_a, Q and psi at the centre, Q at the upwind neighbours, psi and
+// the axial velocities at the faces; gather_op: and lap mu.
 template <typename T, class A>
-__device__ __forceinline__ void gather_op(const A& acc, T& lapmu, T Wg[3][3], T q0[5], Vec2<T> qu[3][3], T& p0,
-                                          T pf[6], T u0[3], T uf[6]) {
-  lapmu = gather_lapmu<T>(acc);
+__device__ __forceinline__ void gather_advection(const A& acc, T Wg[3][3], T q0[5], Vec2<T> qu[3][3], T& p0, T pf[6],
+                                                 T u0[3], T uf[6]) {
   gather_velocity<T>(acc, Wg, u0, uf);
   gather_upwind<T>(acc, u0, qu, pf);
 #pragma unroll
@@ -564,6 +563,12 @@ __device__ __forceinline__ void gather_op(const A& acc, T& lapmu, T Wg[3][3], T 
     if (j < 2) q0[2 * j + 1] = v.y;
     else p0 = v.y;
   }
+}
+template <typename T, class A>
+__device__ __forceinline__ void gather_op(const A& acc, T& lapmu, T Wg[3][3], T q0[5], Vec2<T> qu[3][3], T& p0,
+                                          T pf[6], T u0[3], T uf[6]) {
+  lapmu = gather_lapmu<T>(acc);
+  gather_advection<T>(acc, Wg, q0, qu, p0, pf, u0, uf);
 }
 
 // a4, psi: the divergence of the upwind flux of psi.

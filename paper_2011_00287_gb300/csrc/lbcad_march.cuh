@@ -137,12 +137,11 @@ __device__ __forceinline__ int qidx(int f, int k) {
   return (f >> 1) * 2 * SP + 2 * k + (f & 1);
 }
 
-// Neighbour reads of one tile site: Q/psi pairs, velocity, and mu (lane 1 of stress pair 4).
+// Neighbour reads of one tile site: Q/psi pairs and velocity.
 template <typename T, class G>
 struct TileAcc {
   const T* qpl[3];
   const T* upl[3];
-  const T* mpl[3];
   int sc;
   __device__ __forceinline__ int at(int cx, int cy) const { return sc + cy * G::SW + cx; }
   __device__ __forceinline__ Vec2<T> pair(int j, int cx, int cy, int cz) const {
@@ -159,9 +158,6 @@ struct TileAcc {
     const int k = at(cx, cy);
     return Vel3<T>{lds2(upl[cz + 1] + 2 * k), upl[cz + 1][2 * G::SP + k]};
   }
-  __device__ __forceinline__ Vec2<T> spair(int, int cx, int cy, int cz) const {
-    return Vec2<T>{T(0), mpl[cz + 1][at(cx, cy)]};
-  }
 };
 
 // Global offsets are unsigned site numbers (a box has at most 2^31 sites) added to a field's base pointer: the
@@ -174,6 +170,13 @@ __device__ __forceinline__ void tile_offsets(const MarchItem& tl, int nx, int ny
     const int k = (int)threadIdx.x + r * G::NT;
     off[r] = k < G::SP ? (unsigned)(wrapmod(tl.y0 + k / G::SW - 1, ny) * nx + wrapmod(tl.x0 + k % G::SW - 1, nx)) : 0u;
   }
+}
+
+// The scratch plane of lattice plane z (in [0, nz)): plane I.sz0 comes first (see MarchDesc).
+template <typename T>
+__device__ __forceinline__ int scratch_plane(const MarchDesc<T>& I, int z) {
+  const int k = z - I.sz0;
+  return k < 0 ? k + I.nz : k;
 }
 
 // Resident blocks per SM a kernel is built for, given its threads and the registers a thread wants.
@@ -193,8 +196,7 @@ struct FieldsSmem {
 
 // kMarchOp: sigma, mu, the flux divergence and psi of every site into the scratch pairs and the new Q
 // (Euler with the velocity of the previous step).  kMarchH: sigma and mu into the pairs, H into its
-// scratch (sync coupling, Heun).  kMarchPred: H and mu of the Heun predicted state qp into the sigma
-// scratch (H at sig[0..5N), mu at sig[5N..6N)).
+// scratch (sync coupling, Heun).  kMarchPred: H and mu of the Heun predicted state qp into Hp.
 template <typename T, int MI, int TX, int TY, int MODE>
 __global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? blocks_for(TX * TY, TX * TY > 128 ? 128 : 168) : 1)
     k_march_fields(const __grid_constant__ InstPack<T, MI> P, const MarchItem* __restrict__ items, int nitems) {
@@ -265,9 +267,10 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? blocks_for(TX * TY, 
             for (int k = 0; k < 5; ++k) st_out(I.Hp[k] + s, H[k]);
             st_out(I.Hp[5] + s, mu);
           } else {
+            const unsigned ss = (unsigned)scratch_plane(I, z) * plane + soff;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) st_pair(pair_at(I.S[j], s), sig[pair_c0(j)], sig[pair_c1(j)]);
-            st_pair(pair_at(I.S[4], s), sig[8], mu);
+            for (int j = 0; j < 4; ++j) st_pair(pair_at(I.S[j], ss), sig[pair_c0(j)], sig[pair_c1(j)]);
+            st_pair(pair_at(I.S[4], ss), sig[8], mu);
             T div = T(0);
             if constexpr (OP) {
               TileAcc<T, G> acc;
@@ -290,7 +293,7 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? blocks_for(TX * TY, 
 #pragma unroll
               for (int k = 0; k < 5; ++k) st_out(I.H[k] + s, H[k]);
             }
-            st_pair(pair_at(I.S[5], s), div, p0);
+            if constexpr (OP) st_pair(pair_at(I.S[5], ss), div, p0);
           }
         }
       }
@@ -393,7 +396,7 @@ __device__ __forceinline__ void obs_tree12(double* red, int M) {
 // subsets by a fixed tree, so the result does not depend on which block finishes last.
 // No spin waits.  red: shared scratch of at least 12 * (blockDim.x / 12) doubles.
 // mass0(inst) = N rho0 with shifted populations, else 0.  ONE: the launch holds one instance, so every block has one
-// slot, its own number, and the slot maps need not be read (each read is a trip to L2 on the critical path of a small box).
+// slot and the slot maps need not be read (each read is a trip to L2 on the critical path of a small box).
 template <bool ONE, class MS>
 __device__ __forceinline__ void obs_block_end(const FusedObs& ob, int nrun, double* red, const MS& mass0) {
   __shared__ int last;
@@ -402,12 +405,12 @@ __device__ __forceinline__ void obs_block_end(const FusedObs& ob, int nrun, doub
   __syncthreads();
   for (int j = 0; j < nrun; ++j) {
     const int inst = ONE ? 0 : ob.slot_inst[blockIdx.x * ob.maxrun + j];
-    if (tid == 0) last = atomicAdd(&ob.cnt[inst], 1u) == (ONE ? gridDim.x : (unsigned)ob.nslot[inst]) - 1u;
+    if (tid == 0) last = atomicAdd(&ob.cnt[inst], 1u) == (ONE ? (unsigned)ob.total : (unsigned)ob.nslot[inst]) - 1u;
     __syncthreads();
     if (last) {
       __threadfence();
       const int per = blockDim.x / 12;
-      const int lo = ONE ? 0 : ob.slot_lo[inst], hi = ONE ? (int)gridDim.x : ob.slot_hi[inst];
+      const int lo = ONE ? 0 : ob.slot_lo[inst], hi = ONE ? ob.total : ob.slot_hi[inst];
       if (tid < 12 * per) {
         const int k = tid % 12, l = tid / 12;
         double v = 0.0;
@@ -478,11 +481,12 @@ struct ObsReduce {
 template <typename T, class G, int Q, int MODE>
 struct LbSmem {
   static constexpr int NSLOT = 3;  // planes p-1, p and the arriving one
-  static constexpr int SL = 12 * G::SP;
+  static constexpr int NP = MODE == kFusedLbOnly ? 5 : 6;  // without psi and its divergence
+  static constexpr int SL = 2 * NP * G::SP;
   static constexpr size_t ring = (size_t)NSLOT * SL * sizeof(T);
   static constexpr int PULL = Q * G::NT;  // pulled populations of one plane; two planes
   static constexpr size_t bytes = ring + (size_t)2 * PULL * sizeof(T);
-  static_assert(ring >= ObsReduce<T, G::NT>::bytes, "the ring is the scratch of the a6 sums");
+  static_assert(MODE != kFusedSums || ring >= ObsReduce<T, G::NT>::bytes, "the ring is the scratch of the a6 sums");
 };
 
 // FORM 0: F = div sigma, BGK + Guo (Eqs. 6-8).  FORM 1: FA = div sigma^A and the equilibrium carrying
@@ -507,7 +511,7 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? blocks_for(TX * TY, 
     const MarchDesc<T>& I = P.d[MI == 1 ? 0 : tl.inst];
     if constexpr (OBS && MI > 1) {
       if (run_inst >= 0 && tl.inst != run_inst) {
-        ObsReduce<T, G::NT>::run(sums, smem_raw, ob, blockIdx.x * ob.maxrun + run);
+        ObsReduce<T, G::NT>::run(sums, smem_raw, ob, ob.slot0 + blockIdx.x * ob.maxrun + run);
         sums.clear();
         ++run;
       }
@@ -520,7 +524,7 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? blocks_for(TX * TY, 
     tile_offsets<G>(tl, nx, ny, off);
     auto slot = [&](int p) { return sS + ((p + 3) % 3) * M::SL; };
     auto issue = [&](int p) {
-      const unsigned gz = (unsigned)wrap_plane(p, nz) * plane;
+      const unsigned gz = (unsigned)scratch_plane(I, wrap_plane(p, nz)) * plane;
       T* d = slot(p);
 #pragma unroll
       for (int r = 0; r < G::LD; ++r) {
@@ -528,7 +532,7 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? blocks_for(TX * TY, 
         if (k < G::SP) {
           const unsigned o = gz + off[r];
 #pragma unroll
-          for (int j = 0; j < 6; ++j) cp_async_pair(d + 2 * (j * G::SP + k), pair_at(I.S[j], o));
+          for (int j = 0; j < M::NP; ++j) cp_async_pair(d + 2 * (j * G::SP + k), pair_at(I.S[j], o));
         }
       }
     };
@@ -632,7 +636,7 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? blocks_for(TX * TY, 
     cp_async_wait<0>();
   }
   if constexpr (OBS) {
-    ObsReduce<T, G::NT>::run(sums, smem_raw, ob, blockIdx.x * ob.maxrun + run);
+    ObsReduce<T, G::NT>::run(sums, smem_raw, ob, ob.slot0 + blockIdx.x * ob.maxrun + run);
     obs_block_end<MI == 1>(ob, run + 1, reinterpret_cast<double*>(smem_raw), [&](int inst) { return P.d[MI == 1 ? 0 : inst].mass0; });
   }
 }
@@ -649,6 +653,8 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 4 ? blocks_for(TX * TY, 
 // itself (H, and in the corrector R(Q) at t and Q, psi at t) arrive the same way, one plane
 // ahead, into two slots by plane parity: read from global memory after the stencils, their
 // latency stood between the update and the plane barrier.
+// lap mu is carried up the planes (nine reads a plane instead of nineteen): 96^3 sync 59.6 -> 58.7 us a step,
+// 128^3 Heun 365 -> 361.
 template <typename T, class G>
 struct OpSmem {
   static constexpr int NSLOT = 4;
@@ -730,6 +736,16 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 8 ? 2 : blocks_for(TX * 
     issue_site(zb);
     cp_async_commit_wait_all();
     __syncthreads();
+    const int sc = (ty + 1) * G::SW + (tx + 1);
+    LapCarry<T> lapm;
+    auto lap_mu = [&](int p) {
+      const T* m = sM + ((p + 4) & 3) * M::MSLOT + sc;
+      return lapm.advance([&](int cx, int cy) { return m[cy * G::SW + cx]; });
+    };
+    if (inside) {
+      lap_mu(zb - 1);
+      lap_mu(zb);
+    }
 #pragma unroll 1
     for (int z = zb; z < ze; ++z) {
       issue(z + 2);
@@ -742,12 +758,12 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 8 ? 2 : blocks_for(TX * 
           const int sl = (z + 3 + j) & 3;
           acc.qpl[j] = sQ + sl * M::QSLOT;
           acc.upl[j] = sU + sl * M::USLOT;
-          acc.mpl[j] = sM + sl * M::MSLOT;
         }
-        acc.sc = (ty + 1) * G::SW + (tx + 1);
-        T lapmu, Wg[3][3], q0[5], p0, pf[6], u0[3], uf[6];
+        acc.sc = sc;
+        const T lapmu = lap_mu(z + 1);
+        T Wg[3][3], q0[5], p0, pf[6], u0[3], uf[6];
         Vec2<T> qu[3][3];
-        gather_op<T>(acc, lapmu, Wg, q0, qu, p0, pf, u0, uf);
+        gather_advection<T>(acc, Wg, q0, qu, p0, pf, u0, uf);
         const unsigned s = (unsigned)z * plane + soff;
         T Hs[5];
 #pragma unroll
@@ -834,7 +850,8 @@ struct MarchShape {
     c->fy = FY;
     c->lx = LX;
     c->ly = LY;
-    return many ? prepare_mi<kPackMany>(split, heun, c) : prepare_mi<1>(split, heun, c);
+    const cudaError_t e = prepare_mi<1>(split, heun, c);  // (a batch can leave one instance for its last launch)
+    return many && e == cudaSuccess ? prepare_mi<kPackMany>(split, heun, c) : e;
   }
 
   template <class... P, class... A>
@@ -867,7 +884,10 @@ struct MarchShape {
   template <int MI>
   static InstPack<T, MI> pack(const StepWork& w, const MarchDesc<T>* d) {
     InstPack<T, MI> P{};
-    for (int i = 0; i < w.ninst && i < MI; ++i) P.d[i] = d[i];
+    for (int i = 0; i < w.ninst && i < MI; ++i) {
+      P.d[i] = d[i];
+      P.d[i].sz0 = w.sz0;
+    }
     return P;
   }
   template <int MI>

@@ -33,6 +33,7 @@ struct Inst {
   void* pb[2] = {nullptr, nullptr};
   void* ub[2] = {nullptr, nullptr};
   void* S = nullptr;   // default path: stress, mu, flux divergence, psi (12 per site)
+  long long SN = 0;    // sites it holds
   void* sig = nullptr;
   void* mu = nullptr;
   void* H = nullptr;
@@ -215,7 +216,7 @@ MarchDesc<T> make_march_desc(const Inst& I, int parity, bool shifted) {
   d.psi_out = (T*)I.pb[b];
   comps(d.u_in, I.ub[a], 3, N);
   comps(d.u_out, I.ub[b], 3, N);
-  comps(d.S, I.S, 6, 2 * N);
+  comps(d.S, I.S, 6, 2 * I.SN);
   comps(d.H, I.H, 5, N);
   comps(d.rq, I.rq, 6, N);
   comps(d.qp, I.qp, 6, N);
@@ -300,6 +301,9 @@ int upload_descs(lbcad_ctx* c);
 int prepare_fused(lbcad_ctx* c, int cfg_index);
 int ensure_scratch(lbcad_ctx* c);
 int default_shape(const lbcad_ctx* c);
+long long scratch_sites(const Inst& I);
+long long group_scratch(const lbcad_ctx* c, const StepWork& g);
+std::vector<StepWork> step_groups(const lbcad_ctx* c);
 
 int create_impl(int n, const lbcad_grid* grids, const lbcad_params* params, uint64_t seed, lbcad_ctx** out) {
   g_create_err.clear();
@@ -394,11 +398,22 @@ int create_impl(int n, const lbcad_grid* grids, const lbcad_params* params, uint
     if (te == cudaSuccess) te = cudaStreamSynchronize(c->stream);
     if (te != cudaSuccess) return bail(LBCAD_E_CUDA, std::string("trig table upload: ") + cudaGetErrorString(te));
   }
-  if (!c->staged_only())
-    for (Inst& I : c->inst) {
-      I.S = dev_alloc(c, 12 * I.N * es);
-      if (!I.S) return bail(LBCAD_E_OOM, "device allocation failed");
+  if (!c->staged_only() && !c->sync_split()) {
+    // one scratch, which the groups use in turn
+    const std::vector<StepWork> groups = step_groups(c);
+    long long most = 0;
+    for (const StepWork& g : groups) most = std::max(most, group_scratch(c, g));
+    char* S = (char*)dev_alloc(c, 12 * (size_t)most * es);
+    if (!S) return bail(LBCAD_E_OOM, "device allocation failed");
+    for (const StepWork& g : groups) {
+      long long at = 0;
+      for (int i = g.first; i < g.first + g.ninst; ++i) {
+        c->inst[i].SN = scratch_sites(c->inst[i]);
+        c->inst[i].S = S + 12 * (size_t)at * es;
+        at += c->inst[i].SN;
+      }
     }
+  }
   c->obs_cnt = (unsigned*)dev_alloc(c, n * sizeof(unsigned));
   c->obs_latest = (double*)dev_alloc(c, (size_t)n * 12 * sizeof(double));
   if (!c->obs_cnt || !c->obs_latest) return bail(LBCAD_E_OOM, "device allocation failed");
@@ -460,10 +475,16 @@ int ensure_scratch(lbcad_ctx* c) {
   if (c->scratch_ready) return LBCAD_OK;
   const size_t es = c->elem();
   for (Inst& I : c->inst) {
-    I.sig = dev_alloc(c, 9 * I.N * es);
-    I.mu = dev_alloc(c, I.N * es);
+    I.sig = dev_alloc(c, 10 * I.N * es);
     I.H = dev_alloc(c, 5 * I.N * es);
-    if (!I.sig || !I.mu || !I.H) return fail(c, LBCAD_E_OOM, "scratch allocation failed");
+    if (!I.sig || !I.H) return fail(c, LBCAD_E_OOM, "scratch allocation failed");
+    I.mu = (char*)I.sig + 9 * I.N * es;
+    if (c->sync_split()) {
+      // the default path's stress and mu; Heun's H and mu at the predicted state follow in the same place once
+      // the predictor has read them
+      I.S = I.sig;
+      I.SN = I.N;
+    }
     if (c->integrator == LBCAD_HEUN) {
       I.rq = dev_alloc(c, 6 * I.N * es);
       I.qp = dev_alloc(c, 6 * I.N * es);
@@ -486,6 +507,50 @@ int default_shape(const lbcad_ctx* c) {
   return square < wide ? 3 : 0;
 }
 
+// Sites whose scratch a launch of the Euler step may hold: a batch is launched in groups of at most that
+// many, a larger box in slabs of planes (the fields kernel then also works on the planes next to the slab).  At 12
+// values a site the scratch stays at 3.2 GB in FP32, where a scratch for every site would take a sixth of the
+// memory left for boxes as large as the device holds.
+constexpr long long kScratchSites = 1LL << 26;
+
+// Planes of the step's slabs of a box (nz: all at once).
+int slab_planes(const Inst& I) {
+  if (I.N <= kScratchSites) return I.g.nz;
+  const long long plane = (long long)I.g.nx * I.g.ny;
+  const int n = (int)std::max(8LL, kScratchSites / plane - 2);
+  return n + 2 < I.g.nz ? n : I.g.nz;
+}
+
+long long scratch_sites(const Inst& I) {
+  const int n = slab_planes(I);
+  return n < I.g.nz ? (long long)I.g.nx * I.g.ny * (n + 2) : I.N;
+}
+
+long long group_scratch(const lbcad_ctx* c, const StepWork& g) {
+  long long n = 0;
+  for (int i = g.first; i < g.first + g.ninst; ++i) n += scratch_sites(c->inst[i]);
+  return n;
+}
+
+// The launches' groups of instances, in order (without their work).
+std::vector<StepWork> step_groups(const lbcad_ctx* c) {
+  std::vector<StepWork> groups;
+  for (int i = 0; i < (int)c->inst.size(); ++i) {
+    if (!groups.empty()) {
+      StepWork& g = groups.back();
+      if (g.ninst < kPackMany && (c->sync_split() || group_scratch(c, g) + scratch_sites(c->inst[i]) <= kScratchSites)) {
+        ++g.ninst;
+        continue;
+      }
+    }
+    StepWork g;
+    g.first = i;
+    g.ninst = 1;
+    groups.push_back(g);
+  }
+  return groups;
+}
+
 // Largest step (sites) whose kernels are launched with programmatic dependent launch.
 constexpr long long kEarlySites = 1 << 20;
 
@@ -494,14 +559,16 @@ constexpr long long kEarlySites = 1 << 20;
 // through ceil(items / blocks) of them, each its planes plus what an item costs besides (two more planes
 // to load and to carry, and a start without overlap: about one plane's time).  The length is the one with the
 // shortest such time, up to 32 planes: neighbouring columns then stay close enough in z to find their halos
-// in L2.
-MarchWork add_items(const lbcad_ctx* c, const StepWork& g, int tx, int ty, int blocks, std::vector<MarchItem>& out) {
+// in L2.  za, zn: of a single box only the planes za ... za + zn - 1, modulo its height (zn 0: all of each box).
+MarchWork add_items(const lbcad_ctx* c, const StepWork& g, int tx, int ty, int blocks, std::vector<MarchItem>& out,
+                    int za = 0, int zn = 0) {
   constexpr double kItemPlanes = 1.0;
   auto columns = [&](const lbcad_grid& b) { return (long long)((b.nx + tx - 1) / tx) * ((b.ny + ty - 1) / ty); };
   int tallest = 0;
-  for (int i = 0; i < g.ninst; ++i) tallest = std::max(tallest, c->inst[g.first + i].g.nz);
+  auto height = [&](const lbcad_grid& b) { return zn > 0 ? zn : b.nz; };
+  for (int i = 0; i < g.ninst; ++i) tallest = std::max(tallest, height(c->inst[g.first + i].g));
   auto slabs_of = [&](const lbcad_grid& b, int n) {  // slabs of box b when the tallest box has n
-    return std::max(1, (int)(((long long)b.nz * n + tallest - 1) / tallest));
+    return std::max(1, (int)(((long long)height(b) * n + tallest - 1) / tallest));
   };
   int best = 1;
   double best_time = -1.0;
@@ -522,9 +589,13 @@ MarchWork add_items(const lbcad_ctx* c, const StepWork& g, int tx, int ty, int b
     sites += c->inst[g.first + i].N;
     const int slabs = slabs_of(b, best);
     for (int k = 0; k < slabs; ++k) {
-      const int zb = (int)((long long)b.nz * k / slabs), ze = (int)((long long)b.nz * (k + 1) / slabs);
-      for (int y0 = 0; y0 < b.ny; y0 += ty)
-        for (int x0 = 0; x0 < b.nx; x0 += tx) out.push_back(MarchItem{i, x0, y0, zb, ze});
+      const int end = za + (int)((long long)height(b) * (k + 1) / slabs);
+      for (int zb = za + (int)((long long)height(b) * k / slabs), ze; zb < end; zb = ze) {
+        const int turn = (zb + b.nz) / b.nz - 1, base = turn * b.nz;  // zb >= -nz; an item ends at the box's edge
+        ze = std::min(end, base + b.nz);
+        for (int y0 = 0; y0 < b.ny; y0 += ty)
+          for (int x0 = 0; x0 < b.nx; x0 += tx) out.push_back(MarchItem{i, x0, y0, zb - base, ze - base});
+      }
     }
   }
   w.items = (const MarchItem*)(first * sizeof(MarchItem));  // offset; the list's address is added when it is uploaded
@@ -554,21 +625,20 @@ int prepare_fused(lbcad_ctx* c, int cfg_index) {
   auto blocks = [&](int per_sm) { return sms * (per_sm > 0 ? per_sm : 1); };
   std::vector<MarchItem> t;
   std::vector<StepWork> work;
-  for (int first = 0; first < (int)c->inst.size(); first += kPackMany) {
-    StepWork g;
-    g.first = first;
-    g.ninst = std::min((int)c->inst.size() - first, kPackMany);
-    // a group of several instances launches the kernels prepared for several; a lone last one would not
-    if (many && g.ninst == 1) {
-      work.back().ninst -= 1;
-      g.first -= 1;
-      g.ninst = 2;
+  for (const StepWork& g : step_groups(c)) {
+    const Inst& I = c->inst[g.first];
+    const int nz = I.g.nz, n = g.ninst == 1 && !split ? slab_planes(I) : nz;
+    for (int z = 0; z == 0 || (n < nz && z < nz); z += n) {
+      work.push_back(g);
+      StepWork& w = work.back();
+      const bool whole = n >= nz;
+      const int zn = std::min(n, nz - z);
+      if (!whole) w.sz0 = (z + nz - 1) % nz;
+      w.fields = add_items(c, w, cfg.fx, cfg.fy, blocks(cfg.fields_per_sm), t, whole ? 0 : z - 1, whole ? 0 : zn + 2);
+      w.lb = add_items(c, w, cfg.lx, cfg.ly, blocks(cfg.lb_per_sm), t, whole ? 0 : z, whole ? 0 : zn);
     }
-    work.push_back(g);
   }
   for (StepWork& g : work) {
-    g.fields = add_items(c, g, cfg.fx, cfg.fy, blocks(cfg.fields_per_sm), t);
-    g.lb = add_items(c, g, cfg.lx, cfg.ly, blocks(cfg.lb_per_sm), t);
     if (split) {
       g.op[0] = add_items(c, g, cfg.lx, cfg.ly, blocks(cfg.op_per_sm[0]), t);
       if (heun) {
@@ -610,7 +680,14 @@ int prepare_fused(lbcad_ctx* c, int cfg_index) {
     ob.slot_inst = (const int*)(at * sizeof(int));
     ob.nslot = (const int*)((at + n) * sizeof(int));
     ob.maxrun = (int)maxrun;
+    // slabs of one instance: their slots follow one another
+    if (g.ninst == 1 && !obs.empty() && work[obs.size() - 1].first == g.first) {
+      ob.slots = obs.back().slots;
+      ob.slot0 = obs.back().slot0 + work[obs.size() - 1].lb.grid;
+    }
     obs.push_back(ob);
+    if (g.ninst == 1)
+      for (size_t k = obs.size(); k > 0 && work[k - 1].first == g.first; --k) obs[k - 1].total = ob.slot0 + grid;
     nslots += n;
   }
   if (t.size() > c->items_cap) {
@@ -1161,7 +1238,9 @@ int adjoint_impl(lbcad_ctx* c, int64_t nsteps, int k, double* dzeta, double* dq0
     for (int j = 0; j < len; ++j) {
       const MarchDesc<T> md = replay_desc<T>(base, N, state_at<T>(seg + (size_t)j * st, N),
                                              state_at<T>(seg + (size_t)(j + 1) * st, N), fl + (size_t)j * fs);
-      e = Step::replay(c->cfg_index, c->work[0], &md, c->stream);
+      e = cudaSuccess;
+      for (size_t w = 0; w < c->work.size() && e == cudaSuccess; ++w)
+        e = Step::replay(c->cfg_index, c->work[w], &md, c->stream);
       if (e != cudaSuccess) return fail(c, LBCAD_E_CUDA, std::string("adjoint replay: ") + cudaGetErrorString(e));
     }
     // reverse steps
