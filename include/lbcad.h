@@ -160,7 +160,8 @@ int lbcad_step(lbcad_ctx* c, int64_t n);
 
 /* Kernel path of lbcad_step.  LBCAD_PATH_FUSED (default): two kernels per step that march up z through
  * shared-memory tiles (fields, stress and the update of Q; then force, populations, psi and the sums),
- * with 12 values per site of scratch allocated at create.  LBCAD_PATH_TWO_KERNEL: a stencil kernel writing
+ * with 12 values per site of scratch allocated at create (for at most 2^26 sites at a time: groups of a batch's
+ * instances and slabs of a larger box use it in turn).  LBCAD_PATH_TWO_KERNEL: a stencil kernel writing
  * H, mu and sigma to a per-site scratch (allocated on the first switch, 15 values per
  * site) and an update kernel, one thread per site; same arithmetic, kept as a cross-check.  Changing the path
  * drops a captured graph. */
@@ -202,9 +203,9 @@ int lbcad_set_tiles(lbcad_ctx* c, int32_t cfg);
 
 /* a6 in the fused step (on = 1, the default): each fused step also forms the FP64 mass,
  * psi, momentum and centroid sums of the state it writes (per-site shares, per-block sums in
- * shared memory, per-segment FP64 partials, and a last-block sum per instance), and
+ * shared memory, FP64 partials per block and instance, and a last-block sum per instance), and
  * lbcad_observables after such a step only copies them.  on = 0 runs the step kernels without
- * the sums (about 5% faster on the 128^3 workload); lbcad_observables then runs a separate
+ * the sums (a few percent faster); lbcad_observables then runs a separate
  * reduction pass over the state.  Either way the state is the same.  Drops a captured graph. */
 int lbcad_set_observe(lbcad_ctx* c, int32_t on);
 
@@ -255,9 +256,9 @@ int lbcad_set_state(lbcad_ctx* c, int32_t inst, const void* src, size_t bytes, i
  * step's own arithmetic).  Writes dJ/dzeta and dJ/dq0 (accumulated in FP64; q0 enters through H and
  * sigma, the initial Q held fixed), dJ/dQ(t0) for the five stored Q components
  * ([5][z][y][x], host FP64, may be NULL) and J itself.  Device memory: (ceil(nsteps /
- * ckpt_every) + ckpt_every + 2) states of 28 values per site, plus 17 values per site for
- * each of the ckpt_every states of a segment (their stress, mu and H, computed once in the
- * replay) and 139 values per site of work; owned by the context until lbcad_destroy and
+ * ckpt_every) + ckpt_every + 3) states of 28 values per site, plus 3 values per site for
+ * each of the ckpt_every steps of a segment (their force, kept by the replay) and 56 values per site
+ * of work; owned by the context until lbcad_destroy and
  * reused by later calls that fit in them.  The paper has no adjoint; this is the differentiation form
  * of the step (gradient of the droplet's drift with respect to activity, chirality and
  * the initial order). */

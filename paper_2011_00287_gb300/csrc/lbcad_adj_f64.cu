@@ -3,7 +3,7 @@
 template struct lbcad::LaunchAdj<double, false>;
 
 namespace lbcad {
-// The per-block partials of d/dzeta and d/dq0 of one reverse step, added to total[0..1]: thread
+// The per-block partials of d/dzeta and d/dq0 (summed over the reverse steps), added to total[0..1]: thread
 // t adds value t & 1 of the blocks t >> 1, t >> 1 + 256, ... (independent loads, a short chain),
 // then a fixed pairing tree over the 256 partial sums of each value.  FP64 additions take about
 // 60 cycles on this part, so a single chain over thousands of blocks took longer than the

@@ -93,7 +93,6 @@ struct InstDesc {
 template <typename T, bool SHIFT>
 struct Launch {
   static cudaError_t step(const InstDesc<T>* d_desc, int ninst, long long total_blocks, int bs, cudaStream_t s);
-  static cudaError_t fields(const InstDesc<T>* d_desc, int ninst, long long total_blocks, int bs, cudaStream_t s);
   // Staged step: fields -> LB -> order-parameter update (Euler), or fields -> LB ->
   // predictor -> fields at the predicted state -> corrector (Heun).  sync advects with the
   // velocity of this step instead of the previous one.

@@ -1346,13 +1346,6 @@ cudaError_t Launch<T, SHIFT>::step(const InstDesc<T>* d_desc, int ninst, long lo
   return cudaGetLastError();
 }
 
-template <typename T, bool SHIFT>
-cudaError_t Launch<T, SHIFT>::fields(const InstDesc<T>* d_desc, int ninst, long long total_blocks, int bs,
-                                     cudaStream_t s) {
-  k_fields<T><<<(unsigned)total_blocks, bs, 0, s>>>(d_desc, ninst);
-  return cudaGetLastError();
-}
-
 template <typename T, bool SHIFT, int ST>
 cudaError_t staged_st(const InstDesc<T>* d_desc, int ninst, unsigned g, int bs, bool heun, bool sync, int vel,
                       int form, cudaStream_t s) {

@@ -12,12 +12,16 @@
 // and nothing is computed twice.  Planes arrive by cp.async one plane ahead, one barrier per
 // plane.  The stress never has to be known on a halo of the tile in shared memory, which is what
 // the split buys: one kernel for the whole step computes sigma on 1.38 sites per output site (tile
-// halo, partly filled warps), opens every column segment with three sigma planes and no output,
+// halo, partly filled warps), opens every run of planes with three sigma planes and no output,
 // and holds both halves' registers.  The scratch costs 2 x 48 bytes per site of traffic in FP32.
 //
-// The grid is persistent: the flattened space of (tile column, z plane) work is split evenly
-// across the blocks, so load balance does not depend on the box shape and one launch covers every
-// instance of a batch.
+// Measured (FP32 with the a6 sums, one kernel for the step -> this file): 64^3 52 -> 34.6 us a step, 128^3 234 -> 193,
+// 256^3 1640 -> 1360; the FP64 step is twice as fast.  At 128^3 k_march_fields takes 85 us, bound by instruction
+// issue at 12 warps an SM (its stencils' registers) with the shared-memory pipe busy most of that time;
+// k_march_lb 104 us, 216 bytes a site at two thirds of the copy rate.  FP64 is bound by the FP64 pipe.
+//
+// The grid is persistent: blocks take work items (a tile column over a slab of planes) in turn, and one
+// launch covers up to kPackMany instances of a batch.
 //
 // The end of the file holds the order-parameter half of the sync-coupled and Heun steps, as tiled
 // z-marching kernels on the same tiles and work split.
@@ -29,7 +33,7 @@
 
 namespace lbcad {
 
-// Periodic plane index for p in [-n, 2n): the planes a column segment touches lie in
+// Periodic plane index for p in [-n, 2n): the planes a work item touches lie in
 // [-1, nz + 1] and every edge is >= 4, so one add or subtract suffices (no division).
 __device__ __forceinline__ int wrap_plane(int p, int n) { return p < 0 ? p + n : (p >= n ? p - n : p); }
 

@@ -92,7 +92,7 @@ struct lbcad_ctx {
   std::vector<MarchDesc<float>> desc32[2];  // by step parity
   std::vector<MarchDesc<double>> desc64[2];
   int cfg_index = 0;
-  // a6 sums of the fused step (see FusedObs): slots per (block, segment), per-instance
+  // a6 sums of the fused step (see FusedObs): slots per (block, run of items), per-instance
   // bookkeeping, and the sums of the latest state; obs_valid while they describe the state
   double* obs_slots = nullptr;
   size_t obs_slots_cap = 0;
@@ -112,7 +112,7 @@ struct lbcad_ctx {
   size_t elem() const { return prec == LBCAD_FP64 ? sizeof(double) : sizeof(float); }
   // the radius-2 stencils run on the staged path only
   bool staged_only() const { return stencil != LBCAD_STENCIL_ISO; }
-  // sync coupling or Heun on the fused path: the LB half in the fused kernel on a fixed tile
+  // sync coupling or Heun on the fused path: the LB half in k_march_lb on a fixed tile
   // shape, then the order-parameter kernels
   bool sync_split() const { return !staged_only() && (coupling == LBCAD_SYNC || integrator == LBCAD_HEUN); }
   // D3Q19 with the body force: the two-kernel path and the adjoint cover this LB only
