@@ -1269,18 +1269,20 @@ int adjoint_impl(lbcad_ctx* c, int64_t nsteps, int k, double* dzeta, double* dq0
   // through pinned memory kept with the context: a fresh pageable vector costs its page faults and a staged copy on
   // every call (64^3: 0.4 ms)
   const size_t qn = 5 * (size_t)N;
+  std::vector<T> plain;
   if (dQ0 && c->adj_host_bytes < qn * sizeof(T)) {
     if (c->adj_host) cudaFreeHost(c->adj_host);
     c->adj_host_bytes = 0;
     if (cudaHostAlloc(&c->adj_host, qn * sizeof(T), cudaHostAllocDefault) != cudaSuccess) {
       cudaGetLastError();
       c->adj_host = nullptr;
-      return fail(c, LBCAD_E_OOM, "pinned host allocation failed");
+      plain.resize(qn);  // no page-locked memory left: the copy only takes longer
+    } else {
+      c->adj_host_bytes = qn * sizeof(T);
     }
-    c->adj_host_bytes = qn * sizeof(T);
   }
-  const T* hq = (const T*)c->adj_host;
-  if (dQ0) CK(c, cudaMemcpyAsync(c->adj_host, lcur.q, qn * sizeof(T), cudaMemcpyDeviceToHost, c->stream));
+  T* const hq = plain.empty() ? (T*)c->adj_host : plain.data();
+  if (dQ0) CK(c, cudaMemcpyAsync(hq, lcur.q, qn * sizeof(T), cudaMemcpyDeviceToHost, c->stream));
   CK(c, cudaStreamSynchronize(c->stream));
   if (dzeta) *dzeta = tot[0];
   if (dq0) *dq0 = tot[1];
