@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "lbcad_plan.h"
+
 namespace lbcad {
 
 // D3Q19 velocities (rest, six faces, twelve edges), the order published by
@@ -140,7 +142,6 @@ struct MarchDesc {
 // memory they stayed in registers (128^3 FP32: 88 us for k_march_fields instead of 107, and 122 for
 // k_march_lb instead of 148).  kPackMany instances fit a launch's argument space; larger batches take
 // several launches.
-constexpr int kPackMany = 28;
 template <typename T, int MI>
 struct InstPack {
   MarchDesc<T> d[MI];

@@ -87,7 +87,8 @@ struct lbcad_ctx {
   bool scratch_ready = false;
   MarchItem* items = nullptr;  // work items of the default path, all lists of all groups
   size_t items_cap = 0;
-  std::vector<StepWork> work;  // one per group of instances
+  StepPlan plan;               // the launches of a step and their scratch
+  std::vector<StepWork> work;  // one per launch of the plan
   std::vector<FusedObs> obs;
   std::vector<MarchDesc<float>> desc32[2];  // by step parity
   std::vector<MarchDesc<double>> desc64[2];
@@ -301,9 +302,6 @@ int upload_descs(lbcad_ctx* c);
 int prepare_fused(lbcad_ctx* c, int cfg_index);
 int ensure_scratch(lbcad_ctx* c);
 int default_shape(const lbcad_ctx* c);
-long long scratch_sites(const Inst& I);
-long long group_scratch(const lbcad_ctx* c, const StepWork& g);
-std::vector<StepWork> step_groups(const lbcad_ctx* c);
 
 int create_impl(int n, const lbcad_grid* grids, const lbcad_params* params, uint64_t seed, lbcad_ctx** out) {
   g_create_err.clear();
@@ -398,20 +396,14 @@ int create_impl(int n, const lbcad_grid* grids, const lbcad_params* params, uint
     if (te == cudaSuccess) te = cudaStreamSynchronize(c->stream);
     if (te != cudaSuccess) return bail(LBCAD_E_CUDA, std::string("trig table upload: ") + cudaGetErrorString(te));
   }
+  c->plan = plan_step(std::vector<lbcad_grid>(grids, grids + n), c->sync_split());
   if (!c->staged_only() && !c->sync_split()) {
-    // one scratch, which the groups use in turn
-    const std::vector<StepWork> groups = step_groups(c);
-    long long most = 0;
-    for (const StepWork& g : groups) most = std::max(most, group_scratch(c, g));
-    char* S = (char*)dev_alloc(c, 12 * (size_t)most * es);
+    // one scratch, which the launches use in turn
+    char* S = (char*)dev_alloc(c, 12 * (size_t)c->plan.scratch * es);
     if (!S) return bail(LBCAD_E_OOM, "device allocation failed");
-    for (const StepWork& g : groups) {
-      long long at = 0;
-      for (int i = g.first; i < g.first + g.ninst; ++i) {
-        c->inst[i].SN = scratch_sites(c->inst[i]);
-        c->inst[i].S = S + 12 * (size_t)at * es;
-        at += c->inst[i].SN;
-      }
+    for (int i = 0; i < n; ++i) {
+      c->inst[i].SN = c->plan.place[i].sites;
+      c->inst[i].S = S + 12 * (size_t)c->plan.place[i].at * es;
     }
   }
   c->obs_cnt = (unsigned*)dev_alloc(c, n * sizeof(unsigned));
@@ -507,50 +499,6 @@ int default_shape(const lbcad_ctx* c) {
   return square < wide ? 3 : 0;
 }
 
-// Sites whose scratch a launch of the Euler step may hold: a batch is launched in groups of at most that
-// many, a larger box in slabs of planes (the fields kernel then also works on the planes next to the slab).  At 12
-// values a site the scratch stays at 3.2 GB in FP32, where a scratch for every site would take a sixth of the
-// memory left for boxes as large as the device holds.
-constexpr long long kScratchSites = 1LL << 26;
-
-// Planes of the step's slabs of a box (nz: all at once).
-int slab_planes(const Inst& I) {
-  if (I.N <= kScratchSites) return I.g.nz;
-  const long long plane = (long long)I.g.nx * I.g.ny;
-  const int n = (int)std::max(8LL, kScratchSites / plane - 2);
-  return n + 2 < I.g.nz ? n : I.g.nz;
-}
-
-long long scratch_sites(const Inst& I) {
-  const int n = slab_planes(I);
-  return n < I.g.nz ? (long long)I.g.nx * I.g.ny * (n + 2) : I.N;
-}
-
-long long group_scratch(const lbcad_ctx* c, const StepWork& g) {
-  long long n = 0;
-  for (int i = g.first; i < g.first + g.ninst; ++i) n += scratch_sites(c->inst[i]);
-  return n;
-}
-
-// The launches' groups of instances, in order (without their work).
-std::vector<StepWork> step_groups(const lbcad_ctx* c) {
-  std::vector<StepWork> groups;
-  for (int i = 0; i < (int)c->inst.size(); ++i) {
-    if (!groups.empty()) {
-      StepWork& g = groups.back();
-      if (g.ninst < kPackMany && (c->sync_split() || group_scratch(c, g) + scratch_sites(c->inst[i]) <= kScratchSites)) {
-        ++g.ninst;
-        continue;
-      }
-    }
-    StepWork g;
-    g.first = i;
-    g.ninst = 1;
-    groups.push_back(g);
-  }
-  return groups;
-}
-
 // Largest step (sites) whose kernels are launched with programmatic dependent launch.
 constexpr long long kEarlySites = 1 << 20;
 
@@ -625,18 +573,14 @@ int prepare_fused(lbcad_ctx* c, int cfg_index) {
   auto blocks = [&](int per_sm) { return sms * (per_sm > 0 ? per_sm : 1); };
   std::vector<MarchItem> t;
   std::vector<StepWork> work;
-  for (const StepWork& g : step_groups(c)) {
-    const Inst& I = c->inst[g.first];
-    const int nz = I.g.nz, n = g.ninst == 1 && !split ? slab_planes(I) : nz;
-    for (int z = 0; z == 0 || (n < nz && z < nz); z += n) {
-      work.push_back(g);
-      StepWork& w = work.back();
-      const bool whole = n >= nz;
-      const int zn = std::min(n, nz - z);
-      if (!whole) w.sz0 = (z + nz - 1) % nz;
-      w.fields = add_items(c, w, cfg.fx, cfg.fy, blocks(cfg.fields_per_sm), t, whole ? 0 : z - 1, whole ? 0 : zn + 2);
-      w.lb = add_items(c, w, cfg.lx, cfg.ly, blocks(cfg.lb_per_sm), t, whole ? 0 : z, whole ? 0 : zn);
-    }
+  for (const StepPart& part : c->plan.parts) {
+    StepWork w;
+    w.first = part.first;
+    w.ninst = part.ninst;
+    w.sz0 = part.sz0;
+    w.fields = add_items(c, w, cfg.fx, cfg.fy, blocks(cfg.fields_per_sm), t, part.fz, part.fn);
+    w.lb = add_items(c, w, cfg.lx, cfg.ly, blocks(cfg.lb_per_sm), t, part.lz, part.ln);
+    work.push_back(w);
   }
   for (StepWork& g : work) {
     if (split) {
