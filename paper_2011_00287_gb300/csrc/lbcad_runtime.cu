@@ -86,7 +86,7 @@ struct lbcad_ctx {
   int stencil = LBCAD_STENCIL_ISO;
   bool scratch_ready = false;
   MarchItem* items = nullptr;  // work items of the default path, all lists of all groups
-  size_t items_cap = 0;
+  size_t items_cap = 0;        // bytes, as the other capacities
   StepPlan plan;               // the launches of a step and their scratch
   std::vector<StepWork> work;  // one per launch of the plan
   std::vector<FusedObs> obs;
@@ -148,6 +148,18 @@ void* dev_alloc(lbcad_ctx* c, size_t bytes) {
   }
   if (p) c->allocs.push_back(p);
   return p;
+}
+
+// Makes `p` hold at least `bytes`: a larger buffer replaces it (the old one stays with the context until it is
+// destroyed).  If there is none, p and its capacity stay as they were.
+template <typename P>
+bool grow(lbcad_ctx* c, P*& p, size_t& cap, size_t bytes) {
+  if (bytes <= cap) return true;
+  P* q = (P*)dev_alloc(c, bytes);
+  if (!q) return false;
+  p = q;
+  cap = bytes;
+  return true;
 }
 
 // Buffer i of lbcad_adjoint: the one of an earlier call if it is large enough, else a new one
@@ -556,6 +568,11 @@ MarchWork add_items(const lbcad_ctx* c, const StepWork& g, int tx, int ty, int b
   return w;
 }
 
+void drop_graph(lbcad_ctx* c) {
+  if (c->gexec) { cudaGraphExecDestroy(c->gexec); c->gexec = nullptr; }
+  if (c->graph) { cudaGraphDestroy(c->graph); c->graph = nullptr; }
+}
+
 // Work items of the default path for tile shape `cfg_index`, and the slots of its a6 sums.
 int prepare_fused(lbcad_ctx* c, int cfg_index) {
   FusedCfg cfg;
@@ -634,21 +651,11 @@ int prepare_fused(lbcad_ctx* c, int cfg_index) {
       for (size_t k = obs.size(); k > 0 && work[k - 1].first == g.first; --k) obs[k - 1].total = ob.slot0 + grid;
     nslots += n;
   }
-  if (t.size() > c->items_cap) {
-    c->items = (MarchItem*)dev_alloc(c, t.size() * sizeof(MarchItem));
-    if (!c->items) return fail(c, LBCAD_E_OOM, "work list allocation failed");
-    c->items_cap = t.size();
-  }
-  if (nslots * 12 > c->obs_slots_cap) {
-    c->obs_slots = (double*)dev_alloc(c, nslots * 12 * sizeof(double));
-    if (!c->obs_slots) return fail(c, LBCAD_E_OOM, "a6 slot allocation failed");
-    c->obs_slots_cap = nslots * 12;
-  }
-  if (map.size() > c->obs_map_cap) {
-    c->obs_map = (int*)dev_alloc(c, map.size() * sizeof(int));
-    if (!c->obs_map) return fail(c, LBCAD_E_OOM, "a6 slot map allocation failed");
-    c->obs_map_cap = map.size();
-  }
+  // the launches in use keep their lists until all of the new ones have a place
+  if (!grow(c, c->items, c->items_cap, t.size() * sizeof(MarchItem)) ||
+      !grow(c, c->obs_slots, c->obs_slots_cap, nslots * 12 * sizeof(double)) ||
+      !grow(c, c->obs_map, c->obs_map_cap, map.size() * sizeof(int)))
+    return fail(c, LBCAD_E_OOM, "work list allocation failed");
   auto place = [](auto*& p, void* base) { p = (std::remove_reference_t<decltype(p)>)((char*)base + (size_t)p); };
   for (size_t i = 0; i < work.size(); ++i) {
     StepWork& g = work[i];
@@ -662,6 +669,7 @@ int prepare_fused(lbcad_ctx* c, int cfg_index) {
     ob.cnt = c->obs_cnt + g.first;
     ob.latest = c->obs_latest + 12 * (size_t)g.first;
   }
+  drop_graph(c);  // a captured step reads the lists that change here
   CK(c, cudaMemcpyAsync(c->items, t.data(), t.size() * sizeof(MarchItem), cudaMemcpyHostToDevice, c->stream));
   CK(c, cudaMemcpyAsync(c->obs_map, map.data(), map.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   // the kernels leave the per-instance counters at zero; reset them here as well, so that a
@@ -690,11 +698,6 @@ cudaError_t launch_fused(lbcad_ctx* c, int par) {
   };
   return c->prec == LBCAD_FP64 ? run(LaunchFused<double, false>{}, c->desc64[par])
                                : run(LaunchFused<float, true>{}, c->desc32[par]);
-}
-
-void drop_graph(lbcad_ctx* c) {
-  if (c->gexec) { cudaGraphExecDestroy(c->gexec); c->gexec = nullptr; }
-  if (c->graph) { cudaGraphDestroy(c->graph); c->graph = nullptr; }
 }
 
 int launch_steps(lbcad_ctx* c, int64_t n) {
@@ -806,6 +809,7 @@ int lbcad_autotune(lbcad_ctx* c, int32_t reps, int32_t* chosen, float* ms_per_cf
   const int n = (c->prec == LBCAD_FP64) ? LaunchFused<double, false>::num_configs()
                                         : LaunchFused<float, true>::num_configs();
   const int par = (int)(c->step & 1);
+  const int before = c->cfg_index;
   cudaEvent_t e0, e1;
   CK(c, cudaEventCreate(&e0));
   CK(c, cudaEventCreate(&e1));
@@ -814,10 +818,16 @@ int lbcad_autotune(lbcad_ctx* c, int32_t reps, int32_t* chosen, float* ms_per_cf
   // so a drift of the clocks during tuning does not favour one of them)
   constexpr int kRounds = 3;
   std::vector<float> best_of(n, -1.f);
-  for (int round = 0; round < kRounds; ++round) {
-    for (int k = 0; k < n; ++k) {
+  int code = LBCAD_OK;
+  for (int round = 0; round < kRounds && code == LBCAD_OK; ++round) {
+    for (int k = 0; k < n && code == LBCAD_OK; ++k) {
       if (round > 0 && best_of[k] < 0.f) continue;  // does not fit
-      if (prepare_fused(c, k) != LBCAD_OK) continue;
+      code = prepare_fused(c, k);
+      if (code == LBCAD_E_UNSUPPORTED || code == LBCAD_E_OOM) {  // no such shape, or no memory for its lists
+        code = LBCAD_OK;
+        continue;
+      }
+      if (code != LBCAD_OK) break;
       float ms = -1.f;
       cudaError_t e = launch_fused(c, par);
       if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
@@ -825,12 +835,8 @@ int lbcad_autotune(lbcad_ctx* c, int32_t reps, int32_t* chosen, float* ms_per_cf
       if (e == cudaSuccess) e = cudaEventRecord(e1, c->stream);
       if (e == cudaSuccess) e = cudaEventSynchronize(e1);
       if (e == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess) ms /= reps;
-      if (e != cudaSuccess) {
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-        return fail(c, LBCAD_E_CUDA, std::string("autotune: ") + cudaGetErrorString(e));
-      }
-      if (best_of[k] < 0.f || ms < best_of[k]) best_of[k] = ms;
+      if (e != cudaSuccess) code = fail(c, LBCAD_E_CUDA, std::string("autotune: ") + cudaGetErrorString(e));
+      else if (best_of[k] < 0.f || ms < best_of[k]) best_of[k] = ms;
     }
   }
   cudaEventDestroy(e0);
@@ -838,12 +844,17 @@ int lbcad_autotune(lbcad_ctx* c, int32_t reps, int32_t* chosen, float* ms_per_cf
   int best = -1;
   for (int k = 0; k < n; ++k) {
     if (best_of[k] >= 0.f && (best < 0 || best_of[k] < best_of[best])) best = k;
-    if (ms_per_cfg && k < ncfg) ms_per_cfg[k] = best_of[k];
+    if (code == LBCAD_OK && ms_per_cfg && k < ncfg) ms_per_cfg[k] = best_of[k];
   }
-  if (best < 0) return fail(c, LBCAD_E_UNSUPPORTED, "no fused tile shape fits");
+  if (code == LBCAD_OK && best < 0) code = fail(c, LBCAD_E_UNSUPPORTED, "no fused tile shape fits");
+  if (code != LBCAD_OK) {
+    const std::string why = c->err;
+    prepare_fused(c, before);
+    c->err = why;
+    return code;
+  }
   int r = prepare_fused(c, best);
   if (r) return r;
-  drop_graph(c);
   if (chosen) *chosen = best;
   return LBCAD_OK;
 }
@@ -856,10 +867,7 @@ int lbcad_set_tiles(lbcad_ctx* c, int32_t cfg) {
   const int n = (c->prec == LBCAD_FP64) ? LaunchFused<double, false>::num_configs()
                                         : LaunchFused<float, true>::num_configs();
   if (cfg < 0 || cfg >= n) return fail(c, LBCAD_E_INVALID_ARG, "tile shape index out of range");
-  int r = prepare_fused(c, cfg);
-  if (r) return r;
-  drop_graph(c);
-  return LBCAD_OK;
+  return prepare_fused(c, cfg);
 }
 
 int lbcad_set_observe(lbcad_ctx* c, int32_t on) {
