@@ -160,8 +160,9 @@ int lbcad_step(lbcad_ctx* c, int64_t n);
 
 /* Kernel path of lbcad_step.  LBCAD_PATH_FUSED (default): two kernels per step that march up z through
  * shared-memory tiles (fields, stress and the update of Q; then force, populations, psi and the sums),
- * with 12 values per site of scratch allocated at create (for at most 2^26 sites at a time: groups of a batch's
- * instances and slabs of a larger box use it in turn).  LBCAD_PATH_TWO_KERNEL: a stencil kernel writing
+ * with 12 values per site of scratch allocated at create (for 2^26 sites at most, or ten planes of a box where these
+ * are more: groups of a batch's instances and slabs of a larger box use it in turn; where there is no memory for that
+ * much, for fewer, down to three planes of the largest box, in more launches).  LBCAD_PATH_TWO_KERNEL: a stencil kernel writing
  * H, mu and sigma to a per-site scratch (allocated on the first switch, 15 values per
  * site) and an update kernel, one thread per site; same arithmetic, kept as a cross-check.  Changing the path
  * drops a captured graph. */

@@ -408,10 +408,17 @@ int create_impl(int n, const lbcad_grid* grids, const lbcad_params* params, uint
     if (te == cudaSuccess) te = cudaStreamSynchronize(c->stream);
     if (te != cudaSuccess) return bail(LBCAD_E_CUDA, std::string("trig table upload: ") + cudaGetErrorString(te));
   }
-  c->plan = plan_step(std::vector<lbcad_grid>(grids, grids + n), c->sync_split());
+  const std::vector<lbcad_grid> boxes(grids, grids + n);
+  c->plan = plan_step(boxes, c->sync_split());
   if (!c->staged_only() && !c->sync_split()) {
-    // one scratch, which the launches use in turn
+    // one scratch, which the launches use in turn; near the end of the memory a smaller one, for more launches
     char* S = (char*)dev_alloc(c, 12 * (size_t)c->plan.scratch * es);
+    for (ScratchRule rule; !S && !rule.tightest();) {
+      rule = rule.tighter();
+      const long long before = c->plan.scratch;
+      c->plan = plan_step(boxes, false, rule);
+      if (c->plan.scratch < before) S = (char*)dev_alloc(c, 12 * (size_t)c->plan.scratch * es);
+    }
     if (!S) return bail(LBCAD_E_OOM, "device allocation failed");
     for (int i = 0; i < n; ++i) {
       c->inst[i].SN = c->plan.place[i].sites;

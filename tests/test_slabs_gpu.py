@@ -1,4 +1,4 @@
-"""The step in slabs: boxes above 2^26 sites, and batches that hold one.
+"""The step in slabs: boxes above 2^26 sites, batches that hold one, and boxes whose whole scratch finds no memory.
 
 The arithmetic of a site does not depend on how the step is divided, so every comparison is bit for bit.  The
 states vary everywhere (small noise on every field), so that a plane that is missing, stale or taken from the wrong
@@ -8,14 +8,15 @@ import numpy as np
 import pytest
 
 import paper_2011_00287_gb300 as L
+from paper_2011_00287_gb300 import lbcad as B
 
 pytestmark = pytest.mark.gpu
 
 
 @pytest.fixture(scope="module", autouse=True)
 def built():
-    from paper_2011_00287_gb300 import build as B
-    B.build()
+    from paper_2011_00287_gb300 import build
+    build.build()
 
 
 def _noise(shape, prec, seed, q=19):
@@ -27,7 +28,7 @@ def _noise(shape, prec, seed, q=19):
     dt = torch.float64 if prec == L.FP64 else torch.float32
     s = torch.empty((q + 9) * n, dtype=dt, device="cuda:0")
     at = 0
-    _, w = L.lattice()
+    _, w = L.lattice(L.D3Q15 if q == 15 else L.D3Q19)
     for comps, amp in ((q, 1e-4), (5, 0.02), (1, 0.3), (3, 1e-3)):
         s[at:at + comps * n].uniform_(-amp, amp, generator=gen)
         at += comps * n
@@ -66,3 +67,71 @@ def test_batch_with_a_box_in_slabs_steps_each_box_as_alone(order):
         assert torch.equal(got[k][0], ref), shapes[i]
         # the same FP64 sums of the same state, in another order: rounding of n terms of order one
         assert np.abs(got[k][1] - sums).max() <= 1e-12 * np.prod(shapes[i]), shapes[i]
+
+
+class _Bounded(B._TorchAllocator):
+    """Refuses every request above `most` bytes that is not a buffer of a state."""
+    most, keep, refused = 0, (), 0
+
+    def _alloc(self, nbytes, user):
+        if self.most and nbytes > self.most and nbytes not in self.keep:
+            type(self).refused += 1
+            return None
+        return super()._alloc(nbytes, user)
+
+
+def _bound(monkeypatch, shapes, prec, q, planes):
+    """No scratch of more than `planes` planes of the first box; buffers of the state as they are."""
+    es = 8 if prec == L.FP64 else 4
+    keep = set()
+    for s in shapes:
+        n = s[0] * s[1] * s[2]
+        keep |= {(c * n * es + 255) // 256 * 256 for c in (q, 5, 1, 3)}
+    monkeypatch.setattr(_Bounded, "keep", keep)
+    # (requests come in multiples of 256 bytes)
+    monkeypatch.setattr(_Bounded, "most", (planes * 12 * es * shapes[0][0] * shapes[0][1] + 255) // 256 * 256)
+    monkeypatch.setattr(_Bounded, "refused", 0)
+    monkeypatch.setattr(B, "_TorchAllocator", _Bounded)
+
+
+@pytest.mark.parametrize("prec", [L.FP64, L.FP32], ids=["fp64", "fp32"])
+@pytest.mark.parametrize("planes", [3, 8, 25])
+@pytest.mark.parametrize("shapes,kw", [
+    ([(64, 52, 40)], {}), ([(67, 49, 41), (9, 7, 6), (33, 31, 30)], {}), ([(64, 52, 40)], dict(lattice=L.D3Q15)),
+], ids=["box", "batch", "d3q15"])
+def test_step_with_less_scratch_is_the_same_step(monkeypatch, shapes, kw, planes, prec):
+    """Where the scratch of whole boxes finds no memory, smaller slabs step them; so a box that fitted before there was
+    a scratch still fits.  The seams lie anywhere in the noise of the state."""
+    import torch
+    q = 15 if kw else 19
+    kw = dict(kw, tau=1.5)
+    states = [_noise(s, prec, 21 + i, q) for i, s in enumerate(shapes)]
+    ref = _run(shapes, states, prec, 4, **kw)
+    _bound(monkeypatch, shapes, prec, q, planes)
+    got = _run(shapes, states, prec, 4, **kw)
+    assert _Bounded.refused > 0
+    for s, (a, sums_a), (b, sums_b) in zip(shapes, got, ref):
+        assert torch.isfinite(b).all() and torch.equal(a, b), s
+        assert np.abs(sums_a - sums_b).max() <= 1e-12 * np.prod(s), s
+
+
+def test_adjoint_with_less_scratch_is_the_same(monkeypatch):
+    """The replay of the adjoint steps in the same slabs."""
+    shape = (40, 36, 33)
+
+    def grad():
+        sim = L.Simulation([shape], [L.default_params(shape, R=9.0, p0=12.0, zeta=0.02)], seed=3)
+        out = sim.adjoint(7, 3)
+        sim.close()
+        return out
+
+    ref = grad()
+    n = int(np.prod(shape))
+    _bound(monkeypatch, [shape], L.FP32, 19, 8)
+    # and the adjoint's own: checkpoints, segment, cotangents, work, forces
+    sizes = {(v * n * 4 + 255) // 256 * 256 for v in (3 * 28, 4 * 28, 2 * 28, 56, 9)}
+    monkeypatch.setattr(_Bounded, "keep", _Bounded.keep | sizes)
+    got = grad()
+    assert _Bounded.refused > 0
+    assert np.array_equal(got[3], ref[3])
+    np.testing.assert_allclose(got[:3], ref[:3], rtol=1e-9)

@@ -17,8 +17,8 @@ def plan(tmp_path_factory):
                     "-I" + os.path.join(ROOT, "include"), "-I" + os.path.join(ROOT, "paper_2011_00287_gb300", "csrc"),
                     os.path.join(ROOT, "tests", "step_plan_main.cpp"), "-o", exe], check=True)
 
-    def run(boxes, split=False):
-        text = "%d %d\n%s\n" % (split, len(boxes), "\n".join("%d %d %d" % tuple(b) for b in boxes))
+    def run(boxes, split=False, tighter=0):
+        text = "%d %d %d\n%s\n" % (split, tighter, len(boxes), "\n".join("%d %d %d" % tuple(b) for b in boxes))
         out = subprocess.run([exe], input=text, capture_output=True, text=True, check=True).stdout.split("\n")
         scratch, parts = (int(v) for v in out[0].split())
         rows = [tuple(int(v) for v in line.split()) for line in out[1:-1]]
@@ -72,6 +72,20 @@ def test_random_batches(plan):
     for _ in range(60):
         boxes = [tuple(rng.choice((4, 7, 32, 96, 300, 700, 1200)) for _ in range(3)) for _ in range(rng.randint(1, 40))]
         _check(boxes, *plan(boxes))
+
+
+@pytest.mark.parametrize("boxes", [[LARGE, (32, 32, 32)], [(64, 48, 40), (9, 7, 6), (5, 4, 4)], [(8192, 8192, 18)],
+                                   [(4, 4, 4)], [(1024, 1024, 1024)]])
+def test_smaller_scratch_for_more_launches(plan, boxes):
+    """Each step down needs no more scratch than the one before, the last no more than three planes of the largest box;
+    every one of them steps every plane once, within its scratch."""
+    sizes = []
+    for tighter in range(14):
+        out = plan(boxes, tighter=tighter)
+        _check(boxes, *out)
+        sizes.append(out[0])
+    assert sizes == sorted(sizes, reverse=True)
+    assert sizes[-1] == 3 * max(b[0] * b[1] for b in boxes)
 
 
 def test_split_steps_take_whole_boxes(plan):
