@@ -150,6 +150,12 @@ void* dev_alloc(lbcad_ctx* c, size_t bytes) {
   return p;
 }
 
+// Gives one allocation of the context back, with no work on it in flight.
+void dev_free(lbcad_ctx* c, void* p) {
+  c->allocs.erase(std::find(c->allocs.begin(), c->allocs.end(), p));
+  if (c->free) c->free(p, c->user); else cudaFree(p);
+}
+
 // Makes `p` hold at least `bytes`: a larger buffer replaces it (the old one stays with the context until it is
 // destroyed).  If there is none, p and its capacity stay as they were.
 template <typename P>
@@ -408,23 +414,6 @@ int create_impl(int n, const lbcad_grid* grids, const lbcad_params* params, uint
     if (te == cudaSuccess) te = cudaStreamSynchronize(c->stream);
     if (te != cudaSuccess) return bail(LBCAD_E_CUDA, std::string("trig table upload: ") + cudaGetErrorString(te));
   }
-  const std::vector<lbcad_grid> boxes(grids, grids + n);
-  c->plan = plan_step(boxes, c->sync_split());
-  if (!c->staged_only() && !c->sync_split()) {
-    // one scratch, which the launches use in turn; near the end of the memory a smaller one, for more launches
-    char* S = (char*)dev_alloc(c, 12 * (size_t)c->plan.scratch * es);
-    for (ScratchRule rule; !S && !rule.tightest();) {
-      rule = rule.tighter();
-      const long long before = c->plan.scratch;
-      c->plan = plan_step(boxes, false, rule);
-      if (c->plan.scratch < before) S = (char*)dev_alloc(c, 12 * (size_t)c->plan.scratch * es);
-    }
-    if (!S) return bail(LBCAD_E_OOM, "device allocation failed");
-    for (int i = 0; i < n; ++i) {
-      c->inst[i].SN = c->plan.place[i].sites;
-      c->inst[i].S = S + 12 * (size_t)c->plan.place[i].at * es;
-    }
-  }
   c->obs_cnt = (unsigned*)dev_alloc(c, n * sizeof(unsigned));
   c->obs_latest = (double*)dev_alloc(c, (size_t)n * 12 * sizeof(double));
   if (!c->obs_cnt || !c->obs_latest) return bail(LBCAD_E_OOM, "device allocation failed");
@@ -441,8 +430,31 @@ int create_impl(int n, const lbcad_grid* grids, const lbcad_params* params, uint
   c->obs_partial = (double*)dev_alloc(c, kObsMaxBlocks * 12 * sizeof(double));
   c->obs_out = (double*)dev_alloc(c, 12 * sizeof(double));
   if (!c->obs_partial || !c->obs_out) return bail(LBCAD_E_OOM, "device allocation failed");
-  if (upload_descs(c) != LBCAD_OK) return bail(LBCAD_E_CUDA, "");
-  if ((code = prepare_fused(c, default_shape(c))) != LBCAD_OK) return bail(code, "");
+  // last, the scratch of the Euler step, which its launches use in turn, and their work lists; near the end of the
+  // memory a smaller one, for more launches
+  const std::vector<lbcad_grid> boxes(grids, grids + n);
+  const bool scratch = !c->staged_only() && !c->sync_split();
+  long long before = 0;  // the scratch that did not fit
+  for (ScratchRule rule;; rule = rule.tighter()) {
+    c->plan = plan_step(boxes, c->sync_split(), rule);
+    code = LBCAD_E_OOM;
+    if (before == 0 || c->plan.scratch < before) {
+      char* S = scratch ? (char*)dev_alloc(c, 12 * (size_t)c->plan.scratch * es) : nullptr;
+      if (!scratch || S) {
+        for (int i = 0; i < n && scratch; ++i) {
+          c->inst[i].SN = c->plan.place[i].sites;
+          c->inst[i].S = S + 12 * (size_t)c->plan.place[i].at * es;
+        }
+        if (upload_descs(c) != LBCAD_OK) return bail(LBCAD_E_CUDA, "");
+        code = prepare_fused(c, default_shape(c));
+      }
+      if (code == LBCAD_OK) break;
+      if (code != LBCAD_E_OOM || !scratch) return bail(code, "");
+      if (S) dev_free(c, S);
+      before = c->plan.scratch;
+    }
+    if (rule.tightest()) return bail(code, c->err.empty() ? "device allocation failed" : "");
+  }
   if (c->staged_only() || c->sync_split()) {
     if ((code = ensure_scratch(c)) != LBCAD_OK) return bail(code, "");
   }

@@ -135,3 +135,41 @@ def test_adjoint_with_less_scratch_is_the_same(monkeypatch):
     assert _Bounded.refused > 0
     assert np.array_equal(got[3], ref[3])
     np.testing.assert_allclose(got[:3], ref[:3], rtol=1e-9)
+
+
+class _Budget(B._TorchAllocator):
+    """Gives out at most `total` bytes at a time."""
+    total, asked = None, 0
+
+    def _alloc(self, nbytes, user):
+        held = sum(t.numel() for t in self.live.values())
+        if self.total is not None and held + nbytes > self.total:
+            return None
+        type(self).asked = max(self.asked, held + nbytes)
+        return super()._alloc(nbytes, user)
+
+
+@pytest.mark.parametrize("prec", [L.FP64, L.FP32], ids=["fp64", "fp32"])
+@pytest.mark.parametrize("shapes", [[(64, 52, 40)], [(67, 49, 41), (9, 7, 6), (33, 31, 30)]], ids=["box", "batch"])
+def test_create_wherever_the_scratch_meets_the_end_of_the_memory(monkeypatch, shapes, prec):
+    """The scratch leaves room for what is allocated besides it: a context is created in every budget between the one
+    with the whole scratch and one with three planes of it, the one that only the last work list exceeds included."""
+    import torch
+    monkeypatch.setattr(B, "_TorchAllocator", _Budget)
+    monkeypatch.setattr(_Budget, "asked", 0)
+    states = [_noise(s, prec, 31 + i) for i, s in enumerate(shapes)]
+    ref = _run(shapes, states, prec, 3)
+    whole, es = _Budget.asked, 8 if prec == L.FP64 else 4
+    scratch = 12 * es * sum(int(np.prod(s)) for s in shapes)
+    # (three planes of the largest box, and lists of one-plane slabs: at most 20 bytes an item, 96 a slot)
+    least = whole - scratch + 3 * 12 * es * shapes[0][0] * shapes[0][1] + (1 << 20)
+    assert least < whole
+    for total in (whole - 1, whole - 256, whole - 4096, whole - scratch // 8, (whole + least) // 2, least):
+        monkeypatch.setattr(_Budget, "total", total)
+        got = _run(shapes, states, prec, 3)
+        for s, (a, _), (b, _) in zip(shapes, got, ref):
+            assert torch.equal(a, b), (s, total)
+    monkeypatch.setattr(_Budget, "total", whole - scratch)
+    with pytest.raises(B.LbcadError) as e:
+        _run(shapes, states, prec, 3)
+    assert e.value.code == B.LBCAD_E_OOM
