@@ -221,3 +221,31 @@ def test_fp32_fused_sums_are_the_fp64_sums_of_the_state(tiles):
     assert abs(o[0] - prev[0]) <= 1e-12 * prev[0] and abs(o[0] - cur[0]) <= 1e-12 * cur[0], (o[0], prev[0], cur[0])
     assert np.abs(o[2:5] - cur[2:5]).max() <= 1e-12 * N, (o[2:5], cur[2:5])
     sim.close()
+
+
+@pytest.mark.parametrize("tiles", range(L.lbcad.N_TILE_CONFIGS))
+@pytest.mark.parametrize("shape", [(21, 13, 10), (70, 9, 7), (4, 5, 6)])
+def test_sums_of_every_tile_shape(shape, tiles):
+    """Each shape lays out its blocks' sums in shared memory by its own number of threads (64 to 256)."""
+    sim = L.Simulation([shape], [_lib_params(shape, L.FP32, R=5.0, p0=8.0, zeta=0.01)], seed=3)
+    sim.set_tiles(tiles)
+    sim.step(5)
+    a, b, ag = _fused_and_separate(sim, 0)
+    _check(a, b, sim.sites(0), False, ag)
+
+
+@pytest.mark.parametrize("prec,tiles", [(L.FP32, 0), (L.FP32, 6), (L.FP64, 0)], ids=["fp32", "fp32-8x8", "fp64"])
+def test_sums_of_a_batch_whose_blocks_work_on_several_boxes(prec, tiles):
+    """28 boxes of about 64^3 in one launch: more items than resident blocks (at 8x8, 72 columns of two slabs or more
+    a box, at most eight blocks on each of 152 SMs), so a block goes from one box to another and keeps a slot for each."""
+    shapes = [(66 - i % 4, 61 + i % 3, 58 + i % 5) for i in range(28)]
+    sim = L.Simulation(shapes, [_lib_params(s, prec, R=15.0, p0=16.0, zeta=0.001 * (1 + i))
+                                for i, s in enumerate(shapes)], seed=6)
+    sim.set_tiles(tiles)
+    sim.step(4)
+    fused = [sim.observables(i) for i in range(28)]  # (setting a state ends the fused sums of all boxes)
+    for i in range(28):
+        st = sim.get_state(i)
+        sim.set_state(i, st)
+        g = st.view(np.float32 if prec == L.FP32 else np.float64)[:19 * sim.sites(i)]
+        _check(fused[i], sim.observables(i), sim.sites(i), prec == L.FP64, float(np.abs(g.astype(np.float64)).sum()))
