@@ -77,7 +77,9 @@ typedef struct {
 } lbcad_grid;
 
 /* Device allocator callbacks: alloc returns a device pointer aligned to >= 256 bytes or
- * NULL; free releases it.  Both are called only from lbcad_create* / lbcad_destroy. */
+ * NULL; free releases it.  alloc is called from lbcad_create* and from a call that needs a buffer it has not had
+ * before (another path or tile shape, fields exchanged with the host, the adjoint); free from lbcad_destroy and, where
+ * alloc has returned NULL, to exchange the step's scratch for a smaller one (see lbcad_set_path). */
 typedef void* (*lbcad_alloc_fn)(size_t bytes, void* user);
 typedef void (*lbcad_free_fn)(void* ptr, void* user);
 
@@ -162,7 +164,7 @@ int lbcad_step(lbcad_ctx* c, int64_t n);
  * shared-memory tiles (fields, stress and the update of Q; then force, populations, psi and the sums),
  * with 12 values per site of scratch allocated at create (for 2^26 sites at most, or ten planes of a box where these
  * are more: groups of a batch's instances and slabs of a larger box use it in turn; where there is no memory for that
- * much, for fewer, down to three planes of the largest box, in more launches).  LBCAD_PATH_TWO_KERNEL: a stencil kernel writing
+ * much, or a later call needs some of it, for fewer, down to three planes of the largest box, in more launches).  LBCAD_PATH_TWO_KERNEL: a stencil kernel writing
  * H, mu and sigma to a per-site scratch (allocated on the first switch, 15 values per
  * site) and an update kernel, one thread per site; same arithmetic, kept as a cross-check.  Changing the path
  * drops a captured graph. */

@@ -88,6 +88,8 @@ struct lbcad_ctx {
   MarchItem* items = nullptr;  // work items of the default path, all lists of all groups
   size_t items_cap = 0;        // bytes, as the other capacities
   StepPlan plan;               // the launches of a step and their scratch
+  ScratchRule rule;            // the bound on the scratch that the plan was made for
+  char* scratch = nullptr;     // of the Euler step, which its launches use in turn
   std::vector<StepWork> work;  // one per launch of the plan
   std::vector<FusedObs> obs;
   std::vector<MarchDesc<float>> desc32[2];  // by step parity
@@ -317,6 +319,9 @@ int upload_init(lbcad_ctx* c, Inst& I, uint64_t seed, int idx) {
 }
 
 int upload_descs(lbcad_ctx* c);
+std::vector<lbcad_grid> boxes_of(const lbcad_ctx* c);
+bool place_scratch(lbcad_ctx* c);
+void drop_scratch(lbcad_ctx* c);
 int prepare_fused(lbcad_ctx* c, int cfg_index);
 int ensure_scratch(lbcad_ctx* c);
 int default_shape(const lbcad_ctx* c);
@@ -430,30 +435,24 @@ int create_impl(int n, const lbcad_grid* grids, const lbcad_params* params, uint
   c->obs_partial = (double*)dev_alloc(c, kObsMaxBlocks * 12 * sizeof(double));
   c->obs_out = (double*)dev_alloc(c, 12 * sizeof(double));
   if (!c->obs_partial || !c->obs_out) return bail(LBCAD_E_OOM, "device allocation failed");
-  // last, the scratch of the Euler step, which its launches use in turn, and their work lists; near the end of the
-  // memory a smaller one, for more launches
-  const std::vector<lbcad_grid> boxes(grids, grids + n);
+  // last, the scratch of the Euler step and the work lists; near the end of the memory a smaller scratch, for more
+  // launches
   const bool scratch = !c->staged_only() && !c->sync_split();
   long long before = 0;  // the scratch that did not fit
-  for (ScratchRule rule;; rule = rule.tighter()) {
-    c->plan = plan_step(boxes, c->sync_split(), rule);
-    code = LBCAD_E_OOM;
+  for (;; c->rule = c->rule.tighter()) {
+    c->plan = plan_step(boxes_of(c), !scratch, c->rule);
     if (before == 0 || c->plan.scratch < before) {
-      char* S = scratch ? (char*)dev_alloc(c, 12 * (size_t)c->plan.scratch * es) : nullptr;
-      if (!scratch || S) {
-        for (int i = 0; i < n && scratch; ++i) {
-          c->inst[i].SN = c->plan.place[i].sites;
-          c->inst[i].S = S + 12 * (size_t)c->plan.place[i].at * es;
-        }
+      code = LBCAD_E_OOM;
+      if (!scratch || place_scratch(c)) {
         if (upload_descs(c) != LBCAD_OK) return bail(LBCAD_E_CUDA, "");
         code = prepare_fused(c, default_shape(c));
       }
       if (code == LBCAD_OK) break;
       if (code != LBCAD_E_OOM || !scratch) return bail(code, "");
-      if (S) dev_free(c, S);
+      drop_scratch(c);
       before = c->plan.scratch;
     }
-    if (rule.tightest()) return bail(code, c->err.empty() ? "device allocation failed" : "");
+    if (c->rule.tightest()) return bail(LBCAD_E_OOM, "device allocation failed");
   }
   if (c->staged_only() || c->sync_split()) {
     if ((code = ensure_scratch(c)) != LBCAD_OK) return bail(code, "");
@@ -492,14 +491,72 @@ int upload_descs(lbcad_ctx* c) {
   return LBCAD_OK;
 }
 
+std::vector<lbcad_grid> boxes_of(const lbcad_ctx* c) {
+  std::vector<lbcad_grid> b;
+  for (const Inst& I : c->inst) b.push_back(I.g);
+  return b;
+}
+
+// Allocates the scratch of the plan and gives every instance its place in it; false: no memory.
+bool place_scratch(lbcad_ctx* c) {
+  c->scratch = (char*)dev_alloc(c, 12 * (size_t)c->plan.scratch * c->elem());
+  if (!c->scratch) return false;
+  for (size_t i = 0; i < c->inst.size(); ++i) {
+    c->inst[i].SN = c->plan.place[i].sites;
+    c->inst[i].S = c->scratch + 12 * (size_t)c->plan.place[i].at * c->elem();
+  }
+  return true;
+}
+
+void drop_scratch(lbcad_ctx* c) {
+  if (c->scratch) dev_free(c, c->scratch);
+  c->scratch = nullptr;
+}
+
+// Before a step of the default path.  The scratch is missing only where another owner of the memory took its place
+// while shrink_scratch had given it back.
+int ensure_step_scratch(lbcad_ctx* c) {
+  if (c->scratch || c->staged_only() || c->sync_split()) return LBCAD_OK;
+  if (!place_scratch(c)) return fail(c, LBCAD_E_OOM, "scratch allocation failed");
+  return upload_descs(c);
+}
+
+// A smaller scratch for the step, in more launches, where another call needs its memory: it holds something only while
+// a step runs.  False: it is as small as it gets, or there is no memory for the lists of more launches.
+bool shrink_scratch(lbcad_ctx* c) {
+  if (!c->scratch || cudaStreamSynchronize(c->stream) != cudaSuccess) return false;
+  const StepPlan plan = c->plan;
+  ScratchRule rule = c->rule;
+  do {
+    if (rule.tightest()) {
+      c->plan = plan;
+      return false;
+    }
+    rule = rule.tighter();
+    c->plan = plan_step(boxes_of(c), false, rule);
+  } while (c->plan.scratch >= plan.scratch);
+  drop_scratch(c);
+  const bool smaller = prepare_fused(c, c->cfg_index) == LBCAD_OK;
+  if (smaller) c->rule = rule;
+  else c->plan = plan;  // of the lists still in use
+  return ensure_step_scratch(c) == LBCAD_OK && smaller;
+}
+
+// dev_alloc for a call after lbcad_create, which may take memory from the step's scratch.
+void* dev_alloc_or_shrink(lbcad_ctx* c, size_t bytes) {
+  void* p = dev_alloc(c, bytes);
+  while (!p && shrink_scratch(c)) p = dev_alloc(c, bytes);
+  return p;
+}
+
 // Scratch (sigma, mu, H per site) of the two-kernel and staged paths, allocated on first
 // use; Heun contexts also hold the right-hand side at t and the predicted state.
 int ensure_scratch(lbcad_ctx* c) {
   if (c->scratch_ready) return LBCAD_OK;
   const size_t es = c->elem();
   for (Inst& I : c->inst) {
-    I.sig = dev_alloc(c, 10 * I.N * es);
-    I.H = dev_alloc(c, 5 * I.N * es);
+    if (!I.sig) I.sig = dev_alloc_or_shrink(c, 10 * I.N * es);  // (an earlier call may have found room for some)
+    if (!I.H) I.H = dev_alloc_or_shrink(c, 5 * I.N * es);
     if (!I.sig || !I.H) return fail(c, LBCAD_E_OOM, "scratch allocation failed");
     I.mu = (char*)I.sig + 9 * I.N * es;
     if (c->sync_split()) {
@@ -754,7 +811,7 @@ InstDesc<T> desc_now(const lbcad_ctx* c, int inst) {
 int ensure_staging(lbcad_ctx* c, size_t bytes) {
   if (c->staging_bytes >= bytes) return LBCAD_OK;
   // the old buffer stays in the pool until destroy; staging only grows
-  void* p = dev_alloc(c, bytes);
+  void* p = dev_alloc_or_shrink(c, bytes);
   if (!p) return fail(c, LBCAD_E_OOM, "staging allocation failed");
   c->staging = (double*)p;
   c->staging_bytes = bytes;
@@ -825,6 +882,7 @@ int lbcad_autotune(lbcad_ctx* c, int32_t reps, int32_t* chosen, float* ms_per_cf
   if (c->staged_only()) return fail(c, LBCAD_E_UNSUPPORTED, "tile shapes belong to the fused path (Euler, lagged)");
   if (c->sync_split()) return fail(c, LBCAD_E_UNSUPPORTED, "sync coupling and Heun run on one fixed fused tile shape");
   DeviceGuard dg(c->device);
+  if (int r = ensure_step_scratch(c)) return r;
   const int n = (c->prec == LBCAD_FP64) ? LaunchFused<double, false>::num_configs()
                                         : LaunchFused<float, true>::num_configs();
   const int par = (int)(c->step & 1);
@@ -914,6 +972,8 @@ int lbcad_set_graph(lbcad_ctx* c, int32_t steps_per_graph) {
 int lbcad_step(lbcad_ctx* c, int64_t n) {
   if (!c || n < 0) return LBCAD_E_INVALID_ARG;
   DeviceGuard dg(c->device);
+  if (c->path == LBCAD_PATH_FUSED)
+    if (int r = ensure_step_scratch(c)) return r;
   int64_t left = n;
   if (c->graph_steps > 0) {
     if ((c->step & 1) && left > 0) {
@@ -1277,6 +1337,7 @@ int lbcad_adjoint(lbcad_ctx* c, int64_t nsteps, int32_t ckpt_every, double* dJ_d
     return fail(c, LBCAD_E_UNSUPPORTED, "the adjoint differentiates the Euler, lagged step of D3Q19 with the body force");
   if (nsteps < 1 || ckpt_every < 1) return fail(c, LBCAD_E_INVALID_ARG, "need nsteps >= 1 and ckpt_every >= 1");
   DeviceGuard dg(c->device);
+  if (int r = ensure_step_scratch(c)) return r;
   const int k = (int)std::min<int64_t>(ckpt_every, nsteps);
   const int r = c->prec == LBCAD_FP64 ? adjoint_impl<double, false>(c, nsteps, k, dJ_dzeta, dJ_dq0, dJ_dQ0, J)
                                       : adjoint_impl<float, true>(c, nsteps, k, dJ_dzeta, dJ_dq0, dJ_dQ0, J);

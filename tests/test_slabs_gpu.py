@@ -173,3 +173,81 @@ def test_create_wherever_the_scratch_meets_the_end_of_the_memory(monkeypatch, sh
     with pytest.raises(B.LbcadError) as e:
         _run(shapes, states, prec, 3)
     assert e.value.code == B.LBCAD_E_OOM
+
+
+@pytest.mark.parametrize("graph", [0, 2])
+@pytest.mark.parametrize("prec", [L.FP64, L.FP32], ids=["fp64", "fp32"])
+@pytest.mark.parametrize("shapes", [[(64, 52, 40)], [(67, 49, 41), (9, 7, 6), (33, 31, 30)]], ids=["box", "batch"])
+def test_calls_that_need_the_memory_of_the_scratch(monkeypatch, shapes, prec, graph):
+    """Buffers that later calls need (fields on their way to and from the host, the scratch of another path) may take the
+    memory of the step's scratch; the steps after that, in smaller slabs, are the same steps."""
+    import torch
+    monkeypatch.setattr(B, "_TorchAllocator", _Budget)
+    monkeypatch.setattr(_Budget, "total", None)
+    monkeypatch.setattr(_Budget, "asked", 0)
+    states = [_noise(s, prec, 41 + i) for i, s in enumerate(shapes)]
+    ref = _run(shapes, states, prec, 7)
+    whole, es, n0 = _Budget.asked, 8 if prec == L.FP64 else 4, int(np.prod(shapes[0]))
+
+    def sim_in(total):
+        monkeypatch.setattr(_Budget, "total", total)
+        sim = L.Simulation(list(shapes), [L.default_params(s, R=min(s) / 4.0, p0=16.0, precision=prec) for s in shapes],
+                           seed=1)
+        sim.set_graph(graph)
+        for i, s in enumerate(states):
+            sim.set_state(i, s)
+        return sim
+
+    def check(sim):
+        for i, (r, sums) in enumerate(ref):
+            o = torch.empty_like(r)
+            sim.get_state(i, out=o)
+            assert torch.equal(o, r), shapes[i]
+            assert np.abs(sim.observables(i) - sums).max() <= 1e-12 * r.numel()
+        sim.close()
+
+    # psi of the first box on its way to the host: 8 bytes a site where 1 is left
+    sim = sim_in(whole + n0)
+    sim.step(4)
+    psi = sim.get_fields(0, L.FIELD_PSI)
+    sim.step(2)
+    sim.set_fields(0, {"psi": sim.get_fields(0, L.FIELD_PSI)["psi"]})
+    sim.step(1)
+    assert np.isfinite(psi["psi"]).all()
+    check(sim)
+    # the scratch of the two-kernel path: 15 values a site where as much is left but for half the step's scratch
+    sites = sum(int(np.prod(s)) for s in shapes)
+    sim = sim_in(whole + 15 * es * sites - 6 * es * sites)
+    sim.step(4)
+    sim.set_path(B.PATH_TWO_KERNEL)
+    sim.set_path(B.PATH_FUSED)
+    sim.step(3)
+    check(sim)
+    # more than the scratch can give: refused, and the context steps on
+    sim = sim_in(whole)
+    sim.step(4)
+    with pytest.raises(B.LbcadError) as e:
+        sim.set_path(B.PATH_TWO_KERNEL)
+    assert e.value.code == B.LBCAD_E_OOM
+    sim.step(3)
+    check(sim)
+
+
+def test_adjoint_after_the_scratch_gave_up_memory(monkeypatch):
+    monkeypatch.setattr(B, "_TorchAllocator", _Budget)
+    monkeypatch.setattr(_Budget, "total", None)
+    shape = (40, 36, 33)
+
+    def grad(bounded):
+        sim = L.Simulation([shape], [L.default_params(shape, R=9.0, p0=12.0, zeta=0.02)], seed=3)
+        if bounded:
+            monkeypatch.setattr(_Budget, "total", sum(t.numel() for t in sim._alloc.live.values()) + 1024)
+            sim.get_fields(0, L.FIELD_PSI)
+            monkeypatch.setattr(_Budget, "total", None)
+        out = sim.adjoint(7, 3)
+        sim.close()
+        return out
+
+    ref, got = grad(False), grad(True)
+    assert np.array_equal(got[3], ref[3])
+    np.testing.assert_allclose(got[:3], ref[:3], rtol=1e-9)
