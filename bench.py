@@ -313,8 +313,8 @@ def run_reference(args):
 
 
 def batch_leg(torch, L, steps=100, warmup=3):
-    """64 independent droplets (edges from {48, 64, 80, 96}, seed 7) advanced together by one
-    persistent launch per step, replayed from a CUDA graph: aggregate MLUPS."""
+    """64 independent droplets (edges from {48, 64, 80, 96}, seed 7) advanced together, up to 28
+    in a launch, replayed from a CUDA graph: aggregate MLUPS."""
     from paper_2011_00287_gb300 import workloads as WL
     work = WL.batch_uneven(seed=7, count=64)
     prms = [L.default_params(w["grid"], R=w["R"], p0=w["p0"], zeta=w["zeta"], precision=L.FP32) for w in work]
@@ -329,7 +329,8 @@ def batch_leg(torch, L, steps=100, warmup=3):
     out = {"mlups": sites / (ms * 1e-3) / 1e6, "ms_per_step": ms, "steps": K, "sites": sites,
            "tiles": {"chosen": TILE_NAMES[cfg], "ms_per_cfg": dict(zip(TILE_NAMES, tms))},
            "workload": "64 droplets, edges from {48,64,80,96}, R = edge/4, zeta in [0.001, 0.01], pitch in "
-                       "[12, 40], seed 7, FP32, two launches per step (28 instances each) replayed from a CUDA graph, a6 sums fused",
+                       "[12, 40], seed 7, FP32, six launches per step (two kernels for each of three groups of at most 28 "
+                       "instances) replayed from a CUDA graph, a6 sums fused",
            "clocks": clk.summary()}
     sim.close()
     return out
@@ -371,7 +372,7 @@ def main():
     ap.add_argument("--min-timed-s", type=float, default=1.0,
                     help="repeat the K-step timed region until this much device time has passed")
     ap.add_argument("--workload", default="droplet", choices=["droplet", "batch64"],
-                    help="droplet: the 128^3 benchmark line; batch64: 64 uneven droplets in one launch")
+                    help="droplet: the 128^3 benchmark line; batch64: 64 uneven droplets in one context")
     args = ap.parse_args()
     if args.warmup < 3:
         args.warmup = 3
@@ -558,7 +559,7 @@ def main():
                    "seconds": t_adj, "forward_seconds": t_fwd, "ratio_to_forward": t_adj / t_fwd,
                    "site_steps_per_s": na ** 3 * 500 / t_adj, "dJ_dzeta": dz, "finite": bool(math.isfinite(dz))}
 
-    # batched sweep: 64 uneven droplets in one launch per step (CUDA graph)
+    # batched sweep: 64 uneven droplets, up to 28 in a launch (CUDA graph)
     batch = None
     if not args.no_batch and world == 1:
         batch = batch_leg(torch, L)

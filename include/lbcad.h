@@ -261,7 +261,8 @@ int lbcad_set_state(lbcad_ctx* c, int32_t inst, const void* src, size_t bytes, i
  * ([5][z][y][x], host FP64, may be NULL) and J itself.  Device memory: (ceil(nsteps /
  * ckpt_every) + ckpt_every + 3) states of 28 values per site, plus 3 values per site for
  * each of the ckpt_every steps of a segment (their force, kept by the replay) and 56 values per site
- * of work; owned by the context until lbcad_destroy and
+ * of work; and 5 values per site of page-locked host memory, through which dJ/dQ(t0) reaches the caller (pageable
+ * memory for the length of the call where no more can be locked).  All are owned by the context until lbcad_destroy and
  * reused by later calls that fit in them.  The paper has no adjoint; this is the differentiation form
  * of the step (gradient of the droplet's drift with respect to activity, chirality and
  * the initial order). */

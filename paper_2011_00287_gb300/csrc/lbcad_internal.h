@@ -109,8 +109,9 @@ struct Launch {
   static cudaError_t observables(const InstDesc<T>& I, double* partial, int nblocks, double* out, cudaStream_t s);
 };
 
-// One instance as the marching kernels read it: sizes, coefficients, and a pointer to every component of
-// every field, so that an access's 64-bit address is one multiply-add of a 32-bit site number and a constant.
+// One instance as the marching kernels read it: sizes, coefficients, and a pointer to every component of every field.
+// The kernels add a 32-bit site number to these pointers; k_march_lb takes only the first component of its
+// populations and velocity from here and steps to the others by N (comp in lbcad_march.cuh).
 template <typename T>
 struct MarchDesc {
   int nx, ny, nz;
@@ -139,9 +140,9 @@ struct MarchDesc {
 };
 
 // The instances of one launch, passed by value: kernels read them from the constant bank.  Read from device
-// memory they stayed in registers (128^3 FP32: 88 us for k_march_fields instead of 107, and 122 for
-// k_march_lb instead of 148).  kPackMany instances fit a launch's argument space; larger batches take
-// several launches.
+// memory they stay in registers instead (FP32 Euler step at 32^3, 64^3, 128^3 and 256^3: 16.3, 33.9, 192 and 1362 us by
+// value; 18.4, 40.7, 238 and 1680 us from device memory).  kPackMany instances fit a launch's argument space; larger
+// batches take several launches.
 template <typename T, int MI>
 struct InstPack {
   MarchDesc<T> d[MI];

@@ -15,7 +15,7 @@
 // halo, partly filled warps), opens every run of planes with three sigma planes and no output,
 // and holds both halves' registers.  The scratch costs 2 x 48 bytes per site of traffic in FP32.
 //
-// Measured (FP32 with the a6 sums, one kernel for the step -> this file): 64^3 52 -> 34.6 us a step, 128^3 234 -> 193,
+// Measured (FP32 with the a6 sums, one kernel for the step -> this file): 64^3 52 -> 34.0 us a step, 128^3 234 -> 193,
 // 256^3 1640 -> 1360; the FP64 step is twice as fast.  At 128^3 k_march_fields takes 85 us, bound by instruction
 // issue at 12 warps an SM (its stencils' registers) with the shared-memory pipe busy most of that time;
 // k_march_lb 104 us, 216 bytes a site at two thirds of the copy rate.  FP64 is bound by the FP64 pipe.

@@ -637,9 +637,10 @@ MarchWork add_items(const lbcad_ctx* c, const StepWork& g, int tx, int ty, int b
   w.items = (const MarchItem*)(first * sizeof(MarchItem));  // offset; the list's address is added when it is uploaded
   w.nitems = (int)(out.size() - first);
   w.grid = w.nitems < blocks ? w.nitems : blocks;
-  // dependent launch hides a kernel's start-up (32^3: 17.4 us a step with it, 21.5 without; 64^3: 36.0 and 43.2),
-  // but blocks that start early disturb the even spread of a large step's blocks (128^3: 212 and 206 us,
-  // 256^3: 1508 and 1430)
+  // Dependent launch hides a kernel's start-up (FP32 Euler, us a step with it and without: 16^3 11.7 and 16.4, 32^3 16.3
+  // and 19.5, 64^3 34.1 and 39.0, 96^3 86.0 and 90.4, 112^3 139.4 and 142.2, 128^3 189.7 and 193.7), but blocks that
+  // start early disturb the even spread of a large step's blocks (160^3 348.4 and 349.0, 192^3 618 and 605, 256^3 1404 and
+  // 1362).  The line lies on the safe side of where the two meet, about 2^22 sites.
   w.early = sites <= kEarlySites;
   return w;
 }
