@@ -160,7 +160,11 @@ def default_params(shape=(32, 32, 32), R: float = 8.0, p0: float = 16.0, precisi
 
 
 class _TorchAllocator:
-    """Device memory for the library from PyTorch's caching allocator."""
+    """Device memory for the library from PyTorch's caching allocator.
+
+    A block that the allocator hands out is free on torch's current stream only: kernels queued there may still
+    read or write it for the tensor that held it before.  The library works on its own stream, so a block is passed on
+    when torch's stream has come past them.  (The library gives memory back after its stream has finished with it.)"""
 
     def __init__(self, device: int):
         import torch
@@ -173,6 +177,7 @@ class _TorchAllocator:
     def _alloc(self, nbytes, user):
         try:
             t = self.torch.empty(int(nbytes), dtype=self.torch.uint8, device="cuda:%d" % self.device)
+            self.torch.cuda.current_stream(self.device).synchronize()
         except Exception:
             return None
         p = t.data_ptr()
