@@ -41,7 +41,7 @@ extern "C" {
 /* ---- status codes ---------------------------------------------------------------- */
 #define LBCAD_OK 0
 #define LBCAD_E_INVALID_ARG (-1) /* bad pointer, size, parameter or instance index       */
-#define LBCAD_E_OOM (-2)         /* device allocation failed                             */
+#define LBCAD_E_OOM (-2)         /* a device or host allocation failed                   */
 #define LBCAD_E_CUDA (-3)        /* a CUDA runtime call failed (message has the reason)  */
 #define LBCAD_E_TIMEOUT (-4)     /* reserved: no kernel of this library waits on another */
 #define LBCAD_E_NAN (-5)         /* a non-finite value was found in a reduction          */

@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 
 #include <cstring>
+#include <exception>
 #include <mutex>
 #include <string>
 
@@ -106,7 +107,7 @@ int run(const lbcad_grid& g, const lbcad_params& p, const void* g_in, const void
 
 extern "C" int lbcad_step_noalloc(const lbcad_grid* grid, const lbcad_params* params, const void* g_in,
                                   const void* q_in, const void* psi_in, const void* u_in, void* g_out,
-                                  void* q_out, void* psi_out, void* u_out) {
+                                  void* q_out, void* psi_out, void* u_out) try {
   set_thread_error("");
   if (!grid || !params) return reject(LBCAD_E_INVALID_ARG, "grid and params are required");
   const lbcad_grid& g = *grid;
@@ -141,4 +142,7 @@ extern "C" int lbcad_step_noalloc(const lbcad_grid* grid, const lbcad_params* pa
             : run<float, true>(g, p, g_in, q_in, psi_in, u_in, g_out, q_out, psi_out, u_out, scratch, desc);
   if (prev >= 0 && prev != dev) cudaSetDevice(prev);
   return r;
+} catch (const std::exception&) {
+  set_thread_error("no host memory");
+  return LBCAD_E_OOM;
 }

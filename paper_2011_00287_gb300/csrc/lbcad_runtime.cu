@@ -7,6 +7,8 @@
 #include <cstdio>
 #include <cstring>
 #include <algorithm>
+#include <exception>
+#include <memory>
 #include <new>
 #include <string>
 #include <type_traits>
@@ -132,6 +134,14 @@ int fail(lbcad_ctx* c, int code, const std::string& msg) {
   return code;
 }
 
+// What an entry point returns for an exception of the host runtime (no memory for a list, a vector or a message).
+int caught(lbcad_ctx* c) noexcept {
+  std::string& err = c ? c->err : g_create_err;
+  err.clear();
+  err += "no host memory";  // fits the string's own buffer: cannot throw in turn
+  return LBCAD_E_OOM;
+}
+
 #define CK(ctx, call)                                                                          \
   do {                                                                                         \
     cudaError_t e_ = (call);                                                                   \
@@ -142,6 +152,7 @@ int fail(lbcad_ctx* c, int code, const std::string& msg) {
 void* dev_alloc(lbcad_ctx* c, size_t bytes) {
   bytes = (bytes + 255) & ~(size_t)255;
   void* p = nullptr;
+  if (c->allocs.size() == c->allocs.capacity()) c->allocs.reserve(2 * c->allocs.size() + 16);  // before there is a p to lose
   if (c->alloc) {
     p = c->alloc(bytes, c->user);
   } else if (cudaMalloc(&p, bytes) != cudaSuccess) {
@@ -344,6 +355,7 @@ int create_impl(int n, const lbcad_grid* grids, const lbcad_params* params, uint
   }
   lbcad_ctx* c = new (std::nothrow) lbcad_ctx();
   if (!c) return fail(nullptr, LBCAD_E_OOM, "host allocation failed");
+  std::unique_ptr<lbcad_ctx, void (*)(lbcad_ctx*)> own(c, lbcad_destroy);
   const lbcad_params& p0 = params[0];
   c->prec = p0.precision;
   c->integrator = p0.integrator;
@@ -354,22 +366,14 @@ int create_impl(int n, const lbcad_grid* grids, const lbcad_params* params, uint
   c->alloc = p0.alloc;
   c->free = p0.free;
   c->user = p0.alloc_user;
-  if ((c->alloc == nullptr) != (c->free == nullptr)) {
-    delete c;
+  if ((c->alloc == nullptr) != (c->free == nullptr))
     return fail(nullptr, LBCAD_E_INVALID_ARG, "alloc and free callbacks must be given together");
-  }
-  if (p0.device >= 0) {
-    c->device = p0.device;
-  } else if (cudaGetDevice(&c->device) != cudaSuccess) {
-    delete c;
-    return fail(nullptr, LBCAD_E_CUDA, "no CUDA device");
-  }
+  if (p0.device >= 0) c->device = p0.device;
+  else if (cudaGetDevice(&c->device) != cudaSuccess) return fail(nullptr, LBCAD_E_CUDA, "no CUDA device");
   DeviceGuard dg(c->device);
   int code = LBCAD_OK;
   auto bail = [&](int cd, const std::string& m) {
     g_create_err = m.empty() ? c->err : m;
-    release(c);
-    delete c;
     return cd;
   };
   if (p0.stream) {
@@ -463,12 +467,12 @@ int create_impl(int n, const lbcad_grid* grids, const lbcad_params* params, uint
                                    : upload_init<float>(c, c->inst[i], seed, i);
     if (code != LBCAD_OK) return bail(code, "");
   }
-  *out = c;
+  *out = own.release();
   return LBCAD_OK;
 }
 
-int upload_descs(lbcad_ctx* c) {
-  const int n = (int)c->inst.size();
+// The descriptors of the default path, which stay on the host.  (After the first time their vectors have the room.)
+void march_descs(lbcad_ctx* c) {
   for (int par = 0; par < 2; ++par) {
     c->desc32[par].clear();
     c->desc64[par].clear();
@@ -476,6 +480,13 @@ int upload_descs(lbcad_ctx* c) {
       if (c->prec == LBCAD_FP64) c->desc64[par].push_back(make_march_desc<double>(I, par, false));
       else c->desc32[par].push_back(make_march_desc<float>(I, par, true));
     }
+  }
+}
+
+int upload_descs(lbcad_ctx* c) {
+  const int n = (int)c->inst.size();
+  march_descs(c);
+  for (int par = 0; par < 2; ++par) {
     if (c->prec == LBCAD_FP64) {
       std::vector<InstDesc<double>> h(n);
       for (int i = 0; i < n; ++i) h[i] = make_desc<double>(c->inst[i], par);
@@ -518,27 +529,27 @@ void drop_scratch(lbcad_ctx* c) {
 int ensure_step_scratch(lbcad_ctx* c) {
   if (c->scratch || c->staged_only() || c->sync_split()) return LBCAD_OK;
   if (!place_scratch(c)) return fail(c, LBCAD_E_OOM, "scratch allocation failed");
-  return upload_descs(c);
+  march_descs(c);
+  return LBCAD_OK;
 }
 
 // A smaller scratch for the step, in more launches, where another call needs its memory: it holds something only while
 // a step runs.  False: it is as small as it gets, or there is no memory for the lists of more launches.
 bool shrink_scratch(lbcad_ctx* c) {
   if (!c->scratch || cudaStreamSynchronize(c->stream) != cudaSuccess) return false;
-  const StepPlan plan = c->plan;
+  const std::vector<lbcad_grid> boxes = boxes_of(c);
   ScratchRule rule = c->rule;
+  StepPlan plan;
   do {
-    if (rule.tightest()) {
-      c->plan = plan;
-      return false;
-    }
+    if (rule.tightest()) return false;
     rule = rule.tighter();
-    c->plan = plan_step(boxes_of(c), false, rule);
-  } while (c->plan.scratch >= plan.scratch);
+    plan = plan_step(boxes, false, rule);
+  } while (plan.scratch >= c->plan.scratch);
   drop_scratch(c);
+  std::swap(c->plan, plan);
   const bool smaller = prepare_fused(c, c->cfg_index) == LBCAD_OK;
   if (smaller) c->rule = rule;
-  else c->plan = plan;  // of the lists still in use
+  else std::swap(c->plan, plan);  // that of the lists still in use
   return ensure_step_scratch(c) == LBCAD_OK && smaller;
 }
 
@@ -571,8 +582,9 @@ int ensure_scratch(lbcad_ctx* c) {
       if (!I.rq || !I.qp) return fail(c, LBCAD_E_OOM, "scratch allocation failed");
     }
   }
-  c->scratch_ready = true;
-  return upload_descs(c);
+  const int r = upload_descs(c);
+  c->scratch_ready = r == LBCAD_OK;
+  return r;
 }
 
 // Tile shape of a new context: candidate 0 (rows of 32 sites) or 3 (rows of 16), whichever covers the boxes
@@ -650,8 +662,9 @@ void drop_graph(lbcad_ctx* c) {
   if (c->graph) { cudaGraphDestroy(c->graph); c->graph = nullptr; }
 }
 
-// Work items of the default path for tile shape `cfg_index`, and the slots of its a6 sums.
-int prepare_fused(lbcad_ctx* c, int cfg_index) {
+// Work items of the default path for tile shape `cfg_index`, and the slots of its a6 sums.  Where there is no memory
+// for them, on the host or the device, everything stays as it was.
+int prepare_fused(lbcad_ctx* c, int cfg_index) try {
   FusedCfg cfg;
   const int v = c->fused_variant();
   const bool split = c->sync_split(), heun = c->integrator == LBCAD_HEUN, many = c->inst.size() > 1;
@@ -758,6 +771,8 @@ int prepare_fused(lbcad_ctx* c, int cfg_index) {
   c->obs_valid = false;
   c->cfg_index = cfg_index;
   return LBCAD_OK;
+} catch (const std::exception&) {
+  return caught(c);
 }
 
 cudaError_t launch_fused(lbcad_ctx* c, int par) {
@@ -847,16 +862,20 @@ int lbcad_velocity_set(int32_t lattice, int32_t* c, double* w) {
   return q;
 }
 
-int lbcad_create(const lbcad_grid* grid, const lbcad_params* params, uint64_t seed, lbcad_ctx** out) {
+int lbcad_create(const lbcad_grid* grid, const lbcad_params* params, uint64_t seed, lbcad_ctx** out) try {
   return create_impl(1, grid, params, seed, out);
+} catch (const std::exception&) {
+  return caught(nullptr);
 }
 
 int lbcad_create_batch(int32_t n, const lbcad_grid* grids, const lbcad_params* params, uint64_t seed,
-                       lbcad_ctx** out) {
+                       lbcad_ctx** out) try {
   return create_impl(n, grids, params, seed, out);
+} catch (const std::exception&) {
+  return caught(nullptr);
 }
 
-int lbcad_set_path(lbcad_ctx* c, int32_t path) {
+int lbcad_set_path(lbcad_ctx* c, int32_t path) try {
   if (!c) return LBCAD_E_INVALID_ARG;
   if (path != LBCAD_PATH_FUSED && path != LBCAD_PATH_TWO_KERNEL && path != LBCAD_PATH_STAGED)
     return fail(c, LBCAD_E_INVALID_ARG, "unknown path");
@@ -876,9 +895,11 @@ int lbcad_set_path(lbcad_ctx* c, int32_t path) {
     c->obs_valid = false;
   }
   return LBCAD_OK;
+} catch (const std::exception&) {
+  return caught(c);
 }
 
-int lbcad_autotune(lbcad_ctx* c, int32_t reps, int32_t* chosen, float* ms_per_cfg, int32_t ncfg) {
+int lbcad_autotune(lbcad_ctx* c, int32_t reps, int32_t* chosen, float* ms_per_cfg, int32_t ncfg) try {
   if (!c || reps < 1) return LBCAD_E_INVALID_ARG;
   if (c->staged_only()) return fail(c, LBCAD_E_UNSUPPORTED, "tile shapes belong to the fused path (Euler, lagged)");
   if (c->sync_split()) return fail(c, LBCAD_E_UNSUPPORTED, "sync coupling and Heun run on one fixed fused tile shape");
@@ -935,9 +956,11 @@ int lbcad_autotune(lbcad_ctx* c, int32_t reps, int32_t* chosen, float* ms_per_cf
   if (r) return r;
   if (chosen) *chosen = best;
   return LBCAD_OK;
+} catch (const std::exception&) {
+  return caught(c);
 }
 
-int lbcad_set_tiles(lbcad_ctx* c, int32_t cfg) {
+int lbcad_set_tiles(lbcad_ctx* c, int32_t cfg) try {
   if (!c) return LBCAD_E_INVALID_ARG;
   if (c->staged_only()) return fail(c, LBCAD_E_UNSUPPORTED, "tile shapes belong to the fused path (Euler, lagged)");
   if (c->sync_split()) return fail(c, LBCAD_E_UNSUPPORTED, "sync coupling and Heun run on one fixed fused tile shape");
@@ -946,9 +969,11 @@ int lbcad_set_tiles(lbcad_ctx* c, int32_t cfg) {
                                         : LaunchFused<float, true>::num_configs();
   if (cfg < 0 || cfg >= n) return fail(c, LBCAD_E_INVALID_ARG, "tile shape index out of range");
   return prepare_fused(c, cfg);
+} catch (const std::exception&) {
+  return caught(c);
 }
 
-int lbcad_set_observe(lbcad_ctx* c, int32_t on) {
+int lbcad_set_observe(lbcad_ctx* c, int32_t on) try {
   if (!c || (on != 0 && on != 1)) return LBCAD_E_INVALID_ARG;
   if (c->observe != (on == 1)) {
     c->observe = on == 1;
@@ -956,9 +981,11 @@ int lbcad_set_observe(lbcad_ctx* c, int32_t on) {
     c->obs_valid = false;
   }
   return LBCAD_OK;
+} catch (const std::exception&) {
+  return caught(c);
 }
 
-int lbcad_set_graph(lbcad_ctx* c, int32_t steps_per_graph) {
+int lbcad_set_graph(lbcad_ctx* c, int32_t steps_per_graph) try {
   if (!c) return LBCAD_E_INVALID_ARG;
   // a replay must leave the ping-pong parity unchanged, so a graph holds an even number of steps
   if (steps_per_graph < 0 || (steps_per_graph & 1))
@@ -968,9 +995,11 @@ int lbcad_set_graph(lbcad_ctx* c, int32_t steps_per_graph) {
   if (c->graph) { cudaGraphDestroy(c->graph); c->graph = nullptr; }
   c->graph_steps = steps_per_graph;
   return LBCAD_OK;
+} catch (const std::exception&) {
+  return caught(c);
 }
 
-int lbcad_step(lbcad_ctx* c, int64_t n) {
+int lbcad_step(lbcad_ctx* c, int64_t n) try {
   if (!c || n < 0) return LBCAD_E_INVALID_ARG;
   DeviceGuard dg(c->device);
   if (c->path == LBCAD_PATH_FUSED)
@@ -1004,9 +1033,11 @@ int lbcad_step(lbcad_ctx* c, int64_t n) {
   // after a fused step the a6 sums of the new state are in obs_latest
   if (r == LBCAD_OK && n > 0) c->obs_valid = c->path == LBCAD_PATH_FUSED && c->observe && !c->sync_split();
   return r;
+} catch (const std::exception&) {
+  return caught(c);
 }
 
-int lbcad_get_fields(lbcad_ctx* c, int32_t inst, uint32_t mask, void* dst, size_t bytes, int32_t dst_is_device) {
+int lbcad_get_fields(lbcad_ctx* c, int32_t inst, uint32_t mask, void* dst, size_t bytes, int32_t dst_is_device) try {
   if (!c) return LBCAD_E_INVALID_ARG;
   if (inst < 0 || inst >= (int)c->inst.size()) return fail(c, LBCAD_E_INVALID_ARG, "instance out of range");
   if (!dst || mask == 0 || (mask & ~31u)) return fail(c, LBCAD_E_INVALID_ARG, "bad dst or mask");
@@ -1027,10 +1058,12 @@ int lbcad_get_fields(lbcad_ctx* c, int32_t inst, uint32_t mask, void* dst, size_
   if (!dst_is_device) CK(c, cudaMemcpyAsync(dst, target, need, cudaMemcpyDeviceToHost, c->stream));
   CK(c, cudaStreamSynchronize(c->stream));
   return LBCAD_OK;
+} catch (const std::exception&) {
+  return caught(c);
 }
 
 int lbcad_set_fields(lbcad_ctx* c, int32_t inst, uint32_t mask, const void* src, size_t bytes,
-                     int32_t src_is_device) {
+                     int32_t src_is_device) try {
   if (!c) return LBCAD_E_INVALID_ARG;
   if (inst < 0 || inst >= (int)c->inst.size()) return fail(c, LBCAD_E_INVALID_ARG, "instance out of range");
   if (!src || mask == 0 || (mask & ~31u) || (mask & LBCAD_FIELD_RHO))
@@ -1059,13 +1092,17 @@ int lbcad_set_fields(lbcad_ctx* c, int32_t inst, uint32_t mask, const void* src,
   c->obs_valid = false;
   CK(c, cudaStreamSynchronize(c->stream));
   return LBCAD_OK;
+} catch (const std::exception&) {
+  return caught(c);
 }
 
-int lbcad_state_bytes(lbcad_ctx* c, int32_t inst, size_t* bytes) {
+int lbcad_state_bytes(lbcad_ctx* c, int32_t inst, size_t* bytes) try {
   if (!c || !bytes) return LBCAD_E_INVALID_ARG;
   if (inst < 0 || inst >= (int)c->inst.size()) return fail(c, LBCAD_E_INVALID_ARG, "instance out of range");
   *bytes = (size_t)(c->q() + 9) * (size_t)c->inst[inst].N * c->elem();
   return LBCAD_OK;
+} catch (const std::exception&) {
+  return caught(c);
 }
 
 namespace {
@@ -1096,17 +1133,21 @@ int copy_state(lbcad_ctx* c, int inst, void* ext, size_t bytes, bool ext_is_devi
 }
 }  // namespace
 
-int lbcad_get_state(lbcad_ctx* c, int32_t inst, void* dst, size_t bytes, int32_t dst_is_device) {
+int lbcad_get_state(lbcad_ctx* c, int32_t inst, void* dst, size_t bytes, int32_t dst_is_device) try {
   if (!c) return LBCAD_E_INVALID_ARG;
   return copy_state(c, inst, dst, bytes, dst_is_device != 0, true);
+} catch (const std::exception&) {
+  return caught(c);
 }
 
-int lbcad_set_state(lbcad_ctx* c, int32_t inst, const void* src, size_t bytes, int32_t src_is_device) {
+int lbcad_set_state(lbcad_ctx* c, int32_t inst, const void* src, size_t bytes, int32_t src_is_device) try {
   if (!c) return LBCAD_E_INVALID_ARG;
   return copy_state(c, inst, const_cast<void*>(src), bytes, src_is_device != 0, false);
+} catch (const std::exception&) {
+  return caught(c);
 }
 
-int lbcad_observables(lbcad_ctx* c, int32_t inst, lbcad_obs* out) {
+int lbcad_observables(lbcad_ctx* c, int32_t inst, lbcad_obs* out) try {
   if (!c || !out) return LBCAD_E_INVALID_ARG;
   if (inst < 0 || inst >= (int)c->inst.size()) return fail(c, LBCAD_E_INVALID_ARG, "instance out of range");
   DeviceGuard dg(c->device);
@@ -1137,6 +1178,8 @@ int lbcad_observables(lbcad_ctx* c, int32_t inst, lbcad_obs* out) {
   for (double v : h)
     if (!std::isfinite(v)) return fail(c, LBCAD_E_NAN, "non-finite value in observables");
   return LBCAD_OK;
+} catch (const std::exception&) {
+  return caught(c);
 }
 
 }  // extern "C"
@@ -1331,7 +1374,7 @@ int adjoint_impl(lbcad_ctx* c, int64_t nsteps, int k, double* dzeta, double* dq0
 extern "C" {
 
 int lbcad_adjoint(lbcad_ctx* c, int64_t nsteps, int32_t ckpt_every, double* dJ_dzeta, double* dJ_dq0,
-                  double* dJ_dQ0, double* J) {
+                  double* dJ_dQ0, double* J) try {
   if (!c) return LBCAD_E_INVALID_ARG;
   if (c->inst.size() != 1) return fail(c, LBCAD_E_UNSUPPORTED, "the adjoint runs on single-instance contexts");
   if (c->staged_only() || c->sync_split() || !c->default_lb())
@@ -1344,9 +1387,11 @@ int lbcad_adjoint(lbcad_ctx* c, int64_t nsteps, int32_t ckpt_every, double* dJ_d
                                       : adjoint_impl<float, true>(c, nsteps, k, dJ_dzeta, dJ_dq0, dJ_dQ0, J);
   c->obs_valid = false;  // lbcad_observables forms the sums of the final state again (separate pass)
   return r;
+} catch (const std::exception&) {
+  return caught(c);
 }
 
-int lbcad_adjoint_fields(lbcad_ctx* c, uint32_t mask, void* dst, size_t bytes) {
+int lbcad_adjoint_fields(lbcad_ctx* c, uint32_t mask, void* dst, size_t bytes) try {
   if (!c) return LBCAD_E_INVALID_ARG;
   if (!c->adj_lam) return fail(c, LBCAD_E_INVALID_ARG, "no lbcad_adjoint has run on this context");
   if (!dst || mask == 0 || (mask & ~29u)) return fail(c, LBCAD_E_INVALID_ARG, "bad dst or mask (G, U, Q, PSI)");
@@ -1365,6 +1410,8 @@ int lbcad_adjoint_fields(lbcad_ctx* c, uint32_t mask, void* dst, size_t bytes) {
   CK(c, cudaMemcpyAsync(dst, c->staging, need, cudaMemcpyDeviceToHost, c->stream));
   CK(c, cudaStreamSynchronize(c->stream));
   return LBCAD_OK;
+} catch (const std::exception&) {
+  return caught(c);
 }
 
 int lbcad_num_instances(const lbcad_ctx* c) { return c ? (int)c->inst.size() : 0; }
@@ -1379,12 +1426,14 @@ int64_t lbcad_step_count(const lbcad_ctx* c) { return c ? c->step : -1; }
 
 void* lbcad_stream(const lbcad_ctx* c) { return c ? (void*)c->stream : nullptr; }
 
-int lbcad_sync(lbcad_ctx* c) {
+int lbcad_sync(lbcad_ctx* c) try {
   if (!c) return LBCAD_E_INVALID_ARG;
   DeviceGuard dg(c->device);
   CK(c, cudaStreamSynchronize(c->stream));
   CK(c, cudaGetLastError());
   return LBCAD_OK;
+} catch (const std::exception&) {
+  return caught(c);
 }
 
 void lbcad_destroy(lbcad_ctx* c) {
